@@ -25,13 +25,16 @@
 // 0.833 ms per FP32 step and 0.686 ms per FP16-deviation step, against 0.883 / 0.732 ms with
 // 5 blocks (96 registers) and 0.989 / 0.756 ms with 6; evict-first loads or stores were slower):
 //   LBM_K1_MIN_BLOCKS  minimum resident blocks per SM requested through __launch_bounds__
-//   LBM_K1_LOAD        0: ld.global.nc (__ldg), 1: evict-first (__ldcs), 2: plain load
+//   LBM_K1_LOAD        1: evict-first (__ldcs), 2: plain load. The read-only path (ld.global.nc) is
+//                      not offered: a chained launch starts while the kernel that writes its input
+//                      still runs, so the input is not constant over the launch's lifetime and a
+//                      read-only load could be moved above the wait for that kernel.
 //   LBM_K1_STORE       0: plain store, 1: evict-first streaming store (__stcs)
 #ifndef LBM_K1_MIN_BLOCKS
 #define LBM_K1_MIN_BLOCKS 4
 #endif
 #ifndef LBM_K1_LOAD
-#define LBM_K1_LOAD 0
+#define LBM_K1_LOAD 2
 #endif
 #ifndef LBM_K1_STORE
 #define LBM_K1_STORE 0
@@ -41,9 +44,7 @@ namespace lbm {
 
 template <class T>
 __device__ __forceinline__ T k1_load(const T* p) {
-#if LBM_K1_LOAD == 0
-  return __ldg(p);
-#elif LBM_K1_LOAD == 1
+#if LBM_K1_LOAD == 1
   return __ldcs(p);
 #else
   return *p;
@@ -650,12 +651,13 @@ __device__ __forceinline__ void cell_field_gradient(const P& p, int cell, int x,
 
 // K1 (COLLIDE) / K2 (stream only): pull gather, collide, aligned store.
 template <class L, class CT, class ST, int EQ, bool COLLIDE>
-__global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepParams<CT> p,
-                                                 const ST* __restrict__ fin,
-                                                 ST* __restrict__ fout, CT* __restrict__ phi) {
+__global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepParams<CT> p, const ST* fin, ST* fout,
+                                                                        CT* phi) {
+  chain_release();
   const int cell = blockIdx.x * kBlock + threadIdx.x;
   if (cell >= p.ncells) return;
   const Neigh<L> nb(cell, p);
+  chain_wait();
   const size_t N = size_t(p.ncells);
   CT f[L::Q];
   constexpr bool DEV = is_deviation_storage<ST>();
@@ -690,15 +692,16 @@ __global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepPa
 // kernel is bound by instruction issue rather than HBM; 3 resident blocks leave it 168 registers).
 template <class L, class CT, class ST, int EQ>
 __global__ void __launch_bounds__(kBlock, 3) k_step_high(const StepParams<CT> p,
-                                                          const HighParams<CT> hp,
-                                                          const ST* __restrict__ fin,
-                                                          ST* __restrict__ fout, CT* __restrict__ phi) {
+                                                          const HighParams<CT> hp, const ST* fin, ST* fout,
+                                                          CT* phi) {
   __shared__ HighTable<L, CT> tab;
+  chain_release();
   tab.fill(hp);
   __syncthreads();
   const int cell = blockIdx.x * kBlock + threadIdx.x;
   if (cell >= p.ncells) return;
   const Neigh<L> nb(cell, p);
+  chain_wait();
   const size_t N = size_t(p.ncells);
   CT f[L::Q];
   constexpr bool DEV = is_deviation_storage<ST>();
@@ -804,8 +807,8 @@ __device__ __forceinline__ void batch_cell(const BatchTables<CT>& t, const Solve
                                            HP* hp) {
   const Neigh<L> nb(cell, sd.n, sd.div_m, sd.div_s);
   const size_t N = size_t(sd.ncells);
-  const ST* __restrict__ fin = static_cast<const ST*>(sd.f[parity]);
-  ST* __restrict__ fout = static_cast<ST*>(sd.f[parity ^ 1]);
+  const ST* fin = static_cast<const ST*>(sd.f[parity]);
+  ST* fout = static_cast<ST*>(sd.f[parity ^ 1]);
   const BatchView<CT> p(t, sd, parity);
   constexpr bool DEV = is_deviation_storage<ST>();
   CT f[L::Q];
@@ -835,7 +838,7 @@ __device__ __forceinline__ void batch_cell(const BatchTables<CT>& t, const Solve
 
 // Stage the descriptor of solve `solve` in shared memory (block-wide; call with the whole block).
 template <class CT, int BLOCK>
-__device__ __forceinline__ void stage_desc(SolveDesc<CT>& sd, const SolveDesc<CT>* __restrict__ descs, int solve) {
+__device__ __forceinline__ void stage_desc(SolveDesc<CT>& sd, const SolveDesc<CT>* descs, int solve) {
   constexpr int kWords = int(sizeof(SolveDesc<CT>) / sizeof(int4));
   static_assert(sizeof(SolveDesc<CT>) % sizeof(int4) == 0, "descriptor must be a whole number of int4");
   const int4* src = reinterpret_cast<const int4*>(descs + solve);
@@ -845,9 +848,10 @@ __device__ __forceinline__ void stage_desc(SolveDesc<CT>& sd, const SolveDesc<CT
 
 template <class L, class CT, class ST, int EQ, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, batch_min_blocks<BLOCK>())
-    k_step_batch(const BatchTables<CT> t, const SolveDesc<CT>* __restrict__ descs,
-                 const Tile* __restrict__ tiles, int ntiles, int parity) {
+    k_step_batch(const BatchTables<CT> t, const SolveDesc<CT>* descs, const Tile* tiles, int ntiles, int parity) {
   __shared__ SolveDesc<CT> sd;
+  chain_release();
+  chain_wait();
   int staged = -1;
   for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
     const Tile tile = tiles[ti];
@@ -868,11 +872,12 @@ __global__ void __launch_bounds__(BLOCK, batch_min_blocks<BLOCK>())
 // memory with its descriptor, as k_step_high does for one solve.
 template <class L, class CT, class ST, int EQ>
 __global__ void __launch_bounds__(kBlock, 3)
-    k_step_batch_high(const BatchTables<CT> t, const SolveDesc<CT>* __restrict__ descs,
-                      const HighParams<CT>* __restrict__ highs, const Tile* __restrict__ tiles, int ntiles,
-                      int parity) {
+    k_step_batch_high(const BatchTables<CT> t, const SolveDesc<CT>* descs, const HighParams<CT>* highs,
+                      const Tile* tiles, int ntiles, int parity) {
   __shared__ SolveDesc<CT> sd;
   __shared__ HighTable<L, CT> tab;
+  chain_release();
+  chain_wait();
   int staged = -1;
   for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
     const Tile tile = tiles[ti];
@@ -945,10 +950,9 @@ lbm_status BatchLaunch<KIND>::launch(const BatchGroup& g, int parity, cudaStream
   if (g.high) {
     return batch_kernel_high<L>(g.store, g.eq, [&](auto kernel) -> lbm_status {
       const BatchTables<float>& t = *static_cast<const BatchTables<float>*>(g.tables);
-      kernel<<<g.grid, kBlock, 0, stream>>>(t, static_cast<const SolveDesc<float>*>(g.d_desc),
-                                            static_cast<const HighParams<float>*>(g.d_high), g.d_tiles, g.ntiles,
-                                            parity);
-      cudaError_t err = cudaGetLastError();
+      cudaError_t err = launch_chained(kernel, g.grid, kBlock, 0, stream, t,
+                                       static_cast<const SolveDesc<float>*>(g.d_desc),
+                                       static_cast<const HighParams<float>*>(g.d_high), g.d_tiles, g.ntiles, parity);
       return err == cudaSuccess ? LBM_OK : cuda_error(err, "batched step launch");
     });
   }
@@ -956,9 +960,8 @@ lbm_status BatchLaunch<KIND>::launch(const BatchGroup& g, int parity, cudaStream
     using Kern = decltype(kernel);
     (void)sizeof(Kern);
     const BatchTables<float>& t = *static_cast<const BatchTables<float>*>(g.tables);
-    kernel<<<g.grid, g.block, 0, stream>>>(t, static_cast<const SolveDesc<float>*>(g.d_desc), g.d_tiles, g.ntiles,
-                                           parity);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_chained(kernel, g.grid, g.block, 0, stream, t,
+                                     static_cast<const SolveDesc<float>*>(g.d_desc), g.d_tiles, g.ntiles, parity);
     return err == cudaSuccess ? LBM_OK : cuda_error(err, "batched step launch");
   });
 }
@@ -1053,6 +1056,10 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       p.grad_in = static_cast<const CT*>(m->rho_hist[m->hist_cur]);
       p.rho_out = static_cast<CT*>(m->rho_hist[m->hist_cur ^ 1]);
     }
+    cudaError_t err = cudaSuccess;
+    auto go = [&](auto kernel, int blocks, int threads, size_t smem, const auto&... args) {
+      err = launch_chained(kernel, blocks, threads, smem, m->stream, args..., fin, fout, phi);
+    };
     bool done = false;
     if constexpr (is_deviation_storage<ST>()) {
       if (rows) {
@@ -1061,42 +1068,33 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
         done = true;
       } else if (tensor) {
         if (high) {
-          if (m->eq == LBM_NSE)
-            k_step_tc<L, ST, LBM_NSE, true><<<tgrid, 128, tsmem, m->stream>>>(p, tp, fin, fout, phi);
-          else
-            k_step_tc<L, ST, LBM_NCDE, true><<<tgrid, 128, tsmem, m->stream>>>(p, tp, fin, fout, phi);
+          if (m->eq == LBM_NSE) go(k_step_tc<L, ST, LBM_NSE, true>, tgrid, 128, tsmem, p, tp);
+          else go(k_step_tc<L, ST, LBM_NCDE, true>, tgrid, 128, tsmem, p, tp);
         } else {
-          if (m->eq == LBM_NSE)
-            k_step_tc<L, ST, LBM_NSE, false><<<tgrid, 128, tsmem, m->stream>>>(p, tp, fin, fout, phi);
-          else
-            k_step_tc<L, ST, LBM_NCDE, false><<<tgrid, 128, tsmem, m->stream>>>(p, tp, fin, fout, phi);
+          if (m->eq == LBM_NSE) go(k_step_tc<L, ST, LBM_NSE, false>, tgrid, 128, tsmem, p, tp);
+          else go(k_step_tc<L, ST, LBM_NCDE, false>, tgrid, 128, tsmem, p, tp);
         }
         done = true;
       }
     }
     if constexpr (std::is_same<ST, float>::value) {
       if (tensor32) {
-        if (m->eq == LBM_NSE)
-          k_step_tc32_high<L, LBM_NSE><<<tgrid, 128, tsmem, m->stream>>>(p, tp32, fin, fout, phi);
-        else
-          k_step_tc32_high<L, LBM_NCDE><<<tgrid, 128, tsmem, m->stream>>>(p, tp32, fin, fout, phi);
+        if (m->eq == LBM_NSE) go(k_step_tc32_high<L, LBM_NSE>, tgrid, 128, tsmem, p, tp32);
+        else go(k_step_tc32_high<L, LBM_NCDE>, tgrid, 128, tsmem, p, tp32);
         done = true;
       }
     }
     if (done) {
     } else if (high) {
-      if (m->eq == LBM_NSE)
-        k_step_high<L, CT, ST, LBM_NSE><<<grid, kBlock, 0, m->stream>>>(p, hp, fin, fout, phi);
-      else
-        k_step_high<L, CT, ST, LBM_NCDE><<<grid, kBlock, 0, m->stream>>>(p, hp, fin, fout, phi);
+      if (m->eq == LBM_NSE) go(k_step_high<L, CT, ST, LBM_NSE>, grid, kBlock, 0, p, hp);
+      else go(k_step_high<L, CT, ST, LBM_NCDE>, grid, kBlock, 0, p, hp);
     } else if (!collide_on) {
-      k_step<L, CT, ST, LBM_NSE, false><<<grid, kBlock, 0, m->stream>>>(p, fin, fout, phi);
+      go(k_step<L, CT, ST, LBM_NSE, false>, grid, kBlock, 0, p);
     } else if (m->eq == LBM_NSE) {
-      k_step<L, CT, ST, LBM_NSE, true><<<grid, kBlock, 0, m->stream>>>(p, fin, fout, phi);
+      go(k_step<L, CT, ST, LBM_NSE, true>, grid, kBlock, 0, p);
     } else {
-      k_step<L, CT, ST, LBM_NCDE, true><<<grid, kBlock, 0, m->stream>>>(p, fin, fout, phi);
+      go(k_step<L, CT, ST, LBM_NCDE, true>, grid, kBlock, 0, p);
     }
-    cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_error(err, "collide-stream launch");
     m->cur ^= 1;
     if (hist) m->hist_cur ^= 1;

@@ -53,8 +53,7 @@ __device__ __forceinline__ uint16_t enc16(float v) {
 
 template <class L, class ST, int EQ, bool COLLIDE, bool FULL>
 __global__ void __launch_bounds__(kRowThreads, 2)
-    k_step_rows(const StepParams<float> p, const RowParams rp, const ST* __restrict__ fin, ST* __restrict__ fout,
-                float* __restrict__ phi) {
+    k_step_rows(const StepParams<float> p, const RowParams rp, const ST* fin, ST* fout, float* phi) {
   constexpr int Q = L::Q, RM = L::RMAX, PITCH = kRowPitch, WARPS = kRowThreads / 32;
   constexpr uint32_t ROWB = PITCH * sizeof(ST);  // bytes of one population's row in a buffer
   static_assert(ROWB == 32 * 16, "a row of the buffer is one 16-byte chunk per lane");
@@ -84,11 +83,13 @@ __global__ void __launch_bounds__(kRowThreads, 2)
       z += 1;
     }
   };
+  chain_release();
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) tc::mbar_init(&full[s], kRowThreads);
     tc::mbar_fence_init();
   }
   __syncthreads();
+  chain_wait();
 
   // every thread: its chunks of the Q source rows of row (y, z) into buffer s (warp w takes the
   // populations w, w + 8, ...), then one arrival on the buffer's mbarrier when they have landed
@@ -232,8 +233,8 @@ __global__ void __launch_bounds__(kRowThreads, 2)
 // next row barrier, where the whole CTA stops, waits for what it has in flight and frees its TMEM).
 template <class L, class ST, int EQ, bool HI>
 __global__ void __launch_bounds__(kRowThreads, 2)
-    k_step_rows_tc(const StepParams<float> p, const RowParams rp, const TcParams tp, const ST* __restrict__ fin,
-                   ST* __restrict__ fout, float* __restrict__ phi) {
+    k_step_rows_tc(const StepParams<float> p, const RowParams rp, const TcParams tp, const ST* fin, ST* fout,
+                   float* phi) {
   using Sh = TcShape<L, HI>;
   constexpr int Q = L::Q, R = L::R, RM = L::RMAX, PITCH = kRowPitch, WARPS = kRowThreads / 32;
   constexpr int QP = Sh::QP, RP = Sh::RP, NH = Sh::NH, NHP = Sh::NHP, N1 = Sh::N1, K2 = Sh::K2;
@@ -307,6 +308,8 @@ __global__ void __launch_bounds__(kRowThreads, 2)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  chain_release();  // after the allocation of the tensor memory
+  chain_wait();
   const uint32_t tbase = *tslot + uint32_t(tile) * TILE_COLS;
   const uint32_t lane_off = uint32_t((warp & 3) * 32) << 16;  // this warp's 32 TMEM lanes
   const uint32_t b1_s = tc::smem_addr(b1), b2_s = tc::smem_addr(b2);
@@ -674,17 +677,15 @@ lbm_status RowLaunch<KIND>::launch(const lbm_model* m, const RowPlan& plan, cons
   using L = Lat<KIND>;
   auto go = [&](auto kernel, auto tag) -> lbm_status {
     using ST = decltype(tag);
-    kernel<<<plan.grid, kRowThreads, plan.smem, m->stream>>>(p, plan.rp, static_cast<const ST*>(fin),
-                                                              static_cast<ST*>(fout), phi);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_chained(kernel, plan.grid, kRowThreads, plan.smem, m->stream, p, plan.rp,
+                                     static_cast<const ST*>(fin), static_cast<ST*>(fout), phi);
     return err == cudaSuccess ? LBM_OK : cuda_error(err, "row-staged collide-stream launch");
   };
   if (plan.tensor && collide) {
     auto go_tc = [&](auto kernel, auto tag) -> lbm_status {
       using ST = decltype(tag);
-      kernel<<<plan.grid, kRowThreads, plan.smem, m->stream>>>(p, plan.rp, plan.tp, static_cast<const ST*>(fin),
-                                                                static_cast<ST*>(fout), phi);
-      cudaError_t err = cudaGetLastError();
+      cudaError_t err = launch_chained(kernel, plan.grid, kRowThreads, plan.smem, m->stream, p, plan.rp, plan.tp,
+                                       static_cast<const ST*>(fin), static_cast<ST*>(fout), phi);
       return err == cudaSuccess ? LBM_OK : cuda_error(err, "row-staged tensor-core collide-stream launch");
     };
     return row_tc_kernel<L>(m->store, m->eq, plan.high, go_tc);

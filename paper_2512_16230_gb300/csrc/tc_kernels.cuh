@@ -101,8 +101,7 @@ constexpr int kTcCols = 128;  // TMEM columns per CTA: D1 in [0, N1), then D2 in
 
 template <class L, class ST, int EQ, bool HI>
 __global__ void __launch_bounds__(128, TcShape<L, HI>::CTAS)
-    k_step_tc(const StepParams<float> p, const TcParams tp, const ST* __restrict__ fin, ST* __restrict__ fout,
-              float* __restrict__ phi) {
+    k_step_tc(const StepParams<float> p, const TcParams tp, const ST* fin, ST* fout, float* phi) {
   using S = TcShape<L, HI>;
   constexpr int Q = L::Q, R = L::R, QP = S::QP, RP = S::RP, NH = S::NH, NHP = S::NHP, N1 = S::N1, K2 = S::K2;
   constexpr bool BF = std::is_same<ST, __nv_bfloat16>::value;
@@ -143,6 +142,8 @@ __global__ void __launch_bounds__(128, TcShape<L, HI>::CTAS)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  chain_release();  // after the allocation of the tensor memory
+  chain_wait();
   const uint32_t tmem = sm.tmem;
   const uint32_t row_lane = uint32_t(tid & ~31) << 16;  // this warp's 32 TMEM lanes
   const uint32_t d1 = tmem, d2 = tmem;  // D2 reuses D1's columns once every row has been read
@@ -404,8 +405,7 @@ __device__ __forceinline__ void split16(float v, uint16_t& hi, uint16_t& lo) {
 
 template <class L, int EQ>
 __global__ void __launch_bounds__(128, Tc32Shape<L>::CTAS)
-    k_step_tc32_high(const StepParams<float> p, const Tc32Params tp, const float* __restrict__ fin,
-                     float* __restrict__ fout, float* __restrict__ phi) {
+    k_step_tc32_high(const StepParams<float> p, const Tc32Params tp, const float* fin, float* fout, float* phi) {
   using S = Tc32Shape<L>;
   constexpr int Q = L::Q, QP = S::QP;
   static_assert(QP <= kTc32Cols, "TMEM column plan");
@@ -434,6 +434,8 @@ __global__ void __launch_bounds__(128, Tc32Shape<L>::CTAS)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  chain_release();  // after the allocation of the tensor memory
+  chain_wait();
   const uint32_t tmem = sm.tmem;
   const uint32_t row_lane = uint32_t(tid & ~31) << 16;
   const uint32_t ah_s = tc::smem_addr(sm.a_hi), al_s = tc::smem_addr(sm.a_lo);
