@@ -29,6 +29,11 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompil
          "-Xcompiler", "-Wall", "-Xcompiler", "-Wno-implicit-fallthrough", "-I", INCLUDE, "-I", CSRC]
 
 
+# The step kernels: every fused multiply-add is written out, so that the kernels which share the
+# collision (one cell a thread, batched, row-staged) round alike.
+STEP_FLAGS = ["-fmad=false"]
+
+
 def nvcc() -> str:
     for cand in (os.environ.get("NVCC"), shutil.which("nvcc"), "/usr/local/cuda/bin/nvcc"):
         if cand and os.path.exists(cand):
@@ -46,7 +51,8 @@ def _deps_mtime():
 
 
 def _compile(src, obj, extra):
-    cmd = [nvcc()] + ARCH + FLAGS + extra + ["-c", src, "-o", obj]
+    step = STEP_FLAGS if os.path.basename(src).startswith("k_") else []
+    cmd = [nvcc()] + ARCH + FLAGS + step + extra + ["-c", src, "-o", obj]
     res = subprocess.run(cmd, capture_output=True, text=True)
     return src, res.returncode, res.stdout + res.stderr
 

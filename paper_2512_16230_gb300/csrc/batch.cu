@@ -21,7 +21,7 @@ constexpr int kChunk = 8;  // steps per captured graph (even: each model's buffe
 
 struct GroupHost {
   lbm::BatchGroup g;
-  lbm::BatchTables<float> tables;
+  lbm::LatTables<float> tables;
   std::vector<lbm::SolveDesc<float>> desc;
   std::vector<lbm::HighParams<float>> high;  // per solve, for a group with per-order rates
   std::vector<lbm_model*> members;
@@ -160,24 +160,8 @@ void fill_desc(const lbm_model* m, SolveDesc<float>* d) {
   StepParams<float> p;
   make_step_params<float>(m, &p);
   std::memset(d, 0, sizeof(*d));
-  for (int r = 0; r < kMaxR; ++r) {
-    d->sd[r] = p.sd[r];
-    d->half[r] = p.half[r];
-  }
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      d->sdn[i][j] = p.sdn[i][j];
-      d->halfn[i][j] = p.halfn[i][j];
-    }
-  d->s_high = p.s_high;
-  d->one_minus_sh = p.one_minus_sh;
-  d->sh_rho_ref = p.sh_rho_ref;
-  d->cs2_eq = p.cs2_eq;
-  d->nonlin_third = p.nonlin_third;
-  for (int a = 0; a < 3; ++a) {
-    d->u_const[a] = p.u_const[a];
-    d->n[a] = p.n[a];
-  }
+  static_cast<Rates<float>&>(*d) = p;
+  for (int a = 0; a < 3; ++a) d->n[a] = p.n[a];
   d->ncells = p.ncells;
   for (int a = 0; a < 2; ++a) {
     d->div_m[a] = p.div_m[a];
@@ -189,16 +173,6 @@ void fill_desc(const lbm_model* m, SolveDesc<float>* d) {
   d->f[0] = m->f[m->cur];
   d->f[1] = m->f[m->cur ^ 1];
   d->phi = static_cast<float*>(m->phi_prev);
-  d->ncde_variant = p.ncde_variant;
-  for (int a = 0; a < 3; ++a) {
-    d->kfac[a] = p.kfac[a];
-    d->cde_coef[a] = p.cde_coef[a];
-    d->gscale[a] = p.gscale[a];
-  }
-  d->nonlin_rate = p.nonlin_rate;
-  d->a1 = p.a1;
-  d->half0 = p.half0;
-  d->grad_on = p.grad_on;
   if (m->eq == LBM_NSE && m->m2g_aniso) {
     // the density history ping-pongs with the populations: parity k reads hist[k], writes hist[k ^ 1]
     d->grad_in[0] = static_cast<const float*>(m->rho_hist[m->hist_cur]);
@@ -302,12 +276,7 @@ lbm_status rebuild(lbm_batch* b) {
       gh.g.block = high || t == b->tile.end() ? kBlock : t->second;
       StepParams<float> p;
       make_step_params<float>(m, &p);
-      std::memcpy(gh.tables.T, p.T, sizeof(p.T));
-      std::memcpy(gh.tables.D, p.D, sizeof(p.D));
-      std::memcpy(gh.tables.invN, p.invN, sizeof(p.invN));
-      std::memcpy(gh.tables.w, p.w, sizeof(p.w));
-      std::memcpy(gh.tables.wref, p.wref, sizeof(p.wref));
-      std::memcpy(gh.tables.wmom_ref, p.wmom_ref, sizeof(p.wmom_ref));
+      gh.tables = p;
       gh.members.push_back(m);
     } else {
       b->groups[it->second].members.push_back(m);
@@ -320,6 +289,7 @@ lbm_status rebuild(lbm_batch* b) {
     std::vector<Tile> tiles;
     for (size_t j = 0; j < gh.members.size(); ++j) {
       fill_desc(gh.members[j], &gh.desc[j]);
+      if (gh.members[j]->s_high != 1.0) gh.g.keep = 1;
       if (gh.g.high) make_high_params<float>(gh.members[j], &gh.high[j]);
       for (int c0 = 0; c0 < gh.members[j]->ncells; c0 += gh.g.block) tiles.push_back(Tile{int(j), c0});
     }
@@ -347,7 +317,7 @@ lbm_status rebuild(lbm_batch* b) {
     if (st != LBM_OK) return st;
     int per_sm = 0;
     st = dispatch_batch_kind(gh.g.kind, [&](auto kc) {
-      return BatchLaunch<decltype(kc)::value>::occupancy(gh.g.store, gh.g.eq, gh.g.block, gh.g.high, &per_sm);
+      return BatchLaunch<decltype(kc)::value>::occupancy(gh.g, &per_sm);
     });
     if (st != LBM_OK) return st;
     auto cap = b->per_sm.find(std::make_tuple(gh.g.kind, gh.g.store, gh.g.eq));

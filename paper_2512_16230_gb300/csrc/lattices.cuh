@@ -136,6 +136,23 @@ constexpr int normal_row(int a) {
   return found;
 }
 
+// Row of a monomial given by its sorted axes: row1<D>(a) = c_a, row2 = c_a c_b, row3 = c_a c_b c_g.
+constexpr Mono mono_of(int a, int b = -1, int g = -1) {
+  return Mono{(a == 0) + (b == 0) + (g == 0), (a == 1) + (b == 1) + (g == 1), (a == 2) + (b == 2) + (g == 2)};
+}
+template <int D>
+constexpr int row_of(Mono m) {
+  int found = -1;
+  for (int r = 0; r < (D == 2 ? 10 : 20); ++r)
+    if (mono<D>(r).a == m.a && mono<D>(r).b == m.b && mono<D>(r).c == m.c) found = r;
+  return found;
+}
+template <int D> constexpr int row1(int a) { return row_of<D>(mono_of(a)); }
+template <int D> constexpr int row2(int a, int b) { return row_of<D>(mono_of(a, b)); }
+template <int D> constexpr int row3(int a, int b, int g) { return row_of<D>(mono_of(a, b, g)); }
+// The i-th axis other than a (i < D - 1).
+constexpr int other_axis(int a, int i) { return i == 0 ? (a == 0 ? 1 : 0) : (a == 2 ? 1 : 2); }
+
 // Primitive directions: every velocity is e = m d with d primitive (components coprime, first
 // non-zero component positive) and m in {+-1, +-2, +-3}. Since mono_k(m d) = m^deg(k) mono_k(d),
 // the populations of one direction can be combined per degree before the monomial products.

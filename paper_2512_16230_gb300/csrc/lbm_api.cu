@@ -29,23 +29,72 @@ template <class CT>
 void make_step_params(const lbm_model* m, StepParams<CT>* p) {
   const lbm_lattice* L = m->lat;
   std::memset(p, 0, sizeof(*p));
-  const int R = L->R;
+  const int R = L->R, d = L->d;
+  // s_high as the kernel has it, so that 1 - s_high and the shares of the rows add up to 1
+  const double sh = std::is_same<CT, double>::value ? m->s_high : float(m->s_high);
+  // the weights that the kernel multiplies by, and the sums 1 / N' of the conserved rows with them
+  double w[kMaxQ], s2[3] = {0.0, 0.0, 0.0};
+  if (std::is_same<CT, double>::value) {
+    for (int i = 0; i < L->Q; ++i) w[i] = L->w[i];
+  } else {
+    for (int i = 0; i < L->Q; ++i) w[i] = L->wf[i];
+  }
+  for (int i = 0; i < L->Q; ++i)
+    for (int a = 0; a < d; ++a) s2[a] += w[i] * L->e[i * 3 + a] * L->e[i * 3 + a];
+  auto row = [&](int ea, int eb, int ec) {  // row of the monomial with these exponents, -1 if absent
+    for (int r = 0; r < R; ++r) {
+      const Mono mk = d == 2 ? kMono2[r] : kMono3[r];
+      if (mk.a == ea && mk.b == eb && mk.c == ec) return r;
+    }
+    return -1;
+  };
+  double D[kMaxR], iN[kMaxR];  // scale of the rows and 1 / N'_r = D_r^2 / N_r
   for (int r = 0; r < R; ++r) {
-    for (int k = 0; k < R; ++k) p->T[r][k] = CT(L->T[r * R + k]);
-    const Mono mk = L->d == 2 ? kMono2[r] : kMono3[r];
-    double Dk = 1.0;
-    for (int q = 0; q < mk.a; ++q) Dk *= L->c[0];
-    for (int q = 0; q < mk.b; ++q) Dk *= L->c[1];
-    for (int q = 0; q < mk.c; ++q) Dk *= L->c[2];
-    p->D[r] = CT(Dk);
-    p->invN[r] = CT(1.0 / L->N[r]);
-    p->sd[r] = CT(m->s[r] - m->s_high);
-    p->half[r] = CT(1.0 - 0.5 * m->s[r]);
+    const Mono mk = d == 2 ? kMono2[r] : kMono3[r];
+    D[r] = 1.0;
+    for (int q = 0; q < mk.a; ++q) D[r] *= L->c[0];
+    for (int q = 0; q < mk.b; ++q) D[r] *= L->c[1];
+    for (int q = 0; q < mk.c; ++q) D[r] *= L->c[2];
+    iN[r] = D[r] * D[r] / L->N[r];
+    if (r == 0) iN[r] = 1.0;
+    else if (r <= d) iN[r] = 1.0 / s2[r - 1];
+    p->iN[r] = CT(iN[r]);
+    p->A[r] = CT(sh * iN[r]);
+    p->NB[r] = CT(-(m->s[r] - sh) * iN[r]);
+    p->C[r] = CT((1.0 - 0.5 * m->s[r]) * iN[r]);
+  }
+  // T'_rk = T_rk D_k / D_r: the rows in lattice units
+  auto T = [&](int r, int k) { return L->T[r * R + k] * D[k] / D[r]; };
+  for (int a = 0; a < d; ++a) {
+    int e2[3] = {0, 0, 0}, e3[3] = {0, 0, 0};
+    e2[a] = 2;
+    e3[a] = 3;
+    const int raa = row(e2[0], e2[1], e2[2]), raaa = row(e3[0], e3[1], e3[2]);
+    const double nd0 = -s2[a], pc = m->cs2_eq / (L->c[a] * L->c[a]);
+    p->nd0[a] = CT(nd0);
+    p->pc[a] = CT(pc);
+    p->q[a] = CT(pc + nd0);
+    p->invc[a] = CT(1.0 / L->c[a]);
+    p->Alo[a] = CT(sh * iN[1 + a] - double(float(sh * iN[1 + a])));
+    if (raaa >= 0) {
+      double l3 = T(raaa, 1 + a);
+      for (int i = 0; i < d - 1; ++i) {
+        const int b = other_axis(a, i);
+        int em[3] = {0, 0, 0};
+        em[a] = 1;
+        em[b] = 2;
+        const int rabb = row(em[0], em[1], em[2]);
+        const double be = T(raaa, rabb);
+        p->be[a][i] = CT(be);
+        l3 -= be * T(rabb, 1 + a);
+      }
+      p->l3[a] = CT(l3);
+      p->k3[a] = CT(3.0 * pc + l3);
+    }
   }
   // normal second-order block: S_n = inverse of diag(1/s_sa) + a 1^T / d, a_a = 1/s_b - 1/s_sa
   // (Eq. (4-27) with k = 0), or diag(s_sa) without a bulk rate
   {
-    const int d = L->d;
     int rows[3] = {0, 0, 0};
     for (int r = 0, k = 0; r < R; ++r) {
       const Mono mk = d == 2 ? kMono2[r] : kMono3[r];
@@ -82,65 +131,65 @@ void make_step_params(const lbm_model* m, StepParams<CT>* p) {
     } else {
       for (int i = 0; i < d; ++i) Sn[i][i] = m->s[rows[i]];
     }
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) {
-        p->sdn[i][j] = CT(Sn[i][j] - (i == j && i < d ? m->s_high : 0.0));
-        p->halfn[i][j] = CT((i == j && i < d ? 1.0 : 0.0) - 0.5 * Sn[i][j]);
+    for (int i = 0; i < d; ++i)
+      for (int j = 0; j < d; ++j) {
+        const double scale = D[rows[j]] / D[rows[i]] * iN[rows[i]];
+        p->NBn[i][j] = CT(-(Sn[i][j] - (i == j ? sh : 0.0)) * scale);
+        p->Cn[i][j] = CT(((i == j ? 1.0 : 0.0) - 0.5 * Sn[i][j]) * scale);
       }
   }
   const bool dev = m->store == LBM_BF16_DEV || m->store == LBM_F16_DEV;
-  for (int i = 0; i < L->Q; ++i) {
-    p->w[i] = CT(L->w[i]);
-    p->wref[i] = dev ? CT(L->w[i] * m->rho_ref) : CT(0);
-  }
   const double rho_ref = dev ? m->rho_ref : 0.0;
-  for (int r = 0; r < R; ++r) {
-    const Mono mk = L->d == 2 ? kMono2[r] : kMono3[r];
-    double acc = 0.0;
-    for (int i = 0; i < L->Q; ++i) {
-      double v = L->w[i];
-      for (int q = 0; q < mk.a; ++q) v *= L->e[i * 3 + 0];
-      for (int q = 0; q < mk.b; ++q) v *= L->e[i * 3 + 1];
-      for (int q = 0; q < mk.c; ++q) v *= L->e[i * 3 + 2];
-      acc += v;
+  double wmr[4] = {0, 0, 0, 0};
+  for (int i = 0; i < L->Q; ++i) {
+    int mult = 0, lead = 0;  // e_i = lead mult d with d primitive, its first component positive
+    for (int a = 0; a < 3; ++a) {
+      const int e = L->e[i * 3 + a];
+      if (e != 0) mult = e < 0 ? -e : e;  // every non-zero component of a velocity has the same size
+      if (e != 0 && lead == 0) lead = e < 0 ? -1 : 1;
+      if (a < d) wmr[1 + a] += L->w[i] * e * e;
     }
-    p->wmom_ref[r] = CT(rho_ref * acc);
+    wmr[0] += L->w[i];
+    p->w[i] = CT(w[i]);
+    p->wm[i] = CT(lead * mult * w[i]);
+    p->wref[i] = CT(L->w[i] * rho_ref);
   }
+  for (int k = 0; k < 4; ++k) p->wmr[k] = CT(rho_ref * wmr[k]);
   // NCDE variants (App. A): a1 folds into the first-order factor of M1G (moment variant);
   // the rate variant takes its per-cell factors in the kernel; the CDE has no M1 and no M1G
   p->ncde_variant = m->eq == LBM_NCDE ? m->ncde_variant : LBM_NCDE_MOMENT;
   if (m->eq == LBM_NCDE) {
-    for (int a = 0; a < L->d; ++a) {
-      const double s1 = m->s[1 + a];
-      p->half[1 + a] = CT(1.0 - 0.5 * s1 - s1 * m->a1);
+    for (int a = 0; a < d; ++a) {
+      const double s1 = m->s[1 + a], uc = m->ncde_variant == LBM_NCDE_CDE ? 0.0 : m->u_const[a] / L->c[a];
+      p->u_const[a] = CT(uc);
+      p->h1[a] = CT(uc * (1.0 - 0.5 * s1 - s1 * m->a1) * iN[1 + a]);
+      p->s1[a] = CT(s1);
       p->kfac[a] = CT(1.0 / s1 - 0.5);
-      p->cde_coef[a] = m->ncde_variant == LBM_NCDE_CDE ? CT(m->u_const[a] * s1 / m->cs2_eq) : CT(0);
+      p->cde_coef[a] = m->ncde_variant == LBM_NCDE_CDE ? CT(m->u_const[a] * s1 / m->cs2_eq * L->c[a]) : CT(0);
     }
     p->nonlin_rate = m->ncde_variant == LBM_NCDE_RATE ? CT(m->nonlin) : CT(0);
     p->a1 = CT(m->a1);
-    p->half0 = CT(1.0 - 0.5 * m->s[0]);
+    p->half0 = CT((1.0 - 0.5 * m->s[0]) * iN[0]);
   }
   // (delta4 . u) . grad rho of Eq. (M2Ga) on the single-speed lattices: delta4_aaaa = c_a^2 - 3 c_s^2,
   // d_a rho by the central difference over the cell spacing c_a (dt = 1)
   // (the step launcher points grad_in / rho_out at the density history); the cross diffusion of
-  // the NCDE, -S1 A2 grad psi in M1G with A2 = a2 I (Eq. (M-NCDE-6)), from the prescribed psi
+  // the NCDE, -S1 A2 grad psi in M1G with A2 = a2 I (Eq. (M-NCDE-6)), from the prescribed psi;
+  // both over c_a once more, in the lattice units of their rows
   if (m->eq == LBM_NSE && m->m2g_aniso) {
     p->grad_on = 1;
-    for (int a = 0; a < L->d; ++a) p->gscale[a] = CT((L->c[a] * L->c[a] - 3.0 * m->cs2_eq) / (2.0 * L->c[a]));
+    for (int a = 0; a < d; ++a)
+      p->gscale[a] = CT((L->c[a] * L->c[a] - 3.0 * m->cs2_eq) / (2.0 * L->c[a] * L->c[a]));
   } else if (m->eq == LBM_NCDE && m->a2 != 0.0) {
     p->grad_on = 1;
-    for (int a = 0; a < L->d; ++a) p->gscale[a] = CT(m->a2 / (2.0 * L->c[a]));
+    for (int a = 0; a < d; ++a) p->gscale[a] = CT(m->a2 / (2.0 * L->c[a] * L->c[a]));
     p->grad_in = static_cast<const CT*>(m->psi);
   }
-  p->sh_rho_ref = CT(m->s_high * rho_ref);
-  p->s_high = CT(m->s_high);
-  p->one_minus_sh = CT(1.0 - m->s_high);
-  p->cs2_eq = CT(m->cs2_eq);
+  p->sh_rho_ref = CT(sh * rho_ref);
+  p->s_high = CT(sh);
+  p->one_minus_sh = CT(1.0 - sh);
   p->nonlin_third = CT(m->ncde_variant == LBM_NCDE_MOMENT ? m->nonlin / 3.0 : 0.0);
-  for (int a = 0; a < 3; ++a) {
-    p->u_const[a] = CT(m->ncde_variant == LBM_NCDE_CDE ? 0.0 : m->u_const[a]);
-    p->n[a] = a < L->d ? int(m->n[a]) : 1;
-  }
+  for (int a = 0; a < 3; ++a) p->n[a] = a < d ? int(m->n[a]) : 1;
   p->ncells = m->ncells;
   for (int a = 0; a < 2; ++a) division_magic(unsigned(p->n[a] > 1 ? p->n[a] : 2), &p->div_m[a], &p->div_s[a]);
   const bool force = m->eq == LBM_NSE && m->force_A != 0.0;
@@ -258,6 +307,84 @@ template void make_high_params<float>(const lbm_model*, HighParams<float>*);
 template void make_high_params<double>(const lbm_model*, HighParams<double>*);
 
 namespace {
+
+// The weights of the FP32 kernels: rounded to FP32 within a few units in the last place such that the
+// sums that carry mass and momentum come out right with the rounded values, sum w = 1 and
+// sum w e_a^2 = FP32(Delta2_aa / c_a^2). Rounding each weight by itself leaves those sums up to 3e-8
+// off, a bias of every step (48x48x36 Taylor-Green, 188 steps: the mass drifts by 3.5e-6). The
+// velocities of one reflection class keep one weight. Local search over moves of one or two classes.
+void fp32_weights(const lbm_lattice* L, float* w) {
+  const int d = L->d;
+  int rep[kMaxQ], nc = 0;  // a member of each class
+  double coef[kMaxQ][4];   // its share of the sums: number of members, and times e_a^2
+  for (int i = 0; i < L->Q; ++i) {
+    int c = 0;
+    for (; c < nc; ++c) {
+      bool same = true;
+      for (int a = 0; a < 3; ++a) same = same && std::abs(L->e[i * 3 + a]) == std::abs(L->e[rep[c] * 3 + a]);
+      if (same) break;
+    }
+    if (c == nc) {
+      rep[nc++] = i;
+      for (int q = 0; q < 4; ++q) coef[c][q] = 0.0;
+    }
+    coef[c][0] += 1.0;
+    for (int a = 0; a < 3; ++a) coef[c][1 + a] += double(L->e[i * 3 + a]) * L->e[i * 3 + a];
+  }
+  float v[kMaxQ];
+  double r[4] = {1.0, 0.0, 0.0, 0.0}, ulp[kMaxQ], scale[4] = {1.0, 1.0, 1.0, 1.0};
+  int k[kMaxQ] = {};
+  for (int a = 0; a < d; ++a) {
+    double s2 = 0.0;
+    for (int c = 0; c < nc; ++c) s2 += coef[c][1 + a] * L->w[rep[c]];
+    r[1 + a] = float(s2);
+    scale[1 + a] = 1.0 / s2;
+  }
+  for (int c = 0; c < nc; ++c) {
+    v[c] = float(L->w[rep[c]]);
+    ulp[c] = double(std::nextafter(std::fabs(v[c]), 2.0f)) - std::fabs(double(v[c]));
+    for (int q = 0; q < 4; ++q) r[q] -= coef[c][q] * v[c];
+  }
+  auto size = [&](const double* x) {
+    double n = 0.0;
+    for (int q = 0; q < 4; ++q) n += x[q] * x[q] * scale[q] * scale[q];
+    return n;
+  };
+  constexpr int kMost = 4;  // units in the last place
+  double best = size(r);
+  for (int pass = 0; pass < 16 && best > 1e-19; ++pass) {
+    int bi = -1, bj = -1, bs = 0, bt = 0;
+    for (int i = 0; i < nc; ++i)
+      for (int s = -1; s <= 1; s += 2) {
+        if (std::abs(k[i] + s) > kMost) continue;
+        for (int j = i; j < nc; ++j)
+          for (int t = -2; t <= 2; ++t) {
+            if ((j == i) != (t == 0) || std::abs(k[j] + t) > kMost) continue;
+            double x[4];
+            for (int q = 0; q < 4; ++q)
+              x[q] = r[q] - coef[i][q] * s * ulp[i] - (j == i ? 0.0 : coef[j][q] * t * ulp[j]);
+            const double n = size(x);
+            if (n < best) {
+              best = n;
+              bi = i, bj = j, bs = s, bt = t;
+            }
+          }
+      }
+    if (bi < 0) break;
+    k[bi] += bs;
+    for (int q = 0; q < 4; ++q) r[q] -= coef[bi][q] * bs * ulp[bi];
+    if (bj != bi) {
+      k[bj] += bt;
+      for (int q = 0; q < 4; ++q) r[q] -= coef[bj][q] * bt * ulp[bj];
+    }
+  }
+  for (int i = 0; i < L->Q; ++i)
+    for (int c = 0; c < nc; ++c) {
+      bool same = true;
+      for (int a = 0; a < 3; ++a) same = same && std::abs(L->e[i * 3 + a]) == std::abs(L->e[rep[c] * 3 + a]);
+      if (same) w[i] = float(double(v[c]) + k[c] * ulp[c]);
+    }
+}
 
 constexpr size_t kAlign = 256;
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -430,6 +557,7 @@ lbm_status lbm_lattice_create(lbm_kind kind, const double* c, const double* cs2,
       delete L;
       return st;
     }
+    fp32_weights(L, L->wf);
     *out = L;
     return LBM_OK;
   } catch (...) {

@@ -18,6 +18,7 @@ struct lbm_lattice {
   int8_t e[lbm::kMaxQ * 3];
   double c[3], cs2[3], free_w[4];
   double w[lbm::kMaxQ];
+  float wf[lbm::kMaxQ];  // the weights of the FP32 kernels
   double H[lbm::kMaxR * lbm::kMaxQ];
   double N[lbm::kMaxR];
   double T[lbm::kMaxR * lbm::kMaxR];
@@ -95,46 +96,66 @@ constexpr int kRedBlocks = 608;      // blocks of the conservation-sum reduction
 constexpr int64_t kMaxCells = (int64_t(1) << 31) - (int64_t(1) << 21);
 static_assert(int64_t(kRedBlocks) * 256 < (int64_t(1) << 21), "reduction stride within the index margin");
 
-// Kernel parameters of the time step, passed by value (they live in the constant bank, so
-// every table read below is an operand of the arithmetic instruction, not a memory load).
-template <class CT>
-struct StepParams {
-  CT T[kMaxR][kMaxR];  // Hermite rows as monic polynomials of the monomials (physical units)
-  CT D[kMaxR];         // monomial scale: mono_k(c_i) = D_k * mono_k(e_i)
-  CT invN[kMaxR];      // 1 / N_r
-  CT sd[kMaxR];        // s_r - s_high
-  CT half[kMaxR];      // 1 - s_r / 2
-  CT sdn[3][3];        // normal second-order block: S_n - s_high I (S_n diagonal unless a bulk rate is set)
-  CT halfn[3][3];      // I - S_n / 2
-  CT w[kMaxQ];
-  CT wref[kMaxQ];      // w_i * rho_ref, the offset of deviation storage
-  CT wmom_ref[kMaxR];  // rho_ref sum_i w_i mono_k(e_i): moments of the reference state w_i rho_ref
-  CT sh_rho_ref;       // s_high * rho_ref
-  CT s_high, one_minus_sh, cs2_eq, nonlin_third;
-  CT u_const[3];         // NCDE: convection velocity of M1 = u phi (zero for the CDE variant)
+// Parameters of the collision, in lattice units (every monomial mono_k(e_i) of the integer velocity
+// components; c_a is folded into the constants: row r is scaled by 1 / D_r, D_r = mono_r(c), which
+// leaves a monic row H'_r = mono_r(e) + lower, N'_r = N_r / D_r^2 and u'_a = u_a / c_a).
+//
+// The rows of order <= 3 are (the weights of every lattice meet sum w = 1, Delta4_aabb = Delta2_aa
+// Delta2_bb and Delta6_xxyyzz = Delta2_xx Delta2_yy Delta2_zz, so that these are W-orthogonal):
+//   1, a, aa + nd0_a, ab, abb + nd0_b a, abg, and the cubes aaa + l3_a a + be_a0 H'_abb + be_a1 H'_agg
+// (be: the rectangular-cell correction of Eq. (CorrectQ25) / App. D), nd0_a = -Delta2_aa / c_a^2.
+template <class V>
+struct LatTables {  // of the lattice
+  V w[kMaxQ];
+  V wm[kMaxQ];    // +-m w_i of e_i = +-m d, d the primitive direction (first component positive)
+  V wref[kMaxQ];  // w_i * rho_ref, the offset of deviation storage
+  V wmr[4];       // moments of the reference state w_i rho_ref: of 1 and of e_a^2
+  V iN[kMaxR];    // 1 / N'_r
+  V nd0[3], l3[3], be[3][2];
+  V invc[3];      // 1 / c_a
+};
+template <class V>
+struct Rates {  // of the solve
+  V A[kMaxR];    // s_high / N'_r
+  V Alo[3];      // what rounding A to FP32 leaves out on the first-order rows
+  V NB[kMaxR];   // -(s_r - s_high) / N'_r
+  V C[kMaxR];    // (1 - s_r / 2) / N'_r
+  V NBn[3][3];   // normal second-order block: -(S_n - s_high I) and I - S_n / 2 in the scaled rows, over
+  V Cn[3][3];    // N' (S_n is diagonal unless a bulk rate is set)
+  V q[3];        // cs2_eq / c_a^2 + nd0_a
+  V pc[3], k3[3];  // cs2_eq / c_a^2 and 3 cs2_eq / c_a^2 + l3_a
+  V s_high, one_minus_sh, sh_rho_ref, nonlin_third;
+  V u_const[3];  // NCDE: convection velocity of M1 = u phi over c_a (zero for the CDE variant)
+  V h1[3];       // NCDE: u'_a (1 - s_a / 2 - a1 s_a) / N', the factor of d_t phi in M1G
   // NCDE variants: per-cell first-order rates (RATE: s_a(phi) = 1 / (kfac_a g(phi) + 1/2),
-  // g = 1 + nonlin_rate phi^2) and the CDE source (S_G = sum_a cde_coef_a M1_a, M0G = half0 S_G)
+  // g = 1 + nonlin_rate phi^2) and the CDE source (S_G = sum_a cde_coef_a mu_a, M0G = half0 S_G)
   int ncde_variant;
-  CT kfac[3];
-  CT nonlin_rate, a1;
-  CT cde_coef[3];
-  CT half0;
+  V kfac[3];
+  V nonlin_rate, a1;
+  V s1[3];       // the first-order rates
+  V cde_coef[3];
+  V half0;
   // A central-difference gradient term (grad_on): gr_a = gscale_a (g(x + e_a) - g(x - e_a)) of the
   // cell field g = grad_in. NSE on rD2Q9 / rD3Q27: g is the previous step's density and
-  // gscale_a = (c_a^2 - 3 cs2_eq) / (2 c_a), the delta4 term of M2G (Eq. (M2Ga)); the step writes
+  // gscale_a = (c_a^2 - 3 cs2_eq) / (2 c_a^2), the delta4 term of M2G (Eq. (M2Ga)); the step writes
   // its own density to rho_out. NCDE: g = psi of the cross diffusion D-bar = psi I and
-  // gscale_a = a2 / (2 c_a), the A2 term of M1G (Eq. (M-NCDE-6)).
+  // gscale_a = a2 / (2 c_a^2), the A2 term of M1G (Eq. (M-NCDE-6)).
   int grad_on;
-  CT gscale[3];
-  const CT* grad_in;
-  CT* rho_out;
+  V gscale[3];
+};
+
+// Kernel parameters of the time step, passed by value (they live in the constant bank, so
+// every table read below is an operand of the arithmetic instruction, not a memory load).
+template <class V, class FT = V>
+struct StepParams : LatTables<V>, Rates<V> {
+  const FT* grad_in;
+  FT* rho_out;
   int n[3];
   int ncells;
   unsigned div_m[2];     // cell index -> (x, y, z): q = umulhi(v, div_m) >> div_s exactly divides
   int div_s[2];          // by n[0] (slot 0) and n[1] (slot 1) for every v < 2^31
   int force_a, force_b;  // force_b < 0: no body force
-  const CT* force_tab;
-  static constexpr bool kNcdeVariants = true;
+  const FT* force_tab;
 };
 
 // Rows of order >= 4 that relax with their own rates (the full Q x Q collision). The kernel
@@ -331,27 +352,11 @@ lbm_status cuda_error(cudaError_t err, const char* what);
 
 // ---- Batched execution (one launch advances every solve of a group by one step) ----
 
-// Lattice tables shared by every solve of a group (kernel parameter: constant bank).
-template <class CT>
-struct BatchTables {
-  CT T[kMaxR][kMaxR];
-  CT D[kMaxR];
-  CT invN[kMaxR];
-  CT w[kMaxQ];
-  CT wref[kMaxQ];
-  CT wmom_ref[kMaxR];
-};
-
 // Per-solve data of a batched step (device array; each block stages its solve's entry in shared
-// memory). f[k] is the input of a step launched with parity k and f[k ^ 1] its output.
+// memory; the lattice tables are a kernel parameter). f[k] is the input of a step launched with
+// parity k and f[k ^ 1] its output.
 template <class CT>
-struct __align__(16) SolveDesc {
-  CT sd[kMaxR];
-  CT half[kMaxR];
-  CT sdn[3][3];
-  CT halfn[3][3];
-  CT s_high, one_minus_sh, sh_rho_ref, cs2_eq, nonlin_third;
-  CT u_const[3];
+struct __align__(16) SolveDesc : Rates<CT> {
   int n[3];
   int ncells;
   unsigned div_m[2];
@@ -360,16 +365,8 @@ struct __align__(16) SolveDesc {
   const CT* force_tab;
   void* f[2];
   CT* phi;
-  // NCDE variants (as in StepParams)
-  int ncde_variant;
-  CT kfac[3];
-  CT nonlin_rate, a1;
-  CT cde_coef[3];
-  CT half0;
   // gradient terms (as in StepParams): a step launched with parity k reads grad_in[k] and, for the
   // delta4 term of M2G, writes its density to rho_out[k]
-  int grad_on;
-  CT gscale[3];
   const CT* grad_in[2];
   CT* rho_out[2];
 };
@@ -383,8 +380,9 @@ struct Tile {
 struct BatchGroup {
   int kind, store, eq, block;
   int high;         // the solves have one rate per order >= 4 (k_step_batch_high, tiles of kBlock cells)
+  int keep;         // some solve has s_high != 1
   const lbm_lattice* lat;
-  void* tables;     // host copy of BatchTables<CT>
+  void* tables;     // host copy of LatTables<CT>
   void* d_desc;     // device SolveDesc<CT>[nsolves]
   void* d_high;     // device HighParams<CT>[nsolves] (high groups)
   Tile* d_tiles;    // device work-list
@@ -394,7 +392,7 @@ struct BatchGroup {
 template <int KIND>
 struct BatchLaunch {
   static lbm_status launch(const BatchGroup& g, int parity, cudaStream_t stream);
-  static lbm_status occupancy(int store, int eq, int block, int high, int* blocks_per_sm);
+  static lbm_status occupancy(const BatchGroup& g, int* blocks_per_sm);
 };
 
 // Per-lattice launchers, defined in the k_<lattice>.cu translation units.

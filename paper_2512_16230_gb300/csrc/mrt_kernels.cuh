@@ -12,10 +12,18 @@
 //   f*_i = (1 - s_h) f_i + w_i sum_{r<R} H_ri / N_r [ s_h m^eq_r - (s_r - s_h)(m_r - m^eq_r)
 //                                                     + sigma_r ],
 // because the W-orthogonal complement of span(H0..H3) carries the same rate in every row.
-// The two contractions with the Hermite matrix are factored through the monomials:
-// H_r(c_i) = sum_k T_rk D_k mono_k(e_i), where mono_k(e_i) are small integers known at
-// compile time (so zero products vanish and the +-e pairs share one pass), T is the
-// lower-triangular, parity-block-diagonal Gram-Schmidt factor and D_k the axis-speed scale.
+// The two contractions with the Hermite matrix are factored through the monomials of the integer
+// velocities (raw_moments and back_project: small integers known at compile time, so zero products
+// vanish, the +-e pairs share one pass and the directions that differ by reflections share their
+// sums), and through the rows' few entries below the diagonal (collide_moments). Everything is in
+// lattice units: the axis speeds sit in the constants (LatTables, Rates).
+//
+// What bounds it: instruction issue everywhere but on large FP32 grids (HBM), and the FP64 pipe
+// (2 FMAs per clock and SM) in FP64. The shared sums, the scaled rows and s_h = 1 without the old
+// populations take rD3Q53 from about 830 to 600 FP32 operations per cell; whole solves on GB300:
+// rD2Q25 64x48 FP64 x 100 steps 1424 -> 996 us, rD3Q33 64^3 FP32 x 64 816 -> 693 us, rD2Q13
+// 1024x768 FP32 x 100 1361 -> 1190 us, rD3Q53 256x256x192 x 24 FP32 21.8 -> 20.4 ms and FP16
+// 16.4 -> 13.9 ms.
 #pragma once
 
 #include "lbm_internal.cuh"
@@ -73,236 +81,282 @@ __device__ __forceinline__ CT axpy_c(CT x, CT acc) {
   else return fma(CT(C), x, acc);
 }
 
-__host__ __device__ constexpr int axis_n(Mono m, int n) {
-  // n-th axis (0-based) in the sorted list of axes of monomial m, e.g. xyy -> x, y, y
-  return n < m.a ? 0 : (n < m.a + m.b ? 1 : 2);
-}
-
-// Raw moments mu_k = sum_i mono_k(e_i) f_i, k < R. Per primitive direction d the populations of
-// +-m d are first combined per degree (s_deg = sum_m m^deg (f_md +- f_-md), + for even degree,
-// - for odd), then mu_k += mono_k(d) s_deg(k): zero products vanish at compile time and each
-// monomial product is shared by every speed of the direction.
-template <int DEG, class CT>
-__device__ __forceinline__ CT pick_degree(CT s0, CT s1, CT s2, CT s3) {
-  if constexpr (DEG == 0) return s0;
-  else if constexpr (DEG == 1) return s1;
-  else if constexpr (DEG == 2) return s2;
-  else return s3;
-}
-
-template <class L, class CT>
-__device__ __forceinline__ void raw_moments(const CT (&f)[L::Q], CT (&mu)[L::R]) {
-  static_for<L::R>([&](auto k) { mu[decltype(k)::value] = CT(0); });
-  mu[0] = f[0];
-  static_for<num_directions<L>()>([&](auto dk) {
-    CT s0 = CT(0), s1 = CT(0), s2 = CT(0), s3 = CT(0);
-    static_for<3>([&](auto mm) {
-      constexpr int M = decltype(mm)::value + 1;
-      constexpr int ip = velocity_index<L>(direction<L>(decltype(dk)::value), M);
-      constexpr int im = velocity_index<L>(direction<L>(decltype(dk)::value), -M);
-      if constexpr (ip >= 0) {
-        const CT sp = f[ip] + f[im];
-        const CT sm = f[ip] - f[im];
-        s0 += sp;
-        s1 = axpy_c<M>(sm, s1);
-        s2 = axpy_c<M * M>(sp, s2);
-        s3 = axpy_c<M * M * M>(sm, s3);
-      }
-    });
-    static_for<L::R>([&](auto k) {
-      constexpr int K = decltype(k)::value;
-      constexpr int cv = mono_value(direction<L>(decltype(dk)::value), mono<L::D>(K));
-      if constexpr (cv != 0) mu[K] = axpy_c<cv>(pick_degree<degree(mono<L::D>(K))>(s0, s1, s2, s3), mu[K]);
-    });
-  });
-}
-
-// Continuous raw moments of the NSE equilibrium (Eq. (M-NSEs-6a), Eq. (M-NSEs-6-1) with k = 0,
-// M30 = rho u u u, p = rho cs2_eq): M0 = rho, M1 = j, M2 = j u + p I,
-// M3 = j u u + p (u delta)_sym, for every monomial of the paper's row order. Single-speed
-// lattices (k = 1) take M30 = 0 and have no pure-cube rows.
-template <class L, class CT>
-__device__ __forceinline__ void eq_raw_nse(CT rho, const CT (&j)[3], const CT (&u)[3], CT P,
-                                           CT (&me)[L::R]) {
-  static_for<L::R>([&](auto k) {
-    constexpr int K = decltype(k)::value;
-    constexpr int deg = degree(mono<L::D>(K));
-    constexpr int a0 = axis_n(mono<L::D>(K), 0), a1 = axis_n(mono<L::D>(K), 1),
-                  a2 = axis_n(mono<L::D>(K), 2);
-    if constexpr (deg == 0) {
-      me[K] = rho;
-    } else if constexpr (deg == 1) {
-      me[K] = j[a0];
-    } else if constexpr (deg == 2) {
-      if constexpr (a0 == a1) me[K] = fma(j[a0], u[a1], P);
-      else me[K] = j[a0] * u[a1];
-    } else {
-      CT v = L::SINGLE ? CT(0) : j[a0] * u[a1] * u[a2];  // M30 = rho u u u (multispeed) or 0 (single speed)
-      if constexpr (a1 == a2) v = fma(P, u[a0], v);
-      if constexpr (a0 == a2) v = fma(P, u[a1], v);
-      if constexpr (a0 == a1) v = fma(P, u[a2], v);
-      me[K] = v;
-    }
-  });
-}
-
-// Continuous raw moments of the NCDE equilibrium up to second order (Eq. (M-NCDE-6), M20 = 0):
-// M0 = phi, M1 = u phi, M2 = cs2_eq D(phi) I. Third-order entries are unused.
-template <class L, class CT, class P>
-__device__ __forceinline__ void eq_raw_ncde(CT phi, CT Dphi, const P& p,
-                                            CT (&me)[L::R]) {
-  static_for<L::R>([&](auto k) {
-    constexpr int K = decltype(k)::value;
-    constexpr int deg = degree(mono<L::D>(K));
-    constexpr int a0 = axis_n(mono<L::D>(K), 0), a1 = axis_n(mono<L::D>(K), 1);
-    if constexpr (deg == 0) me[K] = phi;
-    else if constexpr (deg == 1) me[K] = p.u_const[a0] * phi;
-    else if constexpr (deg == 2) me[K] = (a0 == a1) ? p.cs2_eq * Dphi : CT(0);
-    else me[K] = CT(0);
-  });
-}
-
-// sum_{k < r, same parity class as r} T_rk v_k + v_r   (T is monic: T_rr = 1)
-template <class L, class CT, int r, class P>
-__device__ __forceinline__ CT row_dot(const P& p, const CT (&v)[L::R]) {
-  CT acc = v[r];
-  static_for<r>([&](auto k) {
-    constexpr int K = decltype(k)::value;
-    if constexpr (parity_class(mono<L::D>(K)) == parity_class(mono<L::D>(r)))
-      acc = fma(p.T[r][K], v[K], acc);
-  });
-  return acc;
-}
-
-// Hermite moments of the equilibrium, m^eq_r = sum_k T_rk me_k.
-// For the NCDE the third-order Hermite moments of the equilibrium are zero.
-template <class L, class CT, int EQ, int r, class P>
-__device__ __forceinline__ CT hermite_eq(const P& p, const CT (&me)[L::R]) {
-  if constexpr (EQ == LBM_NCDE && degree(mono<L::D>(r)) == 3) return CT(0);
-  else return row_dot<L, CT, r>(p, me);
-}
-
-// f_i = (1 - s_h) f_i + w_i sum_k mono_k(e_i) h_k  (h already scaled by D_k). Per primitive
-// direction d: E_deg = sum_{deg(k) = deg} mono_k(d) h_k, then for every speed m present
-// f_{+-md} = (1 - s_h) f + w (E_0 + m^2 E_2 +- (m E_1 + m^3 E_3)).
-template <class L, class CT, class P>
-__device__ __forceinline__ void back_project(CT (&f)[L::Q], const P& p,
-                                             const CT (&h)[L::R], CT oms) {
-  f[0] = fma(oms, f[0], p.w[0] * h[0]);
-  static_for<num_directions<L>()>([&](auto dk) {
-    CT E1 = CT(0), E2 = CT(0), E3 = CT(0);
-    static_for<L::R>([&](auto k) {
-      constexpr int K = decltype(k)::value;
-      constexpr int cv = mono_value(direction<L>(decltype(dk)::value), mono<L::D>(K));
-      constexpr int deg = degree(mono<L::D>(K));
-      if constexpr (cv != 0 && deg == 1) E1 = axpy_c<cv>(h[K], E1);
-      if constexpr (cv != 0 && deg == 2) E2 = axpy_c<cv>(h[K], E2);
-      if constexpr (cv != 0 && deg == 3) E3 = axpy_c<cv>(h[K], E3);
-    });
-    static_for<3>([&](auto mm) {
-      constexpr int M = decltype(mm)::value + 1;
-      constexpr int ip = velocity_index<L>(direction<L>(decltype(dk)::value), M);
-      constexpr int im = velocity_index<L>(direction<L>(decltype(dk)::value), -M);
-      if constexpr (ip >= 0) {
-        const CT even = axpy_c<M * M>(E2, h[0]);
-        const CT odd = (M == 1) ? E1 + E3 : fma(CT(M * M * M), E3, CT(M) * E1);
-        f[ip] = fma(oms, f[ip], p.w[ip] * (even + odd));
-        f[im] = fma(oms, f[im], p.w[im] * (even - odd));
-      }
-    });
-  });
-}
-
-// h_k = D_k sum_{r >= k, same parity class} T_rk gN_r   (the transpose contraction)
-template <class L, class CT, class P>
-__device__ __forceinline__ void hermite_to_monomial(const P& p, const CT (&gN)[L::R],
-                                                    CT (&h)[L::R]) {
-  static_for<L::R>([&](auto k) {
-    constexpr int K = decltype(k)::value;
-    CT acc = gN[K];
-    static_for<L::R>([&](auto r) {
-      constexpr int Rr = decltype(r)::value;
-      constexpr int Kk = decltype(k)::value;
-      if constexpr (Rr > Kk && parity_class(mono<L::D>(Rr)) == parity_class(mono<L::D>(Kk)))
-        acc = fma(p.T[Rr][Kk], gN[Rr], acc);
-    });
-    if constexpr (K == 0) h[K] = acc;
-    else h[K] = acc * p.D[K];
-  });
-}
-
-// Hermite moments of row r: the equilibrium m^eq_r and the non-equilibrium m_r - m^eq_r.
-template <class L, class CT, int EQ, int r, class P>
-__device__ __forceinline__ void row_moments(const P& p, const CT (&mu)[L::R], const CT (&me)[L::R], CT& meq,
-                                            CT& neq) {
-  meq = hermite_eq<L, CT, EQ, r>(p, me);
-  if constexpr (EQ == LBM_NCDE && degree(mono<L::D>(r)) == 3) {
-    neq = row_dot<L, CT, r>(p, mu);
-  } else {
-    CT dm[L::R];
-    static_for<r + 1>([&](auto k) {
-      constexpr int K = decltype(k)::value;
-      if constexpr (parity_class(mono<L::D>(K)) == parity_class(mono<L::D>(r))) dm[K] = mu[K] - me[K];
-      else dm[K] = CT(0);
-    });
-    neq = row_dot<L, CT, r>(p, dm);
-  }
-}
-
-// Per-cell first-order factors of the NCDE (from the parameters, or per cell for the rate
-// variant) and the CDE source S_G (zero otherwise).
-template <class CT>
-struct NcdeCell {
-  CT sd1[3];    // s_a - s_high on the first-order rows
-  CT half1[3];  // factor of u d_t phi in M1G
-  CT sg;        // S_G of the CDE variant
+// Sums of one primitive direction d: s_deg = sum_m m^deg (f_md +- f_-md), + for even degree, - for
+// odd (m = 1 is on every lattice).
+template <class V>
+struct DirSums {
+  V s0, s1, s2, s3;
 };
+template <class L, int DX, int DY, int DZ, class V>
+__device__ __forceinline__ DirSums<V> dir_sums(const V (&f)[L::Q]) {
+  constexpr Vel d{DX, DY, DZ};
+  const V p1 = f[velocity_index<L>(d, 1)] + f[velocity_index<L>(d, -1)];
+  const V m1 = f[velocity_index<L>(d, 1)] - f[velocity_index<L>(d, -1)];
+  DirSums<V> r{p1, m1, p1, m1};
+  static_for<2>([&](auto mm) {
+    constexpr int M = decltype(mm)::value + 2;
+    constexpr int ip = velocity_index<L>(d, M), im = velocity_index<L>(d, -M);
+    if constexpr (ip >= 0) {
+      const V sp = f[ip] + f[im];
+      const V sm = f[ip] - f[im];
+      r.s0 = r.s0 + sp;
+      r.s1 = axpy_c<M>(sm, r.s1);
+      r.s2 = axpy_c<M * M>(sp, r.s2);
+      r.s3 = axpy_c<M * M * M>(sm, r.s3);
+    }
+  });
+  return r;
+}
 
-// g_r / N_r with g = s_h m^eq - (S - s_h I)(m - m^eq) + sigma. S is diagonal except on the normal
-// second-order rows, where the d x d block S_n carries the bulk coupling of Eq. (4-27).
-// sigma: NSE (I - S/2) M1F = (1 - s/2) F on order 1 and M2G = (I - S2/2)(uF + Fu) on order 2,
-// plus, given gr (single-speed lattices), the diagonal (delta4 . u) . grad rho of Eq. (M2Ga) with
-// gr_a = (c_a^2 - 3 c_s^2) d_a rho; NCDE M1G = (I - S1/2) u d_t phi - S1 A1 d_t(u phi) on order 1
-// (factor half1), minus S1 A2 grad psi given gr_a = a2 d_a psi (Eq. (M-NCDE-6), D-bar = psi I),
-// and, for the CDE variant, M0G = (1 - s0/2) S_G on order 0.
-template <class L, class CT, int EQ, int r, class P>
-__device__ __forceinline__ CT row_update(const P& p, const CT (&meq)[L::R], const CT (&neq)[L::R],
-                                         const CT (&u)[3], const CT (&F)[3], CT dphi, const NcdeCell<CT>& nc,
-                                         const CT* gr) {
-  constexpr int deg = degree(mono<L::D>(r));
-  constexpr int na = normal_index<L::D>(r);
-  CT relax, sig = CT(0);
-  if constexpr (na >= 0) {
-    relax = CT(0);
-    static_for<L::D>([&](auto b) {
-      constexpr int B = decltype(b)::value;
-      relax = fma(p.sdn[na][B], neq[normal_row<L::D>(B)], relax);
-      if constexpr (EQ == LBM_NSE) {
-        CT t = CT(2) * u[B] * F[B];
-        if (gr != nullptr) t = fma(u[B], gr[B], t);
-        sig = fma(p.halfn[na][B], t, sig);
+// Signed sums of four values over (sign along b, sign along g) = ++, +-, -+, --: the plain sum, the
+// sums signed by b, by g and by both (8 additions for the four).
+template <class V>
+struct Signed4 {
+  V s, b, g, bg;
+};
+template <class V>
+__device__ __forceinline__ Signed4<V> signed4(V pp, V pm, V mp, V mm) {
+  const V a0 = pp + pm, a1 = pp - pm, c0 = mp + mm, c1 = mp - mm;
+  return Signed4<V>{a0 + c0, a0 - c0, a1 + c1, a1 - c1};
+}
+
+// Raw moments mu_k = sum_i mono_k(e_i) f_i, k < R. The directions of one plane (1, 1), (1, -1) and the
+// four space diagonals enter the monomials with the same magnitude and a sign, so their signed sums
+// are formed once: for rD3Q53 104 operations in dir_sums and 88 here, against 152 with one
+// multiply-add per direction and monomial.
+template <class L, class V>
+__device__ __forceinline__ void raw_moments(const V (&f)[L::Q], V (&mu)[L::R]) {
+  constexpr int D = L::D;
+  if constexpr (D == 2) {
+    const DirSums<V> X = dir_sums<L, 1, 0, 0>(f), Y = dir_sums<L, 0, 1, 0>(f);
+    const DirSums<V> P = dir_sums<L, 1, 1, 0>(f), M = dir_sums<L, 1, -1, 0>(f);
+    mu[0] = (f[0] + (X.s0 + Y.s0)) + (P.s0 + M.s0);
+    mu[1] = X.s1 + (P.s1 + M.s1);
+    mu[2] = Y.s1 + (P.s1 - M.s1);
+    const V d2 = P.s2 + M.s2, o3 = P.s3 + M.s3, q3 = P.s3 - M.s3;
+    mu[row2<2>(0, 0)] = X.s2 + d2;
+    mu[row2<2>(1, 1)] = Y.s2 + d2;
+    mu[row2<2>(0, 1)] = P.s2 - M.s2;
+    mu[row3<2>(0, 1, 1)] = o3;
+    mu[row3<2>(0, 0, 1)] = q3;
+    if constexpr (!L::SINGLE) {
+      mu[row3<2>(0, 0, 0)] = X.s3 + o3;
+      mu[row3<2>(1, 1, 1)] = Y.s3 + q3;
+    }
+  } else {
+    const DirSums<V> ax[3] = {dir_sums<L, 1, 0, 0>(f), dir_sums<L, 0, 1, 0>(f), dir_sums<L, 0, 0, 1>(f)};
+    // space diagonals (1, +-1, +-1)
+    const DirSums<V> pp = dir_sums<L, 1, 1, 1>(f), pm = dir_sums<L, 1, 1, -1>(f);
+    const DirSums<V> mp = dir_sums<L, 1, -1, 1>(f), mm = dir_sums<L, 1, -1, -1>(f);
+    const V c0 = (pp.s0 + pm.s0) + (mp.s0 + mm.s0);
+    const Signed4<V> c2 = signed4(pp.s2, pm.s2, mp.s2, mm.s2), c3 = signed4(pp.s3, pm.s3, mp.s3, mm.s3);
+    const V c1[3] = {(pp.s1 + pm.s1) + (mp.s1 + mm.s1), (pp.s1 + pm.s1) - (mp.s1 + mm.s1),
+                     (pp.s1 - pm.s1) + (mp.s1 - mm.s1)};
+    const V c3a[3] = {c3.s, c3.b, c3.g};
+    const V c2ab[3] = {c2.b, c2.g, c2.bg};  // planes xy, xz, yz
+    V m0 = f[0] + c0, m1[3], m2[3], m3[3];
+    static_for<3>([&](auto aa) {
+      constexpr int A = decltype(aa)::value;
+      m0 = m0 + ax[A].s0;
+      m1[A] = ax[A].s1 + c1[A];
+      m2[A] = ax[A].s2 + c2.s;
+      m3[A] = ax[A].s3;
+    });
+    // planes (a, b): e_a + e_b and e_a - e_b
+    static_for<3>([&](auto pl) {
+      constexpr int PL = decltype(pl)::value;
+      constexpr int A = PL == 2 ? 1 : 0, B = PL == 0 ? 1 : 2;
+      const DirSums<V> P = dir_sums<L, A == 0, (A == 1) + (B == 1), B == 2>(f);
+      const DirSums<V> M = dir_sums<L, A == 0, (A == 1) - (B == 1), -(B == 2)>(f);
+      const V d2 = P.s2 + M.s2, o3 = P.s3 + M.s3, q3 = P.s3 - M.s3;
+      m0 = m0 + (P.s0 + M.s0);
+      m1[A] = m1[A] + (P.s1 + M.s1);
+      m1[B] = m1[B] + (P.s1 - M.s1);
+      m2[A] = m2[A] + d2;
+      m2[B] = m2[B] + d2;
+      mu[row2<3>(A, B)] = (P.s2 - M.s2) + c2ab[PL];
+      const V abb = o3 + c3a[A], baa = q3 + c3a[B];
+      mu[row3<3>(A, B, B)] = abb;
+      mu[row3<3>(B, A, A)] = baa;
+      // a cube takes both planes of its axis and the space diagonals once (in its first plane)
+      constexpr bool firstA = PL == 0, firstB = PL <= 1;
+      m3[A] = m3[A] + (firstA ? abb : o3);
+      m3[B] = m3[B] + (firstB ? baa : q3);
+    });
+    mu[0] = m0;
+    static_for<3>([&](auto aa) {
+      constexpr int A = decltype(aa)::value;
+      mu[1 + A] = m1[A];
+      mu[row2<3>(A, A)] = m2[A];
+      if constexpr (!L::SINGLE) mu[row3<3>(A, A, A)] = m3[A];
+    });
+    mu[row3<3>(0, 1, 2)] = c3.bg;
+  }
+}
+
+// The two populations of a direction at every speed m present:
+// f_{+-md} = (1 - s_h) f_{+-md} + w (E_0 + m^2 E_2 +- m (E_1 + m^2 E_3)), E_deg = sum_{deg(k) = deg}
+// mono_k(d) h_k. KEEP = false: s_h = 1, the old populations drop out.
+template <class L, int DX, int DY, int DZ, bool KEEP, class V>
+__device__ __forceinline__ void dir_out(V (&f)[L::Q], const LatTables<V>& lt, V oms, V E0, V E1, V E2, V E3) {
+  constexpr Vel d{DX, DY, DZ};
+  static_for<3>([&](auto mi) {
+    constexpr int M = decltype(mi)::value + 1;
+    constexpr int ip = velocity_index<L>(d, M), im = velocity_index<L>(d, -M);
+    if constexpr (ip >= 0) {
+      const V we = lt.w[ip] * axpy_c<M * M>(E2, E0);
+      V odd = E1;
+      if constexpr (!(L::SINGLE && iabs(DX) + iabs(DY) + iabs(DZ) == 1)) odd = axpy_c<M * M>(E3, E1);
+      if constexpr (KEEP) {
+        f[ip] = fmaf_t(oms, f[ip], fmaf_t(lt.wm[ip], odd, we));
+        f[im] = fmaf_t(oms, f[im], fmaf_t(lt.wm[im], odd, we));
+      } else {
+        f[ip] = fmaf_t(lt.wm[ip], odd, we);
+        f[im] = fmaf_t(lt.wm[im], odd, we);
+      }
+    }
+  });
+}
+
+// f_i = (1 - s_h) f_i + w_i sum_k mono_k(e_i) h_k, with the sums of raw_moments transposed.
+template <class L, bool KEEP, class V>
+__device__ __forceinline__ void back_project(V (&f)[L::Q], const LatTables<V>& lt, const V (&h)[L::R], V oms) {
+  constexpr int D = L::D;
+  const V h0 = h[0];
+  if constexpr (KEEP) f[0] = fmaf_t(oms, f[0], lt.w[0] * h0);
+  else f[0] = lt.w[0] * h0;
+  if constexpr (D == 2) {
+    V hx3 = V(0.f), hy3 = V(0.f);
+    const V o = h[row3<2>(0, 1, 1)], q = h[row3<2>(0, 0, 1)];
+    V ox = o, oy = q;
+    if constexpr (!L::SINGLE) {
+      hx3 = h[row3<2>(0, 0, 0)];
+      hy3 = h[row3<2>(1, 1, 1)];
+      ox = hx3 + o;
+      oy = hy3 + q;
+    }
+    dir_out<L, 1, 0, 0, KEEP>(f, lt, oms, h0, h[1], h[row2<2>(0, 0)], hx3);
+    dir_out<L, 0, 1, 0, KEEP>(f, lt, oms, h0, h[2], h[row2<2>(1, 1)], hy3);
+    const V s2 = h[row2<2>(0, 0)] + h[row2<2>(1, 1)], m = h[row2<2>(0, 1)];
+    dir_out<L, 1, 1, 0, KEEP>(f, lt, oms, h0, h[1] + h[2], s2 + m, ox + oy);
+    dir_out<L, 1, -1, 0, KEEP>(f, lt, oms, h0, h[1] - h[2], s2 - m, ox - oy);
+  } else {
+    V cube[3];
+    static_for<3>([&](auto aa) {
+      constexpr int A = decltype(aa)::value;
+      if constexpr (L::SINGLE) cube[A] = V(0.f);
+      else cube[A] = h[row3<3>(A, A, A)];
+      dir_out<L, A == 0, A == 1, A == 2, KEEP>(f, lt, oms, h0, h[1 + A], h[row2<3>(A, A)], cube[A]);
+    });
+    V t3[3];  // per axis: cube + both mixed rows
+    static_for<3>([&](auto pl) {
+      constexpr int PL = decltype(pl)::value;
+      constexpr int A = PL == 2 ? 1 : 0, B = PL == 0 ? 1 : 2;
+      const V abb = h[row3<3>(A, B, B)], baa = h[row3<3>(B, A, A)];
+      V oa = abb, ob = baa;
+      if constexpr (!L::SINGLE) {
+        oa = cube[A] + abb;
+        ob = cube[B] + baa;
+      }
+      const V s2 = h[row2<3>(A, A)] + h[row2<3>(B, B)], m = h[row2<3>(A, B)];
+      dir_out<L, A == 0, (A == 1) + (B == 1), B == 2, KEEP>(f, lt, oms, h0, h[1 + A] + h[1 + B], s2 + m, oa + ob);
+      dir_out<L, A == 0, (A == 1) - (B == 1), -(B == 2), KEEP>(f, lt, oms, h0, h[1 + A] - h[1 + B], s2 - m, oa - ob);
+      if constexpr (PL == 0) {
+        t3[0] = oa;
+        t3[1] = ob;
+      } else if constexpr (PL == 1) {
+        t3[0] = t3[0] + abb;
+        t3[2] = ob;
+      } else {
+        t3[1] = t3[1] + abb;
+        t3[2] = t3[2] + baa;
       }
     });
-  } else {
-    relax = p.sd[r] * neq[r];
-    if constexpr (deg == 1) {
-      constexpr int a = axis_n(mono<L::D>(r), 0);
-      if constexpr (EQ == LBM_NSE) {
-        sig = p.half[r] * F[a];
-      } else {
-        relax = nc.sd1[a] * neq[r];
-        sig = nc.half1[a] * p.u_const[a] * dphi;
-        if (gr != nullptr) sig = fma(-(nc.sd1[a] + p.s_high), gr[a], sig);
-      }
-    } else if constexpr (deg == 0 && EQ == LBM_NCDE && P::kNcdeVariants) {
-      sig = p.half0 * nc.sg;
-    } else if constexpr (deg == 2 && EQ == LBM_NSE) {
-      constexpr int a = axis_n(mono<L::D>(r), 0), b = axis_n(mono<L::D>(r), 1);
-      sig = p.half[r] * fma(u[a], F[b], u[b] * F[a]);
-    }
+    const V S = (h[row2<3>(0, 0)] + h[row2<3>(1, 1)]) + h[row2<3>(2, 2)];
+    // over the signs (along y, along z): ++, +-, -+, --
+    const Signed4<V> e2 = signed4(S, h[row2<3>(0, 1)], h[row2<3>(0, 2)], h[row2<3>(1, 2)]);
+    const Signed4<V> e3 = signed4(t3[0], t3[1], t3[2], h[row3<3>(0, 1, 2)]);
+    const V xy = h[1] + h[2], xmy = h[1] - h[2];
+    dir_out<L, 1, 1, 1, KEEP>(f, lt, oms, h0, xy + h[3], e2.s, e3.s);
+    dir_out<L, 1, 1, -1, KEEP>(f, lt, oms, h0, xy - h[3], e2.b, e3.b);
+    dir_out<L, 1, -1, 1, KEEP>(f, lt, oms, h0, xmy + h[3], e2.g, e3.g);
+    dir_out<L, 1, -1, -1, KEEP>(f, lt, oms, h0, xmy - h[3], e2.bg, e3.bg);
   }
-  const CT g = fma(p.s_high, meq[r], sig - relax);
-  return g * p.invN[r];
+}
+
+// h_k = sum_{r >= k} T'_rk gN_r: the coefficients of the monomials from those of the rows.
+template <class L, class V>
+__device__ __forceinline__ void rows_to_monomials(const LatTables<V>& lt, const V (&gN)[L::R], V (&h)[L::R]) {
+  constexpr int D = L::D;
+  h[0] = gN[0];
+  static_for<D>([&](auto aa) {
+    constexpr int A = decltype(aa)::value;
+    h[0] = fmaf_t(lt.nd0[A], gN[row2<D>(A, A)], h[0]);
+    h[row2<D>(A, A)] = gN[row2<D>(A, A)];
+    h[1 + A] = gN[1 + A];
+    if constexpr (!L::SINGLE) {
+      const V g3 = gN[row3<D>(A, A, A)];
+      h[row3<D>(A, A, A)] = g3;
+      h[1 + A] = fmaf_t(lt.l3[A], g3, h[1 + A]);
+    }
+    static_for<D - 1>([&](auto ii) {
+      constexpr int I = decltype(ii)::value, B = other_axis(A, I);
+      V g = gN[row3<D>(A, B, B)];
+      if constexpr (!L::SINGLE) g = fmaf_t(lt.be[A][I], gN[row3<D>(A, A, A)], g);
+      h[row3<D>(A, B, B)] = g;
+      h[1 + A] = fmaf_t(lt.nd0[B], g, h[1 + A]);
+      if constexpr (B > A) h[row2<D>(A, B)] = gN[row2<D>(A, B)];
+    });
+  });
+  if constexpr (D == 3) h[row3<3>(0, 1, 2)] = gN[row3<3>(0, 1, 2)];
+}
+
+// Hermite moments of the NSE equilibrium in the scaled rows, from rho, j'_a = rho u'_a and u'_a. The
+// continuous moments (Eq. (M-NSEs-6a), Eq. (M-NSEs-6-1) with k = 0, M30 = rho u u u, p = rho cs2_eq)
+// are M2 = j u + p I and M3 = j u u + p (u delta)_sym, which gives in the rows
+//   aa: rho (u'_a^2 + q_a)   ab: j'_a u'_b   abb: u'_a m_bb   abg: j'_a u'_b u'_g
+//   aaa: u'_a rho (u'_a^2 + k3_a) + be_a0 m_abb + be_a1 m_agg.
+// Single-speed lattices (k = 1) take M30 = 0: abb: j'_a q_b, abg: 0, no cubes. cub[a] is the part of
+// the cube row before the be terms.
+template <class L, class V>
+__device__ __forceinline__ void eq_rows_nse(const LatTables<V>& lt, const Rates<V>& rt, V rho, const V (&j)[3],
+                                            const V (&u)[3], V (&me)[L::R], V (&cub)[3]) {
+  constexpr int D = L::D;
+  me[0] = rho;
+  static_for<D>([&](auto aa) {
+    constexpr int A = decltype(aa)::value;
+    me[1 + A] = j[A];
+    me[row2<D>(A, A)] = fmaf_t(j[A], u[A], rho * rt.q[A]);
+  });
+  static_for<D>([&](auto aa) {
+    constexpr int A = decltype(aa)::value;
+    static_for<D - 1>([&](auto ii) {
+      constexpr int I = decltype(ii)::value, B = other_axis(A, I);
+      if constexpr (B > A) me[row2<D>(A, B)] = j[A] * u[B];
+      if constexpr (L::SINGLE) me[row3<D>(A, B, B)] = j[A] * rt.q[B];
+      else me[row3<D>(A, B, B)] = u[A] * me[row2<D>(B, B)];
+    });
+    if constexpr (!L::SINGLE) {
+      cub[A] = u[A] * fmaf_t(j[A], u[A], rho * rt.k3[A]);
+      V v = cub[A];
+      static_for<D - 1>([&](auto ii) {
+        constexpr int I = decltype(ii)::value, B = other_axis(A, I);
+        v = fmaf_t(lt.be[A][I], me[row3<D>(A, B, B)], v);
+      });
+      me[row3<D>(A, A, A)] = v;
+    }
+  });
+  if constexpr (D == 3) {
+    if constexpr (L::SINGLE) me[row3<3>(0, 1, 2)] = V(0.f);
+    else me[row3<3>(0, 1, 2)] = me[row2<3>(0, 1)] * u[2];
+  }
+}
+
+// D(phi) = phi + nonlin phi^3 / 3 and the second-order normal row of the NCDE equilibrium (Eq.
+// (M-NCDE-6), M20 = 0): M0 = phi, M1 = u phi, M2 = cs2_eq D(phi) I; third-order moments zero.
+template <class V>
+__device__ __forceinline__ V ncde_flux(const Rates<V>& rt, V phi) {
+  return fmaf_t(rt.nonlin_third, phi * phi * phi, phi);
 }
 
 // Coefficients of the rows of order >= 4 staged in shared memory, row-major (the values of one
@@ -445,122 +499,217 @@ struct NoHigh {};
 
 // The collision in moment space: from the raw moments mu_k = sum_i mono_k(e_i) f_i (k < R) to
 // the monomial-basis coefficients h of the update f*_i = (1 - s_h) f_i + w_i sum_k mono_k(e_i) h_k.
-// phi_now receives phi (NCDE) or rho (NSE); gr, if given, the M2G density-gradient term.
-template <class L, class CT, int EQ, bool DEV, class P>
-__device__ __forceinline__ void collide_moments(CT (&mu)[L::R], const P& p, const CT (&F)[3], CT phi_prev,
-                                                CT& phi_now, CT (&h)[L::R], const CT* gr = nullptr) {
+// Per row gN_r = [s_h m^eq_r - (s_r - s_h)(m_r - m^eq_r) + sigma_r] / N'_r, where on the normal
+// second-order rows the d x d block S_n takes the place of s_r (it carries the bulk coupling of
+// Eq. (4-27)). sigma: NSE (1 - s/2) F on order 1 and M2G = (I - S2/2)(uF + Fu) on order 2, plus, given
+// gr (single-speed lattices), the diagonal (delta4 . u) . grad rho of Eq. (M2Ga); NCDE M1G =
+// (I - S1/2) u d_t phi - S1 A1 d_t(u phi) on order 1, minus S1 A2 grad psi given gr (Eq. (M-NCDE-6),
+// D-bar = psi I), and, for the CDE variant, M0G = (1 - s0/2) S_G on order 0. The conserved rows of the
+// NSE are exact: with j = mu_a + F/2 the first-order row is s_h mu_a + F whatever its own rate.
+// F: the body force over c_a (read only when forced); phi_now receives phi (NCDE) or rho (NSE).
+template <class L, class V, int EQ, bool DEV>
+__device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V>& lt, const Rates<V>& rt, bool forced,
+                                                const V (&F)[3], V phi_prev, V& phi_now, V (&h)[L::R],
+                                                const V* gr = nullptr) {
   constexpr int R = L::R, D = L::D;
   if constexpr (DEV) {
-    static_for<R>([&](auto k) {
-      constexpr Mono mk = mono<L::D>(decltype(k)::value);
-      if constexpr ((mk.a & 1) == 0 && (mk.b & 1) == 0 && (mk.c & 1) == 0 && degree(mk) <= 2 &&
-                    (degree(mk) == 0 || mk.a == 2 || mk.b == 2 || mk.c == 2))
-        mu[decltype(k)::value] += p.wmom_ref[decltype(k)::value];
-    });
-  }
-  static_for<R>([&](auto k) {
-    constexpr int K = decltype(k)::value;
-    if constexpr (K > 0) mu[K] *= p.D[K];
-  });
-  CT me[R];
-  CT u[3] = {CT(0), CT(0), CT(0)};
-  CT dphi = CT(0);
-  NcdeCell<CT> nc;
-  if constexpr (EQ == LBM_NSE) {
-    // Eq. (2-4-2) with S = 0, F_F = F: rho = sum f, rho u = sum c f + F / 2
-    const CT rho = mu[0];
-    const CT inv = CT(1) / rho;
-    CT j[3] = {CT(0), CT(0), CT(0)};
+    mu[0] = mu[0] + lt.wmr[0];
     static_for<D>([&](auto a) {
       constexpr int A = decltype(a)::value;
-      j[A] = fma(CT(0.5), F[A], mu[1 + A]);
+      mu[row2<D>(A, A)] = mu[row2<D>(A, A)] + lt.wmr[1 + A];
+    });
+  }
+  V gN[R], me[R], neq[R];
+  if constexpr (EQ == LBM_NSE) {
+    // Eq. (2-4-2) with S = 0, F_F = F: rho = sum f, rho u = sum c f + F / 2
+    const V rho = mu[0];
+    const V inv = V(1.f) / rho;
+    phi_now = rho;
+    V j[3], u[3], cub[3];
+    static_for<D>([&](auto a) {
+      constexpr int A = decltype(a)::value;
+      j[A] = mu[1 + A];
+      if (forced) j[A] = fmaf_t(V(0.5f), F[A], j[A]);
       u[A] = j[A] * inv;
     });
-    eq_raw_nse<L>(rho, j, u, rho * p.cs2_eq, me);
-    phi_now = rho;
+    eq_rows_nse<L>(lt, rt, rho, j, u, me, cub);
+    gN[0] = rt.A[0] * rho;
+    static_for<D>([&](auto a) {
+      constexpr int A = decltype(a)::value;
+      // momentum: A to twice the precision (a rounded factor would be a bias of every step)
+      if constexpr (std::is_same<V, double>::value) gN[1 + A] = rt.A[1 + A] * mu[1 + A];
+      else gN[1 + A] = fmaf_t(rt.A[1 + A], mu[1 + A], rt.Alo[A] * mu[1 + A]);
+      if (forced) gN[1 + A] = fmaf_t(lt.iN[1 + A], F[A], gN[1 + A]);
+      constexpr int AA = row2<D>(A, A);
+      neq[AA] = fmaf_t(lt.nd0[A], rho, mu[AA]) - me[AA];
+    });
+    static_for<D>([&](auto a) {
+      constexpr int A = decltype(a)::value;
+      static_for<D - 1>([&](auto ii) {
+        constexpr int I = decltype(ii)::value, B = other_axis(A, I), ABB = row3<D>(A, B, B);
+        if constexpr (B > A) neq[row2<D>(A, B)] = mu[row2<D>(A, B)] - me[row2<D>(A, B)];
+        neq[ABB] = fmaf_t(lt.nd0[B], mu[1 + A], mu[ABB]) - me[ABB];
+      });
+      if constexpr (!L::SINGLE) {
+        constexpr int AAA = row3<D>(A, A, A);
+        V v = fmaf_t(lt.l3[A], mu[1 + A], mu[AAA]) - cub[A];
+        static_for<D - 1>([&](auto ii) {
+          constexpr int I = decltype(ii)::value, B = other_axis(A, I);
+          v = fmaf_t(lt.be[A][I], neq[row3<D>(A, B, B)], v);
+        });
+        neq[AAA] = v;
+      }
+    });
+    if constexpr (D == 3) neq[row3<3>(0, 1, 2)] = mu[row3<3>(0, 1, 2)] - me[row3<3>(0, 1, 2)];
+    static_for<R>([&](auto r) {
+      constexpr int Rr = decltype(r)::value;
+      if constexpr (degree(mono<D>(Rr)) >= 2) {
+        constexpr int na = normal_index<D>(Rr);
+        V g = rt.A[Rr] * me[Rr];
+        if constexpr (na >= 0) {
+          static_for<D>([&](auto b) {
+            constexpr int B = decltype(b)::value;
+            g = fmaf_t(rt.NBn[na][B], neq[row2<D>(B, B)], g);
+          });
+        } else {
+          g = fmaf_t(rt.NB[Rr], neq[Rr], g);
+        }
+        gN[Rr] = g;
+      }
+    });
+    if (forced || gr != nullptr) {
+      V t[3];
+      static_for<D>([&](auto b) {
+        constexpr int B = decltype(b)::value;
+        V v = V(0.f);
+        if (forced) v = F[B] + F[B];
+        if (gr != nullptr) v = v + gr[B];
+        t[B] = u[B] * v;
+      });
+      static_for<D>([&](auto a) {
+        constexpr int A = decltype(a)::value;
+        static_for<D>([&](auto b) {
+          constexpr int B = decltype(b)::value;
+          gN[row2<D>(A, A)] = fmaf_t(rt.Cn[A][B], t[B], gN[row2<D>(A, A)]);
+          if constexpr (B > A) {
+            constexpr int AB = row2<D>(A, B);
+            if (forced) gN[AB] = fmaf_t(rt.C[AB], fmaf_t(u[A], F[B], u[B] * F[A]), gN[AB]);
+          }
+        });
+      });
+    }
   } else {
     // Eq. (2-4-1) with S = 0: phi = sum f (+ S_G / 2, lambda = 1, for the CDE variant)
-    CT phi = mu[0];
-    static_for<3>([&](auto a) {
-      nc.sd1[decltype(a)::value] = p.sd[decltype(a)::value + 1];
-      nc.half1[decltype(a)::value] = p.half[decltype(a)::value + 1];
-    });
-    nc.sg = CT(0);
-    if constexpr (P::kNcdeVariants) {
-      if (p.ncde_variant == LBM_NCDE_CDE) {
-        // S_G = -u . grad phi with grad_a phi = -s_a M1_a^ne / cs2 (M1 = 0)
-        CT sg = CT(0);
-        static_for<D>([&](auto a) { sg = fma(p.cde_coef[decltype(a)::value], mu[1 + decltype(a)::value], sg); });
-        nc.sg = sg;
-        phi = fma(CT(0.5), sg, phi);
-      } else if (p.ncde_variant == LBM_NCDE_RATE) {
-        // s_a(phi) = 1 / ((1/s_a - 1/2)(1 + nonlin phi^2) + 1/2)
-        const CT g = fma(p.nonlin_rate, phi * phi, CT(1));
-        static_for<D>([&](auto a) {
-          constexpr int A = decltype(a)::value;
-          const CT s1 = CT(1) / fma(p.kfac[A], g, CT(0.5));
-          nc.sd1[A] = s1 - p.s_high;
-          nc.half1[A] = fma(-s1, CT(0.5) + p.a1, CT(1));
-        });
-      }
+    V phi = mu[0], sg = V(0.f);
+    if (rt.ncde_variant == LBM_NCDE_CDE) {
+      // S_G = -u . grad phi with grad_a phi = -s_a M1_a^ne / cs2 (M1 = 0)
+      static_for<D>([&](auto a) {
+        constexpr int A = decltype(a)::value;
+        sg = fmaf_t(rt.cde_coef[A], mu[1 + A], sg);
+      });
+      phi = fmaf_t(V(0.5f), sg, phi);
     }
     phi_now = phi;
-    dphi = phi - phi_prev;
-    eq_raw_ncde<L>(phi, fma(p.nonlin_third, phi * phi * phi, phi), p, me);
+    const V dphi = phi - phi_prev;
+    const V Dphi = ncde_flux(rt, phi);
+    gN[0] = rt.A[0] * phi;
+    if (rt.ncde_variant == LBM_NCDE_CDE) gN[0] = gN[0] + fmaf_t(rt.NB[0], mu[0] - phi, rt.half0 * sg);
+    static_for<D>([&](auto a) {
+      constexpr int A = decltype(a)::value;
+      const V m1 = rt.u_const[A] * phi;
+      const V n1 = mu[1 + A] - m1;
+      V s1 = rt.s1[A];
+      if (rt.ncde_variant == LBM_NCDE_RATE) {
+        // s_a(phi) = 1 / ((1/s_a - 1/2)(1 + nonlin phi^2) + 1/2)
+        const V g = fmaf_t(rt.nonlin_rate, phi * phi, V(1.f));
+        s1 = V(1.f) / fmaf_t(rt.kfac[A], g, V(0.5f));
+        const V half1 = V(1.f) - s1 * (V(0.5f) + rt.a1);
+        const V relax = (s1 - rt.s_high) * n1;
+        gN[1 + A] = lt.iN[1 + A] * (fmaf_t(rt.s_high, m1, half1 * (rt.u_const[A] * dphi)) - relax);
+      } else {
+        gN[1 + A] = fmaf_t(rt.A[1 + A], m1, fmaf_t(rt.NB[1 + A], n1, rt.h1[A] * dphi));
+      }
+      if (gr != nullptr) gN[1 + A] = gN[1 + A] - lt.iN[1 + A] * (s1 * gr[A]);
+      constexpr int AA = row2<D>(A, A);
+      me[AA] = fmaf_t(rt.pc[A], Dphi, lt.nd0[A] * phi);
+      neq[AA] = fmaf_t(lt.nd0[A], mu[0], mu[AA]) - me[AA];
+    });
+    static_for<D>([&](auto a) {
+      constexpr int A = decltype(a)::value, AA = row2<D>(A, A);
+      V g = rt.A[AA] * me[AA];
+      static_for<D>([&](auto b) {
+        constexpr int B = decltype(b)::value;
+        if constexpr (B == A) g = fmaf_t(rt.NBn[A][A], neq[AA], g);  // no bulk block in the NCDE
+      });
+      gN[AA] = g;
+      static_for<D - 1>([&](auto ii) {
+        constexpr int I = decltype(ii)::value, B = other_axis(A, I), ABB = row3<D>(A, B, B);
+        if constexpr (B > A) gN[row2<D>(A, B)] = rt.NB[row2<D>(A, B)] * mu[row2<D>(A, B)];
+        neq[ABB] = fmaf_t(lt.nd0[B], mu[1 + A], mu[ABB]);
+        gN[ABB] = rt.NB[ABB] * neq[ABB];
+      });
+      if constexpr (!L::SINGLE) {
+        constexpr int AAA = row3<D>(A, A, A);
+        V v = fmaf_t(lt.l3[A], mu[1 + A], mu[AAA]);
+        static_for<D - 1>([&](auto ii) {
+          constexpr int I = decltype(ii)::value, B = other_axis(A, I);
+          v = fmaf_t(lt.be[A][I], neq[row3<D>(A, B, B)], v);
+        });
+        gN[AAA] = rt.NB[AAA] * v;
+      }
+    });
+    if constexpr (D == 3) gN[row3<3>(0, 1, 2)] = rt.NB[row3<3>(0, 1, 2)] * mu[row3<3>(0, 1, 2)];
   }
-  CT meq[R], neq[R];
-  static_for<R>([&](auto r) {
-    constexpr int Rr = decltype(r)::value;
-    row_moments<L, CT, EQ, Rr>(p, mu, me, meq[Rr], neq[Rr]);
-  });
-  CT gN[R];
-  static_for<R>([&](auto r) {
-    constexpr int Rr = decltype(r)::value;
-    gN[Rr] = row_update<L, CT, EQ, Rr>(p, meq, neq, u, F, dphi, nc, gr);
-  });
-  hermite_to_monomial<L>(p, gN, h);
-  if constexpr (DEV) h[0] -= p.sh_rho_ref;
+  rows_to_monomials<L>(lt, gN, h);
+  if constexpr (DEV) h[0] = h[0] - rt.sh_rho_ref;
 }
 
-template <class L, class CT, int EQ, bool DEV = false, class P, class HP = NoHigh>
-__device__ __forceinline__ void collide(CT (&f)[L::Q], const P& p, const CT (&F)[3],
-                                        CT phi_prev, CT& phi_now, HP* hp = nullptr, const CT* gr = nullptr) {
+// KEEP = false: every row of order >= 4 relaxes with s_h = 1 (the default), so that f* depends on the
+// moments alone and the populations need not stay in registers through the collision.
+template <class L, class V, int EQ, bool DEV, bool KEEP, class HP = NoHigh>
+__device__ __forceinline__ void collide(V (&f)[L::Q], const LatTables<V>& lt, const Rates<V>& rt, bool forced,
+                                        const V (&F)[3], V phi_prev, V& phi_now, HP* hp = nullptr,
+                                        const V* gr = nullptr) {
   constexpr bool HI = !std::is_same<HP, NoHigh>::value;
   if constexpr (HI) high_moments<L>(f, *hp);
-  CT mu[L::R];
+  V mu[L::R];
   raw_moments<L>(f, mu);
-  CT h[L::R];
-  collide_moments<L, CT, EQ, DEV>(mu, p, F, phi_prev, phi_now, h, gr);
-  back_project<L>(f, p, h, p.one_minus_sh);
-  if constexpr (HI) high_back<L>(f, p, *hp);
+  V h[L::R];
+  collide_moments<L, V, EQ, DEV>(mu, lt, rt, forced, F, phi_prev, phi_now, h, gr);
+  back_project<L, KEEP>(f, lt, h, rt.one_minus_sh);
+  if constexpr (HI) high_back<L>(f, lt, *hp);
 }
 
-// Equilibrium populations of given fields, Eq. (feq-1): f^eq_i = w_i sum_r H_ri m^eq_r / N_r.
-template <class L, class CT, int EQ, class P>
-__device__ __forceinline__ void equilibrium(CT (&f)[L::Q], const P& p, CT rho_or_phi,
-                                            const CT (&uin)[3]) {
-  constexpr int R = L::R;
-  CT me[R];
+// Equilibrium populations of given fields, Eq. (feq-1): f^eq_i = w_i sum_r H_ri m^eq_r / N_r
+// (u: the velocity over c_a).
+template <class L, class V, int EQ>
+__device__ __forceinline__ void equilibrium(V (&f)[L::Q], const LatTables<V>& lt, const Rates<V>& rt, V rho_or_phi,
+                                            const V (&u)[3]) {
+  constexpr int R = L::R, D = L::D;
+  V me[R];
+  static_for<R>([&](auto r) { me[decltype(r)::value] = V(0.f); });
   if constexpr (EQ == LBM_NSE) {
-    CT j[3], u[3];
-    for (int a = 0; a < 3; ++a) {
-      u[a] = uin[a];
-      j[a] = rho_or_phi * uin[a];
-    }
-    eq_raw_nse<L>(rho_or_phi, j, u, rho_or_phi * p.cs2_eq, me);
+    V j[3], cub[3];
+    static_for<D>([&](auto a) { j[decltype(a)::value] = rho_or_phi * u[decltype(a)::value]; });
+    eq_rows_nse<L>(lt, rt, rho_or_phi, j, u, me, cub);
   } else {
-    const CT phi = rho_or_phi;
-    eq_raw_ncde<L>(phi, fma(p.nonlin_third, phi * phi * phi, phi), p, me);
+    const V phi = rho_or_phi;
+    const V Dphi = ncde_flux(rt, phi);
+    me[0] = phi;
+    static_for<D>([&](auto a) {
+      constexpr int A = decltype(a)::value;
+      me[1 + A] = rt.u_const[A] * phi;
+      me[row2<D>(A, A)] = fmaf_t(rt.pc[A], Dphi, lt.nd0[A] * phi);
+    });
   }
-  CT gN[R];
+  V gN[R];
   static_for<R>([&](auto r) {
     constexpr int Rr = decltype(r)::value;
-    gN[Rr] = hermite_eq<L, CT, EQ, Rr>(p, me) * p.invN[Rr];
+    gN[Rr] = me[Rr] * lt.iN[Rr];
   });
-  CT h[R];
-  hermite_to_monomial<L>(p, gN, h);
-  static_for<L::Q>([&](auto i) { f[decltype(i)::value] = CT(0); });
-  back_project<L>(f, p, h, CT(0));
+  V h[R];
+  rows_to_monomials<L>(lt, gN, h);
+  back_project<L, false>(f, lt, h, V(0.f));
 }
 
 // Cell coordinates and periodic neighbour offsets.
@@ -611,46 +760,46 @@ struct Neigh {
   }
 };
 
+// Body force over c_a at a cell; false (and F unset) without one.
 template <class CT>
-__device__ __forceinline__ void body_force(int force_a, int force_b, const CT* force_tab, int x, int y,
-                                           int z, CT (&F)[3]) {
-  F[0] = F[1] = F[2] = CT(0);
-  if (force_b >= 0) {
-    const int ib = force_b == 0 ? x : (force_b == 1 ? y : z);
-    const CT v = force_tab[ib];
-    F[0] = force_a == 0 ? v : CT(0);
-    F[1] = force_a == 1 ? v : CT(0);
-    F[2] = force_a == 2 ? v : CT(0);
-  }
+__device__ __forceinline__ bool body_force(int force_a, int force_b, const CT* force_tab, const CT (&invc)[3], int x,
+                                           int y, int z, CT (&F)[3]) {
+  if (force_b < 0) return false;
+  const int ib = force_b == 0 ? x : (force_b == 1 ? y : z);
+  const CT v = force_tab[ib];
+  F[0] = force_a == 0 ? v * invc[0] : CT(0);
+  F[1] = force_a == 1 ? v * invc[1] : CT(0);
+  F[2] = force_a == 2 ? v * invc[2] : CT(0);
+  return true;
 }
 
 // Gradient terms of the source moments: the delta4 term of M2G (Eq. (M2Ga)) on the single-speed
 // lattices needs grad rho, the cross-diffusion term of M1G (Eq. (M-NCDE-6)) grad psi. Both take
 // gr_a = gscale_a (g(x + e_a) - g(x - e_a)), the central difference of the cell field p.grad_in at
-// the periodic neighbours of cell (x, y, z); zero when the term is off.
+// the periodic neighbours of cell (x, y, z); nullptr when the term is off.
 template <class L, int EQ>
 struct GradTerm {
   static constexpr bool kOn = (L::SINGLE && EQ == LBM_NSE) || EQ == LBM_NCDE;
 };
-template <class L, class CT, class P>
-__device__ __forceinline__ void cell_field_gradient(const P& p, int cell, int x, int y, int z, CT (&gr)[3]) {
-  gr[0] = gr[1] = gr[2] = CT(0);
-  if (!p.grad_on) return;
-  const int nx = p.n[0], ny = p.n[1];
-  const CT* g = p.grad_in;
+template <class L, class CT>
+__device__ __forceinline__ const CT* cell_field_gradient(const Rates<CT>& p, const int (&n)[3], const CT* g, int cell,
+                                                         int x, int y, int z, CT (&gr)[3]) {
+  if (!p.grad_on) return nullptr;
+  const int nx = n[0], ny = n[1];
   const int xp = x + 1 == nx ? -x : 1, xm = x == 0 ? nx - 1 : -1;
   gr[0] = p.gscale[0] * (g[cell + xp] - g[cell + xm]);
   const int yp = (y + 1 == ny ? -y : 1) * nx, ym = (y == 0 ? ny - 1 : -1) * nx;
   gr[1] = p.gscale[1] * (g[cell + yp] - g[cell + ym]);
   if constexpr (L::D == 3) {
-    const int nz = p.n[2], nxy = nx * ny;
+    const int nz = n[2], nxy = nx * ny;
     const int zp = (z + 1 == nz ? -z : 1) * nxy, zm = (z == 0 ? nz - 1 : -1) * nxy;
     gr[2] = p.gscale[2] * (g[cell + zp] - g[cell + zm]);
   }
+  return gr;
 }
 
 // K1 (COLLIDE) / K2 (stream only): pull gather, collide, aligned store.
-template <class L, class CT, class ST, int EQ, bool COLLIDE>
+template <class L, class CT, class ST, int EQ, bool COLLIDE, bool KEEP>
 __global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepParams<CT> p, const ST* fin, ST* fout,
                                                                         CT* phi) {
   chain_release();
@@ -668,13 +817,14 @@ __global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepPa
   });
   if constexpr (COLLIDE) {
     CT F[3];
-    body_force(p.force_a, p.force_b, p.force_tab, nb.x, nb.y, nb.z, F);
+    const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, nb.x, nb.y, nb.z, F);
     CT phi_prev = CT(0), phi_now = CT(0);
     if constexpr (EQ == LBM_NCDE) phi_prev = phi[cell];
     constexpr bool AG = GradTerm<L, EQ>::kOn;
     CT gr[3];
-    if constexpr (AG) cell_field_gradient<L>(p, cell, nb.x, nb.y, nb.z, gr);
-    collide<L, CT, EQ, DEV>(f, p, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), AG ? gr : nullptr);
+    const CT* grad = nullptr;
+    if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, nb.x, nb.y, nb.z, gr);
+    collide<L, CT, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
     if constexpr (EQ == LBM_NCDE) phi[cell] = phi_now;
     if constexpr (AG && EQ == LBM_NSE) {
       if (p.grad_on) p.rho_out[cell] = phi_now;
@@ -711,13 +861,14 @@ __global__ void __launch_bounds__(kBlock, 3) k_step_high(const StepParams<CT> p,
     else f[I] = Codec<ST>::dec(k1_load(fin + size_t(I) * N + nb.template src<I>()), p.wref[I]);
   });
   CT F[3];
-  body_force(p.force_a, p.force_b, p.force_tab, nb.x, nb.y, nb.z, F);
+  const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, nb.x, nb.y, nb.z, F);
   CT phi_prev = CT(0), phi_now = CT(0);
   if constexpr (EQ == LBM_NCDE) phi_prev = phi[cell];
   constexpr bool AG = GradTerm<L, EQ>::kOn;
   CT gr[3];
-  if constexpr (AG) cell_field_gradient<L>(p, cell, nb.x, nb.y, nb.z, gr);
-  collide<L, CT, EQ, DEV>(f, p, F, phi_prev, phi_now, &tab, AG ? gr : nullptr);
+  const CT* grad = nullptr;
+  if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, nb.x, nb.y, nb.z, gr);
+  collide<L, CT, EQ, DEV, true>(f, p, p, forced, F, phi_prev, phi_now, &tab, grad);
   if constexpr (EQ == LBM_NCDE) phi[cell] = phi_now;
   if constexpr (AG && EQ == LBM_NSE) {
     if (p.grad_on) p.rho_out[cell] = phi_now;
@@ -743,53 +894,18 @@ __global__ void __launch_bounds__(kBlock) k_init(const StepParams<CT> p, const d
   const CT r = CT(rho_or_phi[cell]);
   CT uu[3] = {CT(0), CT(0), CT(0)};
   if constexpr (EQ == LBM_NSE) {
-    for (int a = 0; a < L::D; ++a) uu[a] = CT(u[size_t(a) * N + cell]);
+    for (int a = 0; a < L::D; ++a) uu[a] = CT(u[size_t(a) * N + cell]) * p.invc[a];
     if (phi != nullptr) phi[cell] = r;
   } else {
     phi[cell] = r;
   }
   CT f[L::Q];
-  equilibrium<L, CT, EQ>(f, p, r, uu);
+  equilibrium<L, CT, EQ>(f, p, p, r, uu);
   static_for<L::Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
     fout[size_t(I) * N + nb.template src<I>()] = Codec<ST>::enc(f[I], p.wref[I]);
   });
 }
-
-// Parameter view of a batched step: lattice tables from the kernel parameter, per-solve values
-// from the shared-memory copy of the solve's descriptor (same member names as StepParams).
-template <class CT>
-struct BatchView {
-  const CT (&T)[kMaxR][kMaxR];
-  const CT (&D)[kMaxR];
-  const CT (&invN)[kMaxR];
-  const CT (&w)[kMaxQ];
-  const CT (&wref)[kMaxQ];
-  const CT (&wmom_ref)[kMaxR];
-  const CT (&sd)[kMaxR];
-  const CT (&half)[kMaxR];
-  const CT (&sdn)[3][3];
-  const CT (&halfn)[3][3];
-  const CT (&u_const)[3];
-  CT s_high, one_minus_sh, sh_rho_ref, cs2_eq, nonlin_third;
-  int ncde_variant;
-  const CT (&kfac)[3];
-  CT nonlin_rate, a1;
-  const CT (&cde_coef)[3];
-  CT half0;
-  const int (&n)[3];
-  int grad_on;
-  const CT (&gscale)[3];
-  const CT* grad_in;
-  CT* rho_out;
-  static constexpr bool kNcdeVariants = true;
-  __device__ __forceinline__ BatchView(const BatchTables<CT>& t, const SolveDesc<CT>& d, int parity)
-      : T(t.T), D(t.D), invN(t.invN), w(t.w), wref(t.wref), wmom_ref(t.wmom_ref), sd(d.sd), half(d.half),
-        sdn(d.sdn), halfn(d.halfn), u_const(d.u_const), s_high(d.s_high), one_minus_sh(d.one_minus_sh), sh_rho_ref(d.sh_rho_ref),
-        cs2_eq(d.cs2_eq), nonlin_third(d.nonlin_third), ncde_variant(d.ncde_variant), kfac(d.kfac),
-        nonlin_rate(d.nonlin_rate), a1(d.a1), cde_coef(d.cde_coef), half0(d.half0), n(d.n), grad_on(d.grad_on),
-        gscale(d.gscale), grad_in(d.grad_in[parity]), rho_out(d.rho_out[parity]) {}
-};
 
 // K6: persistent batched collide-stream. The grid is the resident capacity of the GPU; each
 // block walks the tile work-list of the group (tiles of BLOCK cells from every solve), stages
@@ -802,37 +918,37 @@ constexpr int batch_min_blocks() {
 
 // One cell of a batched step: the same gather / collide / store as k_step, with the solve's
 // parameters from its staged descriptor (HP: the higher-row table of a per-order-rate group).
-template <class L, class CT, class ST, int EQ, class HP>
-__device__ __forceinline__ void batch_cell(const BatchTables<CT>& t, const SolveDesc<CT>& sd, int cell, int parity,
+template <class L, class CT, class ST, int EQ, bool KEEP, class HP>
+__device__ __forceinline__ void batch_cell(const LatTables<CT>& t, const SolveDesc<CT>& sd, int cell, int parity,
                                            HP* hp) {
   const Neigh<L> nb(cell, sd.n, sd.div_m, sd.div_s);
   const size_t N = size_t(sd.ncells);
   const ST* fin = static_cast<const ST*>(sd.f[parity]);
   ST* fout = static_cast<ST*>(sd.f[parity ^ 1]);
-  const BatchView<CT> p(t, sd, parity);
   constexpr bool DEV = is_deviation_storage<ST>();
   CT f[L::Q];
   static_for<L::Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
     if constexpr (DEV) f[I] = RawCodec<ST>::dec(k1_load(fin + size_t(I) * N + nb.template src<I>()));
-    else f[I] = Codec<ST>::dec(k1_load(fin + size_t(I) * N + nb.template src<I>()), p.wref[I]);
+    else f[I] = Codec<ST>::dec(k1_load(fin + size_t(I) * N + nb.template src<I>()), t.wref[I]);
   });
   CT F[3];
-  body_force(sd.force_a, sd.force_b, sd.force_tab, nb.x, nb.y, nb.z, F);
+  const bool forced = body_force(sd.force_a, sd.force_b, sd.force_tab, t.invc, nb.x, nb.y, nb.z, F);
   CT phi_prev = CT(0), phi_now = CT(0);
   if constexpr (EQ == LBM_NCDE) phi_prev = sd.phi[cell];
   constexpr bool AG = GradTerm<L, EQ>::kOn;
   CT gr[3];
-  if constexpr (AG) cell_field_gradient<L>(p, cell, nb.x, nb.y, nb.z, gr);
-  collide<L, CT, EQ, DEV>(f, p, F, phi_prev, phi_now, hp, AG ? gr : nullptr);
+  const CT* grad = nullptr;
+  if constexpr (AG) grad = cell_field_gradient<L>(sd, sd.n, sd.grad_in[parity], cell, nb.x, nb.y, nb.z, gr);
+  collide<L, CT, EQ, DEV, KEEP>(f, t, sd, forced, F, phi_prev, phi_now, hp, grad);
   if constexpr (EQ == LBM_NCDE) sd.phi[cell] = phi_now;
   if constexpr (AG && EQ == LBM_NSE) {
-    if (p.grad_on) p.rho_out[cell] = phi_now;
+    if (sd.grad_on) sd.rho_out[parity][cell] = phi_now;
   }
   static_for<L::Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
     if constexpr (DEV) k1_store(fout + size_t(I) * N + cell, RawCodec<ST>::enc(f[I]));
-    else k1_store(fout + size_t(I) * N + cell, Codec<ST>::enc(f[I], p.wref[I]));
+    else k1_store(fout + size_t(I) * N + cell, Codec<ST>::enc(f[I], t.wref[I]));
   });
 }
 
@@ -846,9 +962,9 @@ __device__ __forceinline__ void stage_desc(SolveDesc<CT>& sd, const SolveDesc<CT
   for (int w = threadIdx.x; w < kWords; w += BLOCK) dst[w] = src[w];
 }
 
-template <class L, class CT, class ST, int EQ, int BLOCK>
+template <class L, class CT, class ST, int EQ, int BLOCK, bool KEEP>
 __global__ void __launch_bounds__(BLOCK, batch_min_blocks<BLOCK>())
-    k_step_batch(const BatchTables<CT> t, const SolveDesc<CT>* descs, const Tile* tiles, int ntiles, int parity) {
+    k_step_batch(const LatTables<CT> t, const SolveDesc<CT>* descs, const Tile* tiles, int ntiles, int parity) {
   __shared__ SolveDesc<CT> sd;
   chain_release();
   chain_wait();
@@ -863,7 +979,7 @@ __global__ void __launch_bounds__(BLOCK, batch_min_blocks<BLOCK>())
     }
     const int cell = tile.cell0 + int(threadIdx.x);
     if (cell >= sd.ncells) continue;
-    batch_cell<L, CT, ST, EQ>(t, sd, cell, parity, static_cast<NoHigh*>(nullptr));
+    batch_cell<L, CT, ST, EQ, KEEP>(t, sd, cell, parity, static_cast<NoHigh*>(nullptr));
   }
 }
 
@@ -872,7 +988,7 @@ __global__ void __launch_bounds__(BLOCK, batch_min_blocks<BLOCK>())
 // memory with its descriptor, as k_step_high does for one solve.
 template <class L, class CT, class ST, int EQ>
 __global__ void __launch_bounds__(kBlock, 3)
-    k_step_batch_high(const BatchTables<CT> t, const SolveDesc<CT>* descs, const HighParams<CT>* highs,
+    k_step_batch_high(const LatTables<CT> t, const SolveDesc<CT>* descs, const HighParams<CT>* highs,
                       const Tile* tiles, int ntiles, int parity) {
   __shared__ SolveDesc<CT> sd;
   __shared__ HighTable<L, CT> tab;
@@ -890,7 +1006,7 @@ __global__ void __launch_bounds__(kBlock, 3)
     }
     const int cell = tile.cell0 + int(threadIdx.x);
     if (cell >= sd.ncells) continue;
-    batch_cell<L, CT, ST, EQ>(t, sd, cell, parity, &tab);
+    batch_cell<L, CT, ST, EQ, true>(t, sd, cell, parity, &tab);
   }
 }
 
@@ -901,13 +1017,17 @@ __global__ void __launch_bounds__(kBlock, 3)
 namespace lbm {
 
 template <class L, class CT, class ST, int EQ, class F>
-lbm_status batch_by_block(int block, F&& fn) {
-  switch (block) {
-    case 64: return fn(k_step_batch<L, CT, ST, EQ, 64>);
-    case 128: return fn(k_step_batch<L, CT, ST, EQ, 128>);
-    case 256: return fn(k_step_batch<L, CT, ST, EQ, 256>);
-  }
-  return set_error(LBM_ERR_ARG, "batched tile size must be 64, 128 or 256 cells");
+lbm_status batch_by_block(int block, bool keep, F&& fn) {
+  auto go = [&](auto k) -> lbm_status {
+    constexpr bool K = decltype(k)::value;
+    switch (block) {
+      case 64: return fn(k_step_batch<L, CT, ST, EQ, 64, K>);
+      case 128: return fn(k_step_batch<L, CT, ST, EQ, 128, K>);
+      case 256: return fn(k_step_batch<L, CT, ST, EQ, 256, K>);
+    }
+    return set_error(LBM_ERR_ARG, "batched tile size must be 64, 128 or 256 cells");
+  };
+  return keep ? go(std::true_type{}) : go(std::false_type{});
 }
 
 template <class L, class F>
@@ -928,18 +1048,18 @@ lbm_status batch_kernel_high(int store, int eq, F&& fn) {
 }
 
 template <class L, class F>
-lbm_status batch_kernel(int store, int eq, int block, F&& fn) {
+lbm_status batch_kernel(int store, int eq, int block, bool keep, F&& fn) {
   if (store == LBM_F32) {
-    if (eq == LBM_NSE) return batch_by_block<L, float, float, LBM_NSE>(block, fn);
-    return batch_by_block<L, float, float, LBM_NCDE>(block, fn);
+    if (eq == LBM_NSE) return batch_by_block<L, float, float, LBM_NSE>(block, keep, fn);
+    return batch_by_block<L, float, float, LBM_NCDE>(block, keep, fn);
   }
   if (store == LBM_F16_DEV) {
-    if (eq == LBM_NSE) return batch_by_block<L, float, __half, LBM_NSE>(block, fn);
-    return batch_by_block<L, float, __half, LBM_NCDE>(block, fn);
+    if (eq == LBM_NSE) return batch_by_block<L, float, __half, LBM_NSE>(block, keep, fn);
+    return batch_by_block<L, float, __half, LBM_NCDE>(block, keep, fn);
   }
   if (store == LBM_BF16_DEV) {
-    if (eq == LBM_NSE) return batch_by_block<L, float, __nv_bfloat16, LBM_NSE>(block, fn);
-    return batch_by_block<L, float, __nv_bfloat16, LBM_NCDE>(block, fn);
+    if (eq == LBM_NSE) return batch_by_block<L, float, __nv_bfloat16, LBM_NSE>(block, keep, fn);
+    return batch_by_block<L, float, __nv_bfloat16, LBM_NCDE>(block, keep, fn);
   }
   return set_error(LBM_ERR_NOT_IMPLEMENTED, "batched execution supports F32, F16_DEV and BF16_DEV storage");
 }
@@ -949,17 +1069,15 @@ lbm_status BatchLaunch<KIND>::launch(const BatchGroup& g, int parity, cudaStream
   using L = Lat<KIND>;
   if (g.high) {
     return batch_kernel_high<L>(g.store, g.eq, [&](auto kernel) -> lbm_status {
-      const BatchTables<float>& t = *static_cast<const BatchTables<float>*>(g.tables);
+      const LatTables<float>& t = *static_cast<const LatTables<float>*>(g.tables);
       cudaError_t err = launch_chained(kernel, g.grid, kBlock, 0, stream, t,
                                        static_cast<const SolveDesc<float>*>(g.d_desc),
                                        static_cast<const HighParams<float>*>(g.d_high), g.d_tiles, g.ntiles, parity);
       return err == cudaSuccess ? LBM_OK : cuda_error(err, "batched step launch");
     });
   }
-  return batch_kernel<L>(g.store, g.eq, g.block, [&](auto kernel) -> lbm_status {
-    using Kern = decltype(kernel);
-    (void)sizeof(Kern);
-    const BatchTables<float>& t = *static_cast<const BatchTables<float>*>(g.tables);
+  return batch_kernel<L>(g.store, g.eq, g.block, g.keep != 0, [&](auto kernel) -> lbm_status {
+    const LatTables<float>& t = *static_cast<const LatTables<float>*>(g.tables);
     cudaError_t err = launch_chained(kernel, g.grid, g.block, 0, stream, t,
                                      static_cast<const SolveDesc<float>*>(g.d_desc), g.d_tiles, g.ntiles, parity);
     return err == cudaSuccess ? LBM_OK : cuda_error(err, "batched step launch");
@@ -967,16 +1085,16 @@ lbm_status BatchLaunch<KIND>::launch(const BatchGroup& g, int parity, cudaStream
 }
 
 template <int KIND>
-lbm_status BatchLaunch<KIND>::occupancy(int store, int eq, int block, int high, int* blocks_per_sm) {
+lbm_status BatchLaunch<KIND>::occupancy(const BatchGroup& g, int* blocks_per_sm) {
   using L = Lat<KIND>;
-  if (high) {
-    return batch_kernel_high<L>(store, eq, [&](auto kernel) -> lbm_status {
+  if (g.high) {
+    return batch_kernel_high<L>(g.store, g.eq, [&](auto kernel) -> lbm_status {
       cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, kBlock, 0);
       return err == cudaSuccess ? LBM_OK : cuda_error(err, "occupancy query");
     });
   }
-  return batch_kernel<L>(store, eq, block, [&](auto kernel) -> lbm_status {
-    cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, block, 0);
+  return batch_kernel<L>(g.store, g.eq, g.block, g.keep != 0, [&](auto kernel) -> lbm_status {
+    cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, g.block, 0);
     return err == cudaSuccess ? LBM_OK : cuda_error(err, "occupancy query");
   });
 }
@@ -1089,11 +1207,13 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       if (m->eq == LBM_NSE) go(k_step_high<L, CT, ST, LBM_NSE>, grid, kBlock, 0, p, hp);
       else go(k_step_high<L, CT, ST, LBM_NCDE>, grid, kBlock, 0, p, hp);
     } else if (!collide_on) {
-      go(k_step<L, CT, ST, LBM_NSE, false>, grid, kBlock, 0, p);
+      go(k_step<L, CT, ST, LBM_NSE, false, true>, grid, kBlock, 0, p);
     } else if (m->eq == LBM_NSE) {
-      go(k_step<L, CT, ST, LBM_NSE, true>, grid, kBlock, 0, p);
+      if (m->s_high == 1.0) go(k_step<L, CT, ST, LBM_NSE, true, false>, grid, kBlock, 0, p);
+      else go(k_step<L, CT, ST, LBM_NSE, true, true>, grid, kBlock, 0, p);
     } else {
-      go(k_step<L, CT, ST, LBM_NCDE, true>, grid, kBlock, 0, p);
+      if (m->s_high == 1.0) go(k_step<L, CT, ST, LBM_NCDE, true, false>, grid, kBlock, 0, p);
+      else go(k_step<L, CT, ST, LBM_NCDE, true, true>, grid, kBlock, 0, p);
     }
     if (err != cudaSuccess) return cuda_error(err, "collide-stream launch");
     m->cur ^= 1;

@@ -51,7 +51,7 @@ __device__ __forceinline__ uint16_t enc16(float v) {
   return b;
 }
 
-template <class L, class ST, int EQ, bool COLLIDE, bool FULL>
+template <class L, class ST, int EQ, bool COLLIDE, bool FULL, bool KEEP>
 __global__ void __launch_bounds__(kRowThreads, 2)
     k_step_rows(const StepParams<float> p, const RowParams rp, const ST* fin, ST* fout, float* phi) {
   constexpr int Q = L::Q, RM = L::RMAX, PITCH = kRowPitch, WARPS = kRowThreads / 32;
@@ -184,13 +184,14 @@ __global__ void __launch_bounds__(kRowThreads, 2)
       if constexpr (COLLIDE) {
         const int cell = r * nx + x;
         float F[3];
-        body_force(p.force_a, p.force_b, p.force_tab, x, y, z, F);
+        const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, x, y, z, F);
         float phi_prev = 0.f, phi_now = 0.f;
         if constexpr (EQ == LBM_NCDE) phi_prev = phi[cell];
         constexpr bool AG = GradTerm<L, EQ>::kOn;
         float gr[3];
-        if constexpr (AG) cell_field_gradient<L>(p, cell, x, y, z, gr);
-        collide<L, float, EQ, true>(f, p, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), AG ? gr : nullptr);
+        const float* grad = nullptr;
+        if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
+        collide<L, float, EQ, true, KEEP>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
         if constexpr (EQ == LBM_NCDE) phi[cell] = phi_now;
         if constexpr (AG && EQ == LBM_NSE) {
           if (p.grad_on) p.rho_out[cell] = phi_now;
@@ -459,17 +460,18 @@ __global__ void __launch_bounds__(kRowThreads, 2)
     }
     // the collision in moment space, in FP32 (the CUDA-core kernel's code)
     const int cell = r * nx + x;
-    float F[3] = {0.f, 0.f, 0.f};
-    body_force(p.force_a, p.force_b, p.force_tab, x, y, z, F);
+    float F[3];
+    const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, x, y, z, F);
     float phi_prev = 0.f, phi_now = 0.f;
     if constexpr (EQ == LBM_NCDE) phi_prev = live ? phi[cell] : 0.f;
     constexpr bool AG = GradTerm<L, EQ>::kOn;
     float gr[3] = {0.f, 0.f, 0.f};
+    const float* grad = nullptr;
     if constexpr (AG) {
-      if (live) cell_field_gradient<L>(p, cell, x, y, z, gr);
+      if (live) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
     }
     float h[R];
-    collide_moments<L, float, EQ, true>(mu, p, F, phi_prev, phi_now, h, AG ? gr : nullptr);
+    collide_moments<L, float, EQ, true>(mu, p, p, forced, F, phi_prev, phi_now, h, grad);
     if constexpr (EQ == LBM_NCDE) {
       if (live) phi[cell] = phi_now;
     }
@@ -625,17 +627,21 @@ bool RowLaunch<KIND>::plan(const lbm_model* m, RowPlan* out, bool tensor, bool h
   return true;
 }
 
-// The kernel of a model: storage type, equation, collision on / off (stream only).
+// The kernel of a model: storage type, equation, collision on / off (stream only), s_high = 1 or not.
 template <class L, class ST, bool FULL, class F>
-lbm_status row_kernel_full(int eq, bool collide, F&& fn) {
-  if (!collide) return fn(k_step_rows<L, ST, LBM_NSE, false, FULL>);
-  if (eq == LBM_NSE) return fn(k_step_rows<L, ST, LBM_NSE, true, FULL>);
-  return fn(k_step_rows<L, ST, LBM_NCDE, true, FULL>);
+lbm_status row_kernel_full(const lbm_model* m, bool collide, F&& fn) {
+  if (!collide) return fn(k_step_rows<L, ST, LBM_NSE, false, FULL, true>);
+  if (m->eq == LBM_NSE) {
+    if (m->s_high == 1.0) return fn(k_step_rows<L, ST, LBM_NSE, true, FULL, false>);
+    return fn(k_step_rows<L, ST, LBM_NSE, true, FULL, true>);
+  }
+  if (m->s_high == 1.0) return fn(k_step_rows<L, ST, LBM_NCDE, true, FULL, false>);
+  return fn(k_step_rows<L, ST, LBM_NCDE, true, FULL, true>);
 }
 template <class L, class ST, class F>
-lbm_status row_kernel(int eq, bool collide, bool full, F&& fn) {
-  if (full) return row_kernel_full<L, ST, true>(eq, collide, fn);
-  return row_kernel_full<L, ST, false>(eq, collide, fn);
+lbm_status row_kernel(const lbm_model* m, bool collide, F&& fn) {
+  if (m->n[0] == kRowPitch) return row_kernel_full<L, ST, true>(m, collide, fn);
+  return row_kernel_full<L, ST, false>(m, collide, fn);
 }
 
 // The tensor-core kernel of a model: fn(kernel, storage tag).
@@ -666,9 +672,8 @@ lbm_status RowLaunch<KIND>::configure(const lbm_model* m, const RowPlan& plan, b
     return LBM_OK;
   };
   if (plan.tensor && collide) return row_tc_kernel<L>(m->store, m->eq, plan.high, [&](auto k, auto) { return set(k); });
-  const bool full = m->n[0] == kRowPitch;
-  if (m->store == LBM_F16_DEV) return row_kernel<L, __half>(m->eq, collide, full, set);
-  return row_kernel<L, __nv_bfloat16>(m->eq, collide, full, set);
+  if (m->store == LBM_F16_DEV) return row_kernel<L, __half>(m, collide, set);
+  return row_kernel<L, __nv_bfloat16>(m, collide, set);
 }
 
 template <int KIND>
@@ -690,11 +695,9 @@ lbm_status RowLaunch<KIND>::launch(const lbm_model* m, const RowPlan& plan, cons
     };
     return row_tc_kernel<L>(m->store, m->eq, plan.high, go_tc);
   }
-  const bool full = m->n[0] == kRowPitch;
   if (m->store == LBM_F16_DEV)
-    return row_kernel<L, __half>(m->eq, collide, full, [&](auto kernel) { return go(kernel, __half()); });
-  return row_kernel<L, __nv_bfloat16>(m->eq, collide, full,
-                                      [&](auto kernel) { return go(kernel, __nv_bfloat16()); });
+    return row_kernel<L, __half>(m, collide, [&](auto kernel) { return go(kernel, __half()); });
+  return row_kernel<L, __nv_bfloat16>(m, collide, [&](auto kernel) { return go(kernel, __nv_bfloat16()); });
 }
 
 }  // namespace lbm

@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(128, TcShape<L, HI>::CTAS)
       y = nb.y;
       z = nb.z;
     }
-    float F[3] = {0.f, 0.f, 0.f};
-    body_force(p.force_a, p.force_b, p.force_tab, x, y, z, F);
+    float F[3];
+    const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, x, y, z, F);
     float phi_prev = 0.f, phi_now = 0.f;
     if constexpr (EQ == LBM_NCDE) phi_prev = live ? phi[cell] : 0.f;
     // HI: z_r = a_r y_r from the higher-row columns of the forward product
@@ -253,10 +253,11 @@ __global__ void __launch_bounds__(128, TcShape<L, HI>::CTAS)
     float h[R];
     constexpr bool AG = GradTerm<L, EQ>::kOn;
     float gr[3] = {0.f, 0.f, 0.f};
+    const float* grad = nullptr;
     if constexpr (AG) {
-      if (live) cell_field_gradient<L>(p, cell, x, y, z, gr);
+      if (live) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
     }
-    collide_moments<L, float, EQ, true>(mu, p, F, phi_prev, phi_now, h, AG ? gr : nullptr);
+    collide_moments<L, float, EQ, true>(mu, p, p, forced, F, phi_prev, phi_now, h, grad);
     if constexpr (EQ == LBM_NCDE) {
       if (live) phi[cell] = phi_now;
     }
@@ -509,16 +510,17 @@ __global__ void __launch_bounds__(128, Tc32Shape<L>::CTAS)
     int xn, yn, zn;
     load_tile(tile + int(gridDim.x), fn, xn, yn, zn);
     // the low-order collision on the CUDA cores meanwhile
-    float F[3] = {0.f, 0.f, 0.f};
-    body_force(p.force_a, p.force_b, p.force_tab, x, y, z, F);
+    float F[3];
+    const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, x, y, z, F);
     float phi_prev = 0.f, phi_now = 0.f;
     if constexpr (EQ == LBM_NCDE) phi_prev = live ? phi[cell] : 0.f;
     constexpr bool AG = GradTerm<L, EQ>::kOn;
     float gr[3] = {0.f, 0.f, 0.f};
+    const float* grad = nullptr;
     if constexpr (AG) {
-      if (live) cell_field_gradient<L>(p, cell, x, y, z, gr);
+      if (live) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
     }
-    collide<L, float, EQ, false>(f, p, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), AG ? gr : nullptr);
+    collide<L, float, EQ, false, true>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
     if constexpr (EQ == LBM_NCDE) {
       if (live) phi[cell] = phi_now;
     }
