@@ -158,7 +158,7 @@ cudaError_t ensure(void** ptr, size_t* cap, size_t bytes) {
 
 void fill_desc(const lbm_model* m, SolveDesc<float>* d) {
   StepParams<float> p;
-  make_step_params<float>(m, &p);
+  make_step_params(m, &p);
   std::memset(d, 0, sizeof(*d));
   static_cast<Rates<float>&>(*d) = p;
   for (int a = 0; a < 3; ++a) d->n[a] = p.n[a];
@@ -275,7 +275,7 @@ lbm_status rebuild(lbm_batch* b) {
       auto t = b->tile.find(std::make_tuple(m->lat->kind, m->store, m->eq));
       gh.g.block = high || t == b->tile.end() ? kBlock : t->second;
       StepParams<float> p;
-      make_step_params<float>(m, &p);
+      make_step_params(m, &p);
       gh.tables = p;
       gh.members.push_back(m);
     } else {

@@ -25,8 +25,8 @@ lbm_status cuda_error(cudaError_t err, const char* what) {
                    std::string(what) + ": " + cudaGetErrorName(err) + " (" + cudaGetErrorString(err) + ")");
 }
 
-template <class CT>
-void make_step_params(const lbm_model* m, StepParams<CT>* p) {
+template <class CT, class FT>
+void make_step_params(const lbm_model* m, StepParams<CT, FT>* p) {
   const lbm_lattice* L = m->lat;
   std::memset(p, 0, sizeof(*p));
   const int R = L->R, d = L->d;
@@ -147,12 +147,12 @@ void make_step_params(const lbm_model* m, StepParams<CT>* p) {
       const int e = L->e[i * 3 + a];
       if (e != 0) mult = e < 0 ? -e : e;  // every non-zero component of a velocity has the same size
       if (e != 0 && lead == 0) lead = e < 0 ? -1 : 1;
-      if (a < d) wmr[1 + a] += L->w[i] * e * e;
+      if (a < d) wmr[1 + a] += w[i] * e * e;
     }
-    wmr[0] += L->w[i];
+    wmr[0] += w[i];
     p->w[i] = CT(w[i]);
     p->wm[i] = CT(lead * mult * w[i]);
-    p->wref[i] = CT(L->w[i] * rho_ref);
+    p->wref[i] = CT(w[i] * rho_ref);
   }
   for (int k = 0; k < 4; ++k) p->wmr[k] = CT(rho_ref * wmr[k]);
   // NCDE variants (App. A): a1 folds into the first-order factor of M1G (moment variant);
@@ -165,9 +165,9 @@ void make_step_params(const lbm_model* m, StepParams<CT>* p) {
       p->h1[a] = CT(uc * (1.0 - 0.5 * s1 - s1 * m->a1) * iN[1 + a]);
       p->s1[a] = CT(s1);
       p->kfac[a] = CT(1.0 / s1 - 0.5);
-      p->cde_coef[a] = m->ncde_variant == LBM_NCDE_CDE ? CT(m->u_const[a] * s1 / m->cs2_eq * L->c[a]) : CT(0);
+      p->cde_coef[a] = CT(m->ncde_variant == LBM_NCDE_CDE ? m->u_const[a] * s1 / m->cs2_eq * L->c[a] : 0.0);
     }
-    p->nonlin_rate = m->ncde_variant == LBM_NCDE_RATE ? CT(m->nonlin) : CT(0);
+    p->nonlin_rate = CT(m->ncde_variant == LBM_NCDE_RATE ? m->nonlin : 0.0);
     p->a1 = CT(m->a1);
     p->half0 = CT((1.0 - 0.5 * m->s[0]) * iN[0]);
   }
@@ -183,7 +183,7 @@ void make_step_params(const lbm_model* m, StepParams<CT>* p) {
   } else if (m->eq == LBM_NCDE && m->a2 != 0.0) {
     p->grad_on = 1;
     for (int a = 0; a < d; ++a) p->gscale[a] = CT(m->a2 / (2.0 * L->c[a] * L->c[a]));
-    p->grad_in = static_cast<const CT*>(m->psi);
+    p->grad_in = static_cast<const FT*>(m->psi);
   }
   p->sh_rho_ref = CT(sh * rho_ref);
   p->s_high = CT(sh);
@@ -195,11 +195,12 @@ void make_step_params(const lbm_model* m, StepParams<CT>* p) {
   const bool force = m->eq == LBM_NSE && m->force_A != 0.0;
   p->force_a = force ? m->force_a : 0;
   p->force_b = force ? m->force_b : -1;
-  p->force_tab = static_cast<const CT*>(m->force_tab);
+  p->force_tab = static_cast<const FT*>(m->force_tab);
 }
 
-template void make_step_params<float>(const lbm_model*, StepParams<float>*);
-template void make_step_params<double>(const lbm_model*, StepParams<double>*);
+template void make_step_params<float, float>(const lbm_model*, StepParams<float>*);
+template void make_step_params<double, double>(const lbm_model*, StepParams<double>*);
+template void make_step_params<F2, float>(const lbm_model*, StepParams<F2, float>*);
 
 double high_rate(const lbm_model* m, int order) {
   const double s = order <= kMaxOrder ? m->s_order[order] : 0.0;

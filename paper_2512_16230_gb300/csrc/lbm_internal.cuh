@@ -9,6 +9,7 @@
 #include <string>
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "lattices.cuh"
 #include "lbm_mrt.h"
 
@@ -197,19 +198,24 @@ struct Tc32Params {
   int no_issue;         // test hook: issue no matrix product (every wait then runs out)
 };
 
-// Row-staged collide-stream kernel (16-bit storage, row_kernels.cuh): row buffers of kRowPitch
-// cells per population (the largest n_x; one cell per thread of a kRowThreads CTA), up to
-// kRowMaxStages buffers behind kRowBarBytes of mbarriers and counters.
+// Row-staged collide-stream kernels (16-bit storage, row_kernels.cuh): buffers of kRowPitch cells per
+// population, up to kRowMaxStages of them behind a head of mbarriers and tables. The CUDA-core kernel
+// fills a buffer with a tile of whole x-rows (as many as fit) and gives every thread two cells; the
+// tensor-core kernel with one row (kRowThreads = one cell per thread).
 constexpr int kRowPitch = 256;
 constexpr int kRowThreads = kRowPitch;
+constexpr int kRowPairs = kRowPitch / 2;  // threads of the CUDA-core kernel
 constexpr int kRowMaxStages = 8;
 constexpr int kRowBarBytes = 256;
+constexpr int kRowHeadBytes = 1024;  // mbarriers, source offsets and velocity components
 struct RowParams {
   // byte offset from the start of row r of the population arrays to the pull-source row of
   // population i, 2 (i N - (e_iy + e_iz n_y) n_x), valid for rows away from the y and z faces
   int64_t src_off[kMaxQ];
   int8_t ey[kMaxQ], ez[kMaxQ];  // y and z velocity components (source rows next to a face)
   int nrows;                    // n_y n_z
+  int rpt, ntiles;              // CUDA-core kernel: rows per tile and number of tiles
+  int chunks, lanes;            // 16-byte pieces of a row; lanes that copy one population (a power of two)
   int stages;                   // row buffers per CTA
   uint32_t stage_bytes;         // Q * pitch * 2
   int* status;
@@ -231,8 +237,8 @@ struct RowLaunch {
   // `high`: with one rate per order >= 4 (needs `tensor`)
   static bool plan(const lbm_model* m, RowPlan* out, bool tensor = false, bool high = false);
   static lbm_status configure(const lbm_model* m, const RowPlan& plan, bool collide);
-  static lbm_status launch(const lbm_model* m, const RowPlan& plan, const StepParams<float>& p, const void* fin,
-                           void* fout, float* phi, bool collide);
+  static lbm_status launch(const lbm_model* m, const RowPlan& plan, const StepParams<float>& p,
+                           const StepParams<F2, float>& p2, const void* fin, void* fout, float* phi, bool collide);
 };
 
 // Multiply-high division by a runtime divisor 2 <= d < 2^31, exact for numerators below 2^31:
@@ -422,8 +428,8 @@ void batch_mark_dirty(lbm_batch* b);
 lbm_status setup_lattice_fp64(lbm_lattice* lat);
 
 // Host-side construction of the step parameters from a model.
-template <class CT>
-void make_step_params(const lbm_model* m, StepParams<CT>* p);
+template <class V, class FT>
+void make_step_params(const lbm_model* m, StepParams<V, FT>* p);
 template <class CT>
 void make_high_params(const lbm_model* m, HighParams<CT>* hp);
 // true when some row of order >= 4 relaxes with a rate other than s_high

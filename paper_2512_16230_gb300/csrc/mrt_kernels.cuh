@@ -70,7 +70,18 @@ __device__ __forceinline__ void k1_store(T* p, T v) {
 
 template <class CT>
 __device__ __forceinline__ CT fmaf_t(CT a, CT b, CT c) {
-  return fma(a, b, c);
+  if constexpr (std::is_same<CT, F2>::value) return fma2(a, b, c);
+  else return fma(a, b, c);
+}
+
+// a b where the product's only use is in a sum. The assembler fuses a packed product into the packed
+// addition that takes it, whatever the rounding modifiers say, and would round once where the scalar
+// kernels round twice; a multiply-add with zero is not fused. (For every product it costs registers:
+// rD3Q53 FP16 256x256x192 448 -> 472 us a step.)
+template <class V>
+__device__ __forceinline__ V product(V a, V b) {
+  if constexpr (std::is_same<V, F2>::value) return fma2(a, b, F2(0.f));
+  else return a * b;
 }
 
 // acc + c * x for a compile-time integer c
@@ -78,7 +89,7 @@ template <int C, class CT>
 __device__ __forceinline__ CT axpy_c(CT x, CT acc) {
   if constexpr (C == 1) return acc + x;
   else if constexpr (C == -1) return acc - x;
-  else return fma(CT(C), x, acc);
+  else return fmaf_t(CT(C), x, acc);
 }
 
 // Sums of one primitive direction d: s_deg = sum_m m^deg (f_md +- f_-md), + for even degree, - for
@@ -623,13 +634,13 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
         // s_a(phi) = 1 / ((1/s_a - 1/2)(1 + nonlin phi^2) + 1/2)
         const V g = fmaf_t(rt.nonlin_rate, phi * phi, V(1.f));
         s1 = V(1.f) / fmaf_t(rt.kfac[A], g, V(0.5f));
-        const V half1 = V(1.f) - s1 * (V(0.5f) + rt.a1);
-        const V relax = (s1 - rt.s_high) * n1;
+        const V half1 = V(1.f) - product(s1, V(0.5f) + rt.a1);
+        const V relax = product(s1 - rt.s_high, n1);
         gN[1 + A] = lt.iN[1 + A] * (fmaf_t(rt.s_high, m1, half1 * (rt.u_const[A] * dphi)) - relax);
       } else {
         gN[1 + A] = fmaf_t(rt.A[1 + A], m1, fmaf_t(rt.NB[1 + A], n1, rt.h1[A] * dphi));
       }
-      if (gr != nullptr) gN[1 + A] = gN[1 + A] - lt.iN[1 + A] * (s1 * gr[A]);
+      if (gr != nullptr) gN[1 + A] = gN[1 + A] - product(lt.iN[1 + A], s1 * gr[A]);
       constexpr int AA = row2<D>(A, A);
       me[AA] = fmaf_t(rt.pc[A], Dphi, lt.nd0[A] * phi);
       neq[AA] = fmaf_t(lt.nd0[A], mu[0], mu[AA]) - me[AA];
@@ -644,9 +655,9 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
       gN[AA] = g;
       static_for<D - 1>([&](auto ii) {
         constexpr int I = decltype(ii)::value, B = other_axis(A, I), ABB = row3<D>(A, B, B);
-        if constexpr (B > A) gN[row2<D>(A, B)] = rt.NB[row2<D>(A, B)] * mu[row2<D>(A, B)];
+        if constexpr (B > A) gN[row2<D>(A, B)] = product(rt.NB[row2<D>(A, B)], mu[row2<D>(A, B)]);
         neq[ABB] = fmaf_t(lt.nd0[B], mu[1 + A], mu[ABB]);
-        gN[ABB] = rt.NB[ABB] * neq[ABB];
+        gN[ABB] = product(rt.NB[ABB], neq[ABB]);
       });
       if constexpr (!L::SINGLE) {
         constexpr int AAA = row3<D>(A, A, A);
@@ -655,10 +666,10 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
           constexpr int I = decltype(ii)::value, B = other_axis(A, I);
           v = fmaf_t(lt.be[A][I], neq[row3<D>(A, B, B)], v);
         });
-        gN[AAA] = rt.NB[AAA] * v;
+        gN[AAA] = product(rt.NB[AAA], v);
       }
     });
-    if constexpr (D == 3) gN[row3<3>(0, 1, 2)] = rt.NB[row3<3>(0, 1, 2)] * mu[row3<3>(0, 1, 2)];
+    if constexpr (D == 3) gN[row3<3>(0, 1, 2)] = product(rt.NB[row3<3>(0, 1, 2)], mu[row3<3>(0, 1, 2)]);
   }
   rows_to_monomials<L>(lt, gN, h);
   if constexpr (DEV) h[0] = h[0] - rt.sh_rho_ref;
@@ -773,6 +784,18 @@ __device__ __forceinline__ bool body_force(int force_a, int force_b, const CT* f
   return true;
 }
 
+// The same for two cells side by side.
+__device__ __forceinline__ bool body_force(int force_a, int force_b, const float* force_tab, const F2 (&invc)[3],
+                                           int x, int y, int z, F2 (&F)[3]) {
+  if (force_b < 0) return false;
+  const int ib = force_b == 0 ? x : (force_b == 1 ? y : z);
+  const F2 v(force_tab[ib], force_tab[force_b == 0 ? ib + 1 : ib]);
+  F[0] = force_a == 0 ? v * invc[0] : F2(0.f);
+  F[1] = force_a == 1 ? v * invc[1] : F2(0.f);
+  F[2] = force_a == 2 ? v * invc[2] : F2(0.f);
+  return true;
+}
+
 // Gradient terms of the source moments: the delta4 term of M2G (Eq. (M2Ga)) on the single-speed
 // lattices needs grad rho, the cross-diffusion term of M1G (Eq. (M-NCDE-6)) grad psi. Both take
 // gr_a = gscale_a (g(x + e_a) - g(x - e_a)), the central difference of the cell field p.grad_in at
@@ -782,19 +805,39 @@ struct GradTerm {
   static constexpr bool kOn = (L::SINGLE && EQ == LBM_NSE) || EQ == LBM_NCDE;
 };
 template <class L, class CT>
-__device__ __forceinline__ const CT* cell_field_gradient(const Rates<CT>& p, const int (&n)[3], const CT* g, int cell,
-                                                         int x, int y, int z, CT (&gr)[3]) {
-  if (!p.grad_on) return nullptr;
+__device__ __forceinline__ void field_differences(const int (&n)[3], const CT* g, int cell, int x, int y, int z,
+                                                  CT (&d)[3]) {
   const int nx = n[0], ny = n[1];
   const int xp = x + 1 == nx ? -x : 1, xm = x == 0 ? nx - 1 : -1;
-  gr[0] = p.gscale[0] * (g[cell + xp] - g[cell + xm]);
+  d[0] = g[cell + xp] - g[cell + xm];
   const int yp = (y + 1 == ny ? -y : 1) * nx, ym = (y == 0 ? ny - 1 : -1) * nx;
-  gr[1] = p.gscale[1] * (g[cell + yp] - g[cell + ym]);
+  d[1] = g[cell + yp] - g[cell + ym];
   if constexpr (L::D == 3) {
     const int nz = n[2], nxy = nx * ny;
     const int zp = (z + 1 == nz ? -z : 1) * nxy, zm = (z == 0 ? nz - 1 : -1) * nxy;
-    gr[2] = p.gscale[2] * (g[cell + zp] - g[cell + zm]);
+    d[2] = g[cell + zp] - g[cell + zm];
   }
+}
+template <class L, class CT>
+__device__ __forceinline__ const CT* cell_field_gradient(const Rates<CT>& p, const int (&n)[3], const CT* g, int cell,
+                                                         int x, int y, int z, CT (&gr)[3]) {
+  if (!p.grad_on) return nullptr;
+  field_differences<L>(n, g, cell, x, y, z, gr);
+  static_for<L::D>([&](auto a) { gr[decltype(a)::value] = p.gscale[decltype(a)::value] * gr[decltype(a)::value]; });
+  return gr;
+}
+// The same for two cells side by side, (x, y, z) and (x + 1, y, z).
+template <class L>
+__device__ __forceinline__ const F2* cell_field_gradient(const Rates<F2>& p, const int (&n)[3], const float* g,
+                                                         int cell, int x, int y, int z, F2 (&gr)[3]) {
+  if (!p.grad_on) return nullptr;
+  float d0[3], d1[3];
+  field_differences<L>(n, g, cell, x, y, z, d0);
+  field_differences<L>(n, g, cell + 1, x + 1, y, z, d1);
+  static_for<L::D>([&](auto a) {
+    constexpr int A = decltype(a)::value;
+    gr[A] = p.gscale[A] * F2(d0[A], d1[A]);
+  });
   return gr;
 }
 
@@ -1103,7 +1146,7 @@ lbm_status BatchLaunch<KIND>::occupancy(const BatchGroup& g, int* blocks_per_sm)
 template <class L, class CT, class ST>
 lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
   StepParams<CT> p;
-  make_step_params<CT>(m, &p);
+  make_step_params(m, &p);
   const int grid = (m->ncells + kBlock - 1) / kBlock;
   CT* phi = static_cast<CT*>(m->phi_prev);
   const bool high = collide_on && has_high_rates(m);
@@ -1151,6 +1194,7 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
   // 16-bit storage: the row-staged gather where it applies (or is forced), with the contractions
   // on the CUDA cores or, when the tensor cores are selected, on tcgen05
   [[maybe_unused]] RowPlan rplan;
+  [[maybe_unused]] StepParams<F2, float> p2;  // the row-staged CUDA-core kernel works on two cells at a time
   bool rows = false;
   if constexpr (is_deviation_storage<ST>()) {
     if (m->gather == LBM_GATHER_ROWS && high && !tensor)
@@ -1162,17 +1206,23 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       if (rows && nsteps > 0) {
         const lbm_status st = RowLaunch<L::KIND>::configure(m, rplan, collide_on);
         if (st != LBM_OK) return st;
+        make_step_params(m, &p2);
       }
     }
   }
   const bool hist = collide_on && m->m2g_aniso;
   p.grad_on = collide_on && p.grad_on;
+  if (rows) p2.grad_on = p.grad_on;
   for (int64_t s = 0; s < nsteps; ++s) {
     const ST* fin = static_cast<const ST*>(m->f[m->cur]);
     ST* fout = static_cast<ST*>(m->f[m->cur ^ 1]);
     if (hist) {
       p.grad_in = static_cast<const CT*>(m->rho_hist[m->hist_cur]);
       p.rho_out = static_cast<CT*>(m->rho_hist[m->hist_cur ^ 1]);
+      if constexpr (std::is_same<CT, float>::value) {
+        p2.grad_in = p.grad_in;
+        p2.rho_out = p.rho_out;
+      }
     }
     cudaError_t err = cudaSuccess;
     auto go = [&](auto kernel, int blocks, int threads, size_t smem, const auto&... args) {
@@ -1181,7 +1231,7 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
     bool done = false;
     if constexpr (is_deviation_storage<ST>()) {
       if (rows) {
-        const lbm_status st = RowLaunch<L::KIND>::launch(m, rplan, p, fin, fout, phi, collide_on);
+        const lbm_status st = RowLaunch<L::KIND>::launch(m, rplan, p, p2, fin, fout, phi, collide_on);
         if (st != LBM_OK) return st;
         done = true;
       } else if (tensor) {
@@ -1227,7 +1277,7 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
 template <class L, class CT, class ST>
 lbm_status launch_init_typed(lbm_model* m, const double* rho_or_phi, const double* u) {
   StepParams<CT> p;
-  make_step_params<CT>(m, &p);
+  make_step_params(m, &p);
   const int grid = (m->ncells + kBlock - 1) / kBlock;
   ST* fout = static_cast<ST*>(m->f[m->cur]);
   CT* phi = static_cast<CT*>(m->eq == LBM_NSE ? m->rho_hist[m->hist_cur] : m->phi_prev);

@@ -1,21 +1,17 @@
-// Row-staged collide-stream kernel for 16-bit deviation storage (FP16 or BF16 deviations
+// Row-staged collide-stream kernels for 16-bit deviation storage (FP16 or BF16 deviations
 // f_i - w_i rho_ref, collision arithmetic in FP32).
 //
 // The per-thread pull gather and store of k_step move 64 bytes per warp access when a population
 // takes 2 bytes, too little per memory request to keep HBM busy. Here a CTA works on whole x-rows
-// of the grid, one cell per thread, and moves memory in 512-byte warp accesses. For the row (y, z)
-// the pull sources of population i (Eq. (2-2b)) are the cells (x - e_ix, y - e_iy, z - e_iz): the
-// x-row (y - e_iy, z - e_iz) of array i, read with a periodic shift along x. The warps copy these
-// Q source rows into a shared-memory row buffer with 16-byte cp.async copies (one warp instruction
-// per population row, completing on the buffer's mbarrier); the periodic wraps in y and z are the
-// choice of source row, the wrap in x an index wrap: every thread reads its sources at
-// (x - e_ix) mod n_x. After a CTA barrier (every source read) the threads write their
-// post-collision populations back into the buffer at their own x; after the next row's barrier
-// the warps store the Q rows with 16-byte stores. A ring of row buffers keeps the following rows
-// in flight while the current one is collided. The collision is the code of k_step on the same
-// inputs, so the results are bitwise the same.
+// of the grid. For the row (y, z) the pull sources of population i (Eq. (2-2b)) are the cells
+// (x - e_ix, y - e_iy, z - e_iz): the x-row (y - e_iy, z - e_iz) of array i, read with a periodic
+// shift along x. The warps copy these source rows into a shared-memory buffer with 16-byte cp.async
+// copies (up to 512 bytes per warp instruction, completing on the buffer's mbarrier); the periodic
+// wraps in y and z are the choice of source row, the wrap in x an index wrap: a thread reads its
+// sources at (x - e_ix) mod n_x. A ring of buffers keeps the following rows in flight. The collision
+// is the code of k_step on the same inputs, so the results are bitwise the same.
 //
-// The wait for a row's copies is bounded: on timeout (decided for the whole CTA at the next
+// The wait for a buffer's copies is bounded: on timeout (decided for the whole CTA at the next
 // barrier) the CTA records an error in the model's status word, waits for its own copies and
 // returns.
 #pragma once
@@ -51,172 +47,206 @@ __device__ __forceinline__ uint16_t enc16(float v) {
   return b;
 }
 
-template <class L, class ST, int EQ, bool COLLIDE, bool FULL, bool KEEP>
-__global__ void __launch_bounds__(kRowThreads, 2)
-    k_step_rows(const StepParams<float> p, const RowParams rp, const ST* fin, ST* fout, float* phi) {
-  constexpr int Q = L::Q, RM = L::RMAX, PITCH = kRowPitch, WARPS = kRowThreads / 32;
-  constexpr uint32_t ROWB = PITCH * sizeof(ST);  // bytes of one population's row in a buffer
-  static_assert(ROWB == 32 * 16, "a row of the buffer is one 16-byte chunk per lane");
+// Two neighbouring values of a row, decoded into a packed pair; the 32-bit word at a register address
+// plus a compile-time byte offset.
+template <int OFF>
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(OFF));
+  return v;
+}
+template <class ST>
+__device__ __forceinline__ F2 dec16x2(uint32_t b) {
+  return F2(dec16<ST>(uint16_t(b & 0xFFFFu)), dec16<ST>(uint16_t(b >> 16)));
+}
+
+// Resident CTAs per SM (128 threads each). 4 leave 128 registers and, on the largest lattice, two
+// buffers per CTA; with the old populations kept through the collision (s_high != 1) 2 and 255.
+template <bool KEEP>
+constexpr int row_ctas() {
+  return KEEP ? 2 : 4;
+}
+
+// The CUDA-core kernel: a tile of rp.rpt rows (at most kRowPitch cells, consecutive in memory) per
+// buffer, two cells x, x + 1 (x even) per thread in packed FP32 arithmetic. Per tile: the sources from
+// the buffer (one 32-bit shared load for an even e_x, two 16-bit ones for an odd e_x) and their raw
+// moments, a barrier that frees the buffer for the tile stages ahead, the moment-space collision, and
+// 4-byte stores straight to memory (128 bytes per warp).
+//
+// What bounds it: the one-cell form of this kernel (256 threads, results staged back through shared
+// memory) issued 1,425 instructions per cell and was issue-bound at 65% of HBM; packing halves the
+// FP32 arithmetic, a pair's conversion to 16 bits and its store are one instruction, and without the
+// staged stores a buffer is free as soon as it has been read. rD3Q53 FP16 256x256x192 516 -> 448 us a step
+// (88% of HBM at 212 bytes per cell), rD3Q33 96^3 63 -> 29 us (tiles of two rows); with 3 CTAs per SM
+// 454 and 33 us.
+template <class L, class ST, int EQ, bool COLLIDE, bool KEEP>
+__global__ void __launch_bounds__(kRowPairs, row_ctas<KEEP && COLLIDE>())
+    k_step_rows(const StepParams<F2, float> p, const RowParams rp, const ST* fin, ST* fout, float* phi) {
+  constexpr int Q = L::Q, RM = L::RMAX, WARPS = kRowPairs / 32;
+  constexpr uint32_t ROWB = kRowPitch * sizeof(ST);  // bytes of one population in a buffer
   extern __shared__ __align__(128) uint8_t row_smem[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(row_smem);  // every thread's copies of the row landed
-  ST* rows = reinterpret_cast<ST*>(row_smem + kRowBarBytes);
-  const uint32_t rows_s = tc::smem_addr(row_smem + kRowBarBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(row_smem);  // every thread's copies of the tile landed
+  int64_t* s_off = reinterpret_cast<int64_t*>(row_smem + 128);
+  short2* s_e = reinterpret_cast<short2*>(s_off + kMaxQ);
+  static_assert(128 + kMaxQ * (8 + 4) <= kRowHeadBytes, "head of the row buffers");
+  const uint32_t rows_s = tc::smem_addr(row_smem + kRowHeadBytes);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nx = p.n[0], ny = p.n[1], nz = L::D == 3 ? p.n[2] : 1;
   const int G = int(gridDim.x);
-  const int K = (rp.nrows - int(blockIdx.x) + G - 1) / G;  // rows of this CTA (the grid is <= nrows)
-  const int NS = rp.stages;
-  const uint32_t stage_elems = rp.stage_bytes / uint32_t(sizeof(ST));
+  const int K = (rp.ntiles - int(blockIdx.x) + G - 1) / G;  // tiles of this CTA (the grid is <= ntiles)
+  const int NS = rp.stages, RPT = rp.rpt;
   const size_t N = size_t(p.ncells);
-  const size_t pop_bytes = N * sizeof(ST);
-  const int x = tid;
-  // FULL: n_x equals the pitch, every thread has a cell and every lane a 16-byte chunk of a row
-  const bool live = FULL || x < nx;
-  const bool lane_chunk = FULL || lane * 8 < nx;
-  // rows of this CTA are r = blockIdx.x + k G: (y, z) advance by (G mod n_y, G div n_y) with a carry
-  const int gy = G % ny, gz = G / ny;
-  auto advance = [&](int& y, int& z) {
-    y += gy;
-    z += gz;
-    if (y >= ny) {
-      y -= ny;
-      z += 1;
-    }
-  };
   chain_release();
   if (tid == 0) {
-    for (int s = 0; s < NS; ++s) tc::mbar_init(&full[s], kRowThreads);
+    for (int s = 0; s < NS; ++s) tc::mbar_init(&full[s], kRowPairs);
     tc::mbar_fence_init();
+  }
+  if (tid < Q) {
+    s_off[tid] = rp.src_off[tid];
+    s_e[tid] = make_short2(rp.ey[tid], rp.ez[tid]);
   }
   __syncthreads();
   chain_wait();
 
-  // every thread: its chunks of the Q source rows of row (y, z) into buffer s (warp w takes the
-  // populations w, w + 8, ...), then one arrival on the buffer's mbarrier when they have landed
-  auto load_row = [&](int y, int z, int s) {
+  // copies: lane group g of a warp takes the populations warp * groups + g, + 4 groups, ...; lane c of
+  // the group takes 16-byte piece c of the tile's rows
+  const int groups = 32 / rp.lanes;
+  const int c = lane & (rp.lanes - 1), pop0 = warp * groups + lane / rp.lanes, pstep = WARPS * groups;
+  const int cj = c / rp.chunks, cx = (c - cj * rp.chunks) * 8;
+  auto load_tile = [&](int t, int s) {
     if (rp.no_copy) return;  // test hook: nothing lands, every wait on the buffer runs out
-    if (lane_chunk) {
-      const size_t r = size_t(z) * ny + y;
-      const uint8_t* base = reinterpret_cast<const uint8_t*>(fin) + (r * nx + lane * 8) * sizeof(ST);
-      const uint32_t dst = rows_s + uint32_t(s) * rp.stage_bytes + uint32_t(lane * 16);
+    const int r = t * RPT + cj;
+    if (cj < RPT && r < rp.nrows) {
+      int y = r, z = 0;
+      if constexpr (L::D == 3) {
+        z = int(__umulhi(unsigned(r), p.div_m[1]) >> p.div_s[1]);
+        y = r - z * ny;
+      }
+      const uint8_t* base = reinterpret_cast<const uint8_t*>(fin) + (size_t(r) * nx + cx) * sizeof(ST);
+      uint32_t dst = rows_s + uint32_t(s) * rp.stage_bytes + uint32_t(c * 16) + uint32_t(pop0) * ROWB;
       const bool inner = y >= RM && y < ny - RM && (L::D == 2 || (z >= RM && z < nz - RM));
       if (inner) {
-        static_for<(Q + WARPS - 1) / WARPS>([&](auto m) {
-          const int i = warp + WARPS * decltype(m)::value;
-          if (i < Q) bulk::cp_async16(dst + uint32_t(i) * ROWB, base + rp.src_off[i]);
-        });
+#pragma unroll 4
+        for (int i = pop0; i < Q; i += pstep, dst += uint32_t(pstep) * ROWB) bulk::cp_async16(dst, base + s_off[i]);
       } else {
-        const uint8_t* b0 = reinterpret_cast<const uint8_t*>(fin) + size_t(lane * 8) * sizeof(ST);
-        for (int i = warp; i < Q; i += WARPS) {
-          int ys = y - rp.ey[i];
+        const uint8_t* b0 = reinterpret_cast<const uint8_t*>(fin) + size_t(cx) * sizeof(ST);
+        for (int i = pop0; i < Q; i += pstep, dst += uint32_t(pstep) * ROWB) {
+          int ys = y - s_e[i].x;
           ys += ys < 0 ? ny : 0;
           ys -= ys >= ny ? ny : 0;
           int zs = 0;
           if constexpr (L::D == 3) {
-            zs = z - rp.ez[i];
+            zs = z - s_e[i].y;
             zs += zs < 0 ? nz : 0;
             zs -= zs >= nz ? nz : 0;
           }
-          bulk::cp_async16(dst + uint32_t(i) * ROWB,
-                           b0 + size_t(i) * pop_bytes + (size_t(zs) * ny + ys) * nx * sizeof(ST));
+          bulk::cp_async16(dst, b0 + (size_t(i) * N + (size_t(zs) * ny + ys) * nx) * sizeof(ST));
         }
       }
     }
     bulk::cp_async_arrive(&full[s]);
   };
 
-  int ly = int(blockIdx.x) % ny, lz = int(blockIdx.x) / ny;  // next row to load
-  int y = ly, z = lz;                                          // row being collided
-  // one warp-wide 16-byte store per population row of buffer sb to row (sy, sz) of the output
-  auto store_row = [&](int sy, int sz, int sb) {
-    if (lane_chunk) {
-      const size_t sr = size_t(sz) * ny + sy;
-      const uint8_t* src = reinterpret_cast<const uint8_t*>(rows + size_t(sb) * stage_elems) + warp * ROWB + lane * 16;
-      uint8_t* dst = reinterpret_cast<uint8_t*>(fout) + (sr * nx + lane * 8) * sizeof(ST) + warp * pop_bytes;
-      static_for<(Q + WARPS - 1) / WARPS>([&](auto m) {
-        constexpr int M = decltype(m)::value;
-        if (warp + WARPS * M < Q)
-          *reinterpret_cast<uint4*>(dst + M * WARPS * pop_bytes) = *reinterpret_cast<const uint4*>(src + M * WARPS * ROWB);
-      });
-    }
-  };
-
-  // Ring of NS buffers: while row k is collided (in its buffer), row k - 1 is stored from its
-  // buffer and rows k + 1 .. k + NS - 2 are in flight; one CTA barrier per row separates the reads
-  // of row k from the in-place writes, and the writes of row k - 1 from its store.
-  for (int j = 0; j < K && j < NS - 2; ++j) {
-    load_row(ly, lz, j);
-    advance(ly, lz);
-  }
-  bool failed = false;
-  int py = y, pz = z;  // row k - 1
-  for (int k = 0; k < K; ++k) {
-    const int s = k % NS;
-    const bool landed = tc::mbar_wait_bounded(&full[s], uint32_t(k / NS) & 1u, rp.wait_limit);
-    const int r = z * ny + y;
-    const uint32_t st_s = rows_s + uint32_t(s) * rp.stage_bytes;
-    float f[Q];
-    if (live && landed) {
-      uint32_t xa[2 * RM + 1];  // address of (x - sh) mod n_x in row 0 of the buffer, sh = -RM..RM
+  // this thread's cells: elements 2 tid, 2 tid + 1 of the tile, (x, j) with x even; byte offsets of
+  // (x + m) mod n_x of its row, m = -RM .. RM + 1
+  const int j = (2 * tid) / nx, x = 2 * tid - j * nx;
+  uint32_t xo[2 * RM + 2];
 #pragma unroll
-      for (int sh = -RM; sh <= RM; ++sh) {
-        int v = x - sh;
-        if (sh > 0) v += v < 0 ? nx : 0;
-        if (sh < 0) v -= v >= nx ? nx : 0;
-        xa[sh + RM] = st_s + uint32_t(v) * uint32_t(sizeof(ST));
-      }
+  for (int m = -RM; m <= RM + 1; ++m) {
+    int v = x + m;
+    v += v < 0 ? nx : 0;
+    v -= v >= nx ? nx : 0;
+    xo[m + RM] = uint32_t(j * nx + v) * uint32_t(sizeof(ST));
+  }
+
+  for (int k = 0; k < K && k < NS; ++k) load_tile(int(blockIdx.x) + k * G, k);
+  bool failed = false;
+  int s = 0;
+  uint32_t phase = 0;
+  for (int k = 0; k < K; ++k) {
+    const int t = int(blockIdx.x) + k * G;
+    const int r = t * RPT + j;
+    const bool live = j < RPT && r < rp.nrows;
+    const bool landed = tc::mbar_wait_bounded(&full[s], phase, rp.wait_limit);
+    const uint32_t st_s = rows_s + uint32_t(s) * rp.stage_bytes;
+    uint32_t raw[Q];
+    F2 mu[L::R];
+    if (live && landed) {
       static_for<Q>([&](auto i) {
-        constexpr int I = decltype(i)::value;
-        f[I] = dec16<ST>(lds16<I * int(ROWB)>(xa[RM + L::e(I).x]));
+        constexpr int I = decltype(i)::value, EX = L::e(I).x, B = I * int(ROWB);
+        if constexpr (EX % 2 == 0) raw[I] = lds32<B>(st_s + xo[RM - EX]);
+        else raw[I] = uint32_t(lds16<B>(st_s + xo[RM - EX])) | (uint32_t(lds16<B>(st_s + xo[RM + 1 - EX])) << 16);
       });
+      if constexpr (COLLIDE) {
+        F2 f[Q];
+        static_for<Q>([&](auto i) { f[decltype(i)::value] = dec16x2<ST>(raw[decltype(i)::value]); });
+        raw_moments<L>(f, mu);
+      }
     }
-    // every source of row k read, row k - 1 collided into its buffer, row k - 2 stored
+    // every source of the tile is read: the buffer takes the tile NS ahead
     if (__syncthreads_or(!landed)) {
       failed = true;
       break;
     }
-    if (k >= 1) store_row(py, pz, (k - 1) % NS);
-    if (k + NS - 2 < K) {  // into the buffer of row k - 2
-      load_row(ly, lz, (k + NS - 2) % NS);
-      advance(ly, lz);
+    if (k + NS < K) load_tile(t + NS * G, s);
+    if (++s == NS) {
+      s = 0;
+      phase ^= 1u;
     }
     if (live) {
+      const int cell = r * nx + x;
+      ST* out = fout + cell;
       if constexpr (COLLIDE) {
-        const int cell = r * nx + x;
-        float F[3];
-        const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, x, y, z, F);
-        float phi_prev = 0.f, phi_now = 0.f;
-        if constexpr (EQ == LBM_NCDE) phi_prev = phi[cell];
-        constexpr bool AG = GradTerm<L, EQ>::kOn;
-        float gr[3];
-        const float* grad = nullptr;
-        if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
-        collide<L, float, EQ, true, KEEP>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
-        if constexpr (EQ == LBM_NCDE) phi[cell] = phi_now;
-        if constexpr (AG && EQ == LBM_NSE) {
-          if (p.grad_on) p.rho_out[cell] = phi_now;
+        int y = r, z = 0;
+        if constexpr (L::D == 3) {
+          z = int(__umulhi(unsigned(r), p.div_m[1]) >> p.div_s[1]);
+          y = r - z * ny;
         }
+        F2 F[3];
+        const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, x, y, z, F);
+        F2 phi_prev(0.f), phi_now(0.f);
+        if constexpr (EQ == LBM_NCDE) phi_prev = *reinterpret_cast<const F2*>(phi + cell);
+        constexpr bool AG = GradTerm<L, EQ>::kOn;
+        F2 gr[3];
+        const F2* grad = nullptr;
+        if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
+        F2 h[L::R];
+        collide_moments<L, F2, EQ, true>(mu, p, p, forced, F, phi_prev, phi_now, h, grad);
+        if constexpr (EQ == LBM_NCDE) *reinterpret_cast<F2*>(phi + cell) = phi_now;
+        if constexpr (AG && EQ == LBM_NSE) {
+          if (p.grad_on) *reinterpret_cast<F2*>(p.rho_out + cell) = phi_now;
+        }
+        F2 f[Q];
+        if constexpr (KEEP) {
+          static_for<Q>([&](auto i) {
+            constexpr int I = decltype(i)::value;
+            asm volatile("" : "+r"(raw[I]));  // decoded again, not kept decoded since the moments
+            f[I] = dec16x2<ST>(raw[I]);
+          });
+        }
+        back_project<L, KEEP>(f, p, h, p.one_minus_sh);
+        static_for<Q>([&](auto i) {
+          constexpr int I = decltype(i)::value;
+          float a, b;
+          f[I].get(a, b);
+          *reinterpret_cast<uint32_t*>(out + size_t(I) * N) = pack16x2<ST>(a, b);
+        });
+      } else {
+        static_for<Q>([&](auto i) {
+          constexpr int I = decltype(i)::value;
+          *reinterpret_cast<uint32_t*>(out + size_t(I) * N) = raw[I];
+        });
       }
-      const uint32_t xs = st_s + uint32_t(x) * uint32_t(sizeof(ST));
-      static_for<Q>([&](auto i) {
-        constexpr int I = decltype(i)::value;
-        sts16<I * int(ROWB)>(xs, enc16<ST>(f[I]));
-      });
     }
-    py = y;
-    pz = z;
-    advance(y, z);
-  }
-  if (!failed && K > 0) {
-    __syncthreads();  // the last row is complete in its buffer
-    store_row(py, pz, (K - 1) % NS);
   }
   if (failed && tid == 0) atomicExch(rp.status, 1);
   bulk::cp_async_wait_all();  // no copy of this thread is still writing the CTA's shared memory
 }
 
-// The same row-staged step with the two contractions of the collision on the tensor cores. A CTA
-// is two tiles of 128 cells (warps 0-3: cells 0..127 of the row, warps 4-7: 128..255), each with
+// The row-staged step with the two contractions of the collision on the tensor cores, one row per
+// buffer and one cell per thread; the threads write their post-collision populations back into the
+// buffer at their own x after a CTA barrier (every source read), and after the next row's barrier the
+// warps store the Q rows with 16-byte stores. A CTA is two tiles of 128 cells (warps 0-3: cells 0..127 of the row, warps 4-7: 128..255), each with
 // its own 128 TMEM columns. Per row and tile:
 //   forward  mu (128 x RP) = D (128 x QP) . M^T, D the stored 16-bit deviations, written by each
 //            thread into its own TMEM lane (A from tensor memory), M_ki = mono_k(e_i) in shared
@@ -570,9 +600,12 @@ __global__ void __launch_bounds__(kRowThreads, 2)
   if (warp == 0) tc::dealloc(*tslot, 2 * TILE_COLS);
 }
 
-// Launch plan: the kernel applies to 16-bit storage with n_x a multiple of 8 (16-byte rows) and
-// at most the row pitch (256 cells). Two CTAs per SM when three row buffers each fit, otherwise
-// one; as many buffers (up to kRowMaxStages) as the shared memory of a CTA holds.
+// Launch plan: the kernels apply to 16-bit storage with n_x a multiple of 8 (16-byte rows) and
+// at most the row pitch (256 cells). The CUDA-core kernel: as many rows per tile as the pitch holds,
+// fewer where that would leave SMs without a tile, row_ctas CTAs per SM and as many buffers (2 to
+// kRowMaxStages) as their shared memory holds. The tensor-core kernel: two CTAs per SM when three row
+// buffers each fit (the row being collided, the row being stored, at least one in flight),
+// otherwise one.
 template <int KIND>
 bool RowLaunch<KIND>::plan(const lbm_model* m, RowPlan* out, bool tensor, bool high) {
   using L = Lat<KIND>;
@@ -594,12 +627,14 @@ bool RowLaunch<KIND>::plan(const lbm_model* m, RowPlan* out, bool tensor, bool h
     return size_t(Sh::N1) * Sh::QP * 2 + size_t(Sh::QP) * Sh::K2 * 2;
   };
   const size_t tables = !tensor ? 0 : high ? table_bytes(TcShape<L, true>{}) : table_bytes(TcShape<L, false>{});
+  const size_t head = (tensor ? kRowBarBytes : kRowHeadBytes) + tables;
+  const int want = tensor ? 2 : m->s_high == 1.0 ? row_ctas<false>() : row_ctas<true>(), least = tensor ? 3 : 2;
   RowPlan p{};
   int ctas = 0, stages = 0;
-  for (int c = 2; c >= 1 && ctas == 0; --c) {
+  for (int c = want; c >= 1 && ctas == 0; --c) {
     const size_t avail = std::min<size_t>(size_t(per_block), size_t(per_sm) / c - 1024);  // 1 KB reserved per CTA
-    const int ns = int(std::min<size_t>(kRowMaxStages, (avail - kRowBarBytes - tables) / stage_bytes));
-    if (ns >= 3) {  // the row being collided, the row being stored, at least one in flight
+    const int ns = avail < head ? 0 : int(std::min<size_t>(kRowMaxStages, (avail - head) / stage_bytes));
+    if (ns >= least) {
       ctas = c;
       stages = ns;
     }
@@ -607,6 +642,13 @@ bool RowLaunch<KIND>::plan(const lbm_model* m, RowPlan* out, bool tensor, bool h
   if (ctas == 0) return false;
   const int64_t nrows = m->n[1] * m->n[2];
   p.rp.nrows = int(nrows);
+  int rpt = int(std::min<int64_t>(kRowPitch / nx, nrows));
+  while (rpt > 1 && (nrows + rpt - 1) / rpt < sms) --rpt;
+  p.rp.rpt = rpt;
+  p.rp.ntiles = int((nrows + rpt - 1) / rpt);
+  p.rp.chunks = int(nx / 8);
+  p.rp.lanes = 1;
+  while (p.rp.lanes < rpt * p.rp.chunks) p.rp.lanes *= 2;
   p.rp.stages = stages;
   p.rp.stage_bytes = uint32_t(stage_bytes);
   p.rp.status = m->status;
@@ -618,8 +660,8 @@ bool RowLaunch<KIND>::plan(const lbm_model* m, RowPlan* out, bool tensor, bool h
     p.rp.ez[i] = int8_t(L::e(i).z);
     p.rp.src_off[i] = 2 * (int64_t(i) * N - (int64_t(L::e(i).y) + int64_t(L::e(i).z) * m->n[1]) * nx);
   }
-  p.grid = int(std::min<int64_t>(nrows, int64_t(sms) * ctas));
-  p.smem = kRowBarBytes + tables + size_t(stages) * stage_bytes;
+  p.grid = int(std::min<int64_t>(tensor ? nrows : p.rp.ntiles, int64_t(sms) * ctas));
+  p.smem = head + size_t(stages) * stage_bytes;
   p.tensor = tensor;
   p.high = high;
   if (tensor) make_tc_params(m, &p.tp);
@@ -628,20 +670,15 @@ bool RowLaunch<KIND>::plan(const lbm_model* m, RowPlan* out, bool tensor, bool h
 }
 
 // The kernel of a model: storage type, equation, collision on / off (stream only), s_high = 1 or not.
-template <class L, class ST, bool FULL, class F>
-lbm_status row_kernel_full(const lbm_model* m, bool collide, F&& fn) {
-  if (!collide) return fn(k_step_rows<L, ST, LBM_NSE, false, FULL, true>);
-  if (m->eq == LBM_NSE) {
-    if (m->s_high == 1.0) return fn(k_step_rows<L, ST, LBM_NSE, true, FULL, false>);
-    return fn(k_step_rows<L, ST, LBM_NSE, true, FULL, true>);
-  }
-  if (m->s_high == 1.0) return fn(k_step_rows<L, ST, LBM_NCDE, true, FULL, false>);
-  return fn(k_step_rows<L, ST, LBM_NCDE, true, FULL, true>);
-}
 template <class L, class ST, class F>
 lbm_status row_kernel(const lbm_model* m, bool collide, F&& fn) {
-  if (m->n[0] == kRowPitch) return row_kernel_full<L, ST, true>(m, collide, fn);
-  return row_kernel_full<L, ST, false>(m, collide, fn);
+  if (!collide) return fn(k_step_rows<L, ST, LBM_NSE, false, true>);
+  if (m->eq == LBM_NSE) {
+    if (m->s_high == 1.0) return fn(k_step_rows<L, ST, LBM_NSE, true, false>);
+    return fn(k_step_rows<L, ST, LBM_NSE, true, true>);
+  }
+  if (m->s_high == 1.0) return fn(k_step_rows<L, ST, LBM_NCDE, true, false>);
+  return fn(k_step_rows<L, ST, LBM_NCDE, true, true>);
 }
 
 // The tensor-core kernel of a model: fn(kernel, storage tag).
@@ -678,11 +715,12 @@ lbm_status RowLaunch<KIND>::configure(const lbm_model* m, const RowPlan& plan, b
 
 template <int KIND>
 lbm_status RowLaunch<KIND>::launch(const lbm_model* m, const RowPlan& plan, const StepParams<float>& p,
-                                   const void* fin, void* fout, float* phi, bool collide) {
+                                   const StepParams<F2, float>& p2, const void* fin, void* fout, float* phi,
+                                   bool collide) {
   using L = Lat<KIND>;
   auto go = [&](auto kernel, auto tag) -> lbm_status {
     using ST = decltype(tag);
-    cudaError_t err = launch_chained(kernel, plan.grid, kRowThreads, plan.smem, m->stream, p, plan.rp,
+    cudaError_t err = launch_chained(kernel, plan.grid, kRowPairs, plan.smem, m->stream, p2, plan.rp,
                                      static_cast<const ST*>(fin), static_cast<ST*>(fout), phi);
     return err == cudaSuccess ? LBM_OK : cuda_error(err, "row-staged collide-stream launch");
   };

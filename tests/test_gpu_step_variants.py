@@ -1,0 +1,66 @@
+"""The variants of the collide-stream step that a call is given by its grid, storage and rates: each one
+gives bitwise the populations of the one-cell-per-thread kernels, at the sizes where its tiling ends."""
+import numpy as np
+import pytest
+
+from paper_2512_16230_gb300 import workloads as W
+
+from _harness import gpu_model, oracle_lattice
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _lib(lbm_lib):
+    return lbm_lib
+
+
+def _populations(spec, n, seed, eq):
+    w = oracle_lattice(spec).w
+    r = np.random.default_rng(seed).uniform(-0.1, 0.1, size=(len(w),) + tuple(reversed(n)))
+    return w.reshape((-1,) + (1,) * len(n)) * (1.0 if eq == "nse" else 0.7) * (1.0 + r)
+
+
+def _kwargs(eq, d, s_high):
+    if eq == "nse":
+        return dict(s_high=s_high, cs2_eq=0.55, force=(0, d - 1, 3e-3, 1, 0.4))
+    return dict(s_high=s_high, cs2_eq=0.55, u_const=tuple(np.linspace(0.03, 0.06, d)), nonlin=1.0)
+
+
+def _rates(spec):
+    return np.random.default_rng(3).uniform(0.6, 1.9, spec.R)
+
+
+# row-staged kernel: tiles of several rows that wrap in y and z within the tile, a last tile with fewer
+# rows, one row of 8 cells per thread group
+@pytest.mark.parametrize("s_high", [1.0, 1.3])
+@pytest.mark.parametrize("eq", ["nse", "ncde"])
+@pytest.mark.parametrize("name,n", [("rD2Q17", (8, 5000)), ("rD3Q33", (24, 47, 53)), ("rD3Q53", (40, 31, 37))])
+def test_row_tiles_of_several_rows(name, n, eq, s_high):
+    spec = W.LATTICES[name]
+    f0 = _populations(spec, n, 5, eq)
+    out = {}
+    for mode in ("rows", "threads"):
+        gm = gpu_model(spec, eq, n, _rates(spec), store="f16_dev", **_kwargs(eq, spec.d, s_high))
+        gm.set_gather(mode)
+        gm.set_populations(f0)
+        gm.step(3)
+        out[mode] = gm.get_populations()
+        gm.close()
+    assert np.array_equal(out["rows"], out["threads"])
+
+
+def test_row_tiles_with_per_cell_rates_and_cross_diffusion():
+    spec, n = W.LATTICES["rD2Q25"], (8, 5000)
+    f0 = _populations(spec, n, 6, "ncde")
+    psi = np.random.default_rng(7).uniform(-1, 1, size=(n[1], n[0]))
+    out = {}
+    for mode in ("rows", "threads"):
+        gm = gpu_model(spec, "ncde", n, _rates(spec), store="bf16_dev", ncde_mode="rate", a1=-0.2, a2=0.02, psi=psi,
+                       **_kwargs("ncde", 2, 1.0))
+        gm.set_gather(mode)
+        gm.set_populations(f0)
+        gm.step(3)
+        out[mode] = gm.get_populations()
+        gm.close()
+    assert np.array_equal(out["rows"], out["threads"])
