@@ -250,25 +250,6 @@ inline void division_magic(unsigned d, unsigned* m, int* shift) {
   *shift = s - 1;
 }
 
-// Parameters of the generic (lattice-agnostic, non-hot) kernels.
-struct GenParams {
-  int Q, d, n[3], ncells;
-  int8_t e[kMaxQ][3];
-  double c[3];
-  double wref[kMaxQ];
-  double cde_half[3];  // NCDE CDE variant: phi = sum f + sum_a cde_half_a sum_i c_ia f_i
-  int force_a, force_b;
-  const void* force_tab;
-};
-
-// Per-velocity tables of the generic kernels in their compute dtype (c_ia and w_i rho_ref), so
-// that no FP64 arithmetic runs per population when the model computes in FP32.
-template <class CT>
-struct GenTables {
-  CT ce[kMaxQ][3];
-  CT wref[kMaxQ];
-};
-
 // Storage codecs: FP64/FP32 store f itself; BF16/FP16 store the deviation f - w_i rho_ref.
 template <class ST>
 struct Codec;
@@ -401,15 +382,24 @@ struct BatchLaunch {
   static lbm_status occupancy(const BatchGroup& g, int* blocks_per_sm);
 };
 
+// One launch of the kernels around the step (io_kernels.cuh).
+struct IoCall {
+  enum What { kGather, kScatter, kFields, kPhi, kSums } what;
+  const char* name;
+  const double* in;
+  double *out, *out2;  // kFields: rho (phi) and u; kSums: the sums and the block partials
+  void* field;         // kPhi: a cell field in the compute dtype
+};
+
 // Per-lattice launchers, defined in the k_<lattice>.cu translation units.
 template <int KIND>
 struct Launch {
+  static lbm_status io(lbm_model* m, const IoCall& io);
   static lbm_status step(lbm_model* m, int64_t nsteps, bool collide);
   static lbm_status init(lbm_model* m, const double* rho_or_phi, const double* u);
 };
 
-// Generic kernels (aux_kernels.cu).
-lbm_status gen_params(const lbm_model* m, GenParams* gp);
+// The kernels around the step (aux_kernels.cu).
 lbm_status launch_gather(lbm_model* m, double* out);          // f-bar(x) from the stored array
 lbm_status launch_scatter(lbm_model* m, const double* in);    // stored array from f-bar(x)
 lbm_status launch_fields(lbm_model* m, double* rho, double* u);

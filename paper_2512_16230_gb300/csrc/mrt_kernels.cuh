@@ -1055,6 +1055,7 @@ __global__ void __launch_bounds__(kBlock, 3)
 
 }  // namespace lbm
 
+#include "io_kernels.cuh"
 #include "tc_kernels.cuh"
 
 namespace lbm {

@@ -64,3 +64,19 @@ def test_row_tiles_with_per_cell_rates_and_cross_diffusion():
         out[mode] = gm.get_populations()
         gm.close()
     assert np.array_equal(out["rows"], out["threads"])
+
+
+def test_population_io_keeps_every_value():
+    """set_populations followed by get_populations returns FP32 values unchanged, also those for which the
+    widening takes the conversion instruction: zeros of both signs, subnormals, infinities and NaN."""
+    spec = W.LATTICES["rD2Q9"]
+    n = (37, 5)
+    v = np.array([0.0, -0.0, 1e-45, -1e-40, 1.1754944e-38, 3.4028235e38, -1.0, 1.0 + 2.0 ** -23, np.inf, -np.inf, np.nan,
+                  0.1], dtype=np.float32)
+    f0 = np.resize(v, 9 * n[0] * n[1]).reshape(9, n[1], n[0]).astype(np.float64)
+    gm = gpu_model(spec, "nse", n, np.ones(spec.R), store="f32")
+    gm.set_populations(f0)
+    g = gm.get_populations()
+    gm.close()
+    assert np.array_equal(g, f0, equal_nan=True)
+    assert np.array_equal(np.signbit(g[f0 == 0]), np.signbit(f0[f0 == 0]))
