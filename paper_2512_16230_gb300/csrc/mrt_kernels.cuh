@@ -784,12 +784,12 @@ __device__ __forceinline__ bool body_force(int force_a, int force_b, const CT* f
   return true;
 }
 
-// The same for two cells side by side.
+// The same for two cells.
 __device__ __forceinline__ bool body_force(int force_a, int force_b, const float* force_tab, const F2 (&invc)[3],
-                                           int x, int y, int z, F2 (&F)[3]) {
+                                           const int (&c0)[3], const int (&c1)[3], F2 (&F)[3]) {
   if (force_b < 0) return false;
-  const int ib = force_b == 0 ? x : (force_b == 1 ? y : z);
-  const F2 v(force_tab[ib], force_tab[force_b == 0 ? ib + 1 : ib]);
+  const F2 v(force_tab[force_b == 0 ? c0[0] : (force_b == 1 ? c0[1] : c0[2])],
+             force_tab[force_b == 0 ? c1[0] : (force_b == 1 ? c1[1] : c1[2])]);
   F[0] = force_a == 0 ? v * invc[0] : F2(0.f);
   F[1] = force_a == 1 ? v * invc[1] : F2(0.f);
   F[2] = force_a == 2 ? v * invc[2] : F2(0.f);
@@ -826,14 +826,15 @@ __device__ __forceinline__ const CT* cell_field_gradient(const Rates<CT>& p, con
   static_for<L::D>([&](auto a) { gr[decltype(a)::value] = p.gscale[decltype(a)::value] * gr[decltype(a)::value]; });
   return gr;
 }
-// The same for two cells side by side, (x, y, z) and (x + 1, y, z).
+// The same for two cells, the second one following the first in memory.
 template <class L>
 __device__ __forceinline__ const F2* cell_field_gradient(const Rates<F2>& p, const int (&n)[3], const float* g,
-                                                         int cell, int x, int y, int z, F2 (&gr)[3]) {
+                                                         int cell, const int (&c0)[3], const int (&c1)[3],
+                                                         F2 (&gr)[3]) {
   if (!p.grad_on) return nullptr;
   float d0[3], d1[3];
-  field_differences<L>(n, g, cell, x, y, z, d0);
-  field_differences<L>(n, g, cell + 1, x + 1, y, z, d1);
+  field_differences<L>(n, g, cell, c0[0], c0[1], c0[2], d0);
+  field_differences<L>(n, g, cell + 1, c1[0], c1[1], c1[2], d1);
   static_for<L::D>([&](auto a) {
     constexpr int A = decltype(a)::value;
     gr[A] = p.gscale[A] * F2(d0[A], d1[A]);
@@ -877,6 +878,140 @@ __global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepPa
     constexpr int I = decltype(i)::value;
     if constexpr (DEV) k1_store(fout + size_t(I) * N + cell, RawCodec<ST>::enc(f[I]));
     else k1_store(fout + size_t(I) * N + cell, Codec<ST>::enc(f[I], p.wref[I]));
+  });
+}
+
+// Two 16-bit values in one word, decoded.
+template <class ST>
+__device__ __forceinline__ F2 dec_word(uint32_t b) {
+  if constexpr (std::is_same<ST, __half>::value) {
+    const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&b));
+    return F2(v.x, v.y);
+  } else {
+    return F2(__uint_as_float(b << 16), __uint_as_float(b & 0xFFFF0000u));
+  }
+}
+template <class ST>
+__device__ __forceinline__ uint32_t enc_word(float a, float b) {
+  uint32_t r;
+  if constexpr (std::is_same<ST, __half>::value) {
+    const __half2 h = __floats2half2_rn(a, b);
+    r = *reinterpret_cast<const uint32_t*>(&h);
+  } else {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    r = *reinterpret_cast<const uint32_t*>(&h);
+  }
+  return r;
+}
+
+// K1 on two neighbouring cells per thread in packed FP32 arithmetic (f32x2.cuh), for FP32 and 16-bit
+// storage: bitwise the populations of k_step. EVEN: n_x is even, the cells are (x, x + 1) of one row
+// with x even; an even e_x is one load of both sources, the stores are pairs. Otherwise the cells are
+// 2 t and 2 t + 1 of the array and every access is by cell (the last cell of an odd grid is done alone).
+//
+// What bounds it: HBM on large FP32 grids, instruction issue elsewhere; packing halves the FP32 arithmetic. us a
+// step on GB300, one cell / two cells per thread: rD2Q13 1024x768 FP32 11.5 / 8.8, rD3Q33 64^3 FP32
+// 10.2 / 8.4, rD3Q53 256x256x192 FP32 776 / 759, rD3Q53 150x131x147 BF16 153 / 116, rD3Q45 101x103x97
+// FP32 62.8 / 59.2. 4 blocks per SM leave 128 registers; on rD3Q53 the single accesses spill at that, with 3
+// blocks 81^3 FP32 takes 39.0 us (one cell per thread 40.0) and 149x131x147 BF16 139 us (156).
+template <class L, class ST, int EQ, bool KEEP, bool EVEN>
+__global__ void __launch_bounds__(kBlock, KEEP && L::Q > 33 ? 2 : (L::Q > 45 && (!EVEN || is_deviation_storage<ST>()) ? 3 : 4))
+    k_step_pair(const StepParams<F2, float> p, const ST* fin, ST* fout, float* phi) {
+  constexpr int Q = L::Q, RM = L::RMAX;
+  constexpr bool DEV = is_deviation_storage<ST>();
+  chain_release();
+  const int cell = 2 * (blockIdx.x * kBlock + threadIdx.x);
+  if (cell >= p.ncells) return;
+  const size_t N = size_t(p.ncells);
+  const bool two = EVEN || cell + 1 < p.ncells;
+  const Neigh<L> n0(cell, p.n, p.div_m, p.div_s);
+  F2 f[Q];
+  auto one = [&](const ST* a) -> float {
+    if constexpr (DEV) return RawCodec<ST>::dec(k1_load(a));
+    else return k1_load(a);
+  };
+  int c0[3] = {n0.x, n0.y, n0.z}, c1[3] = {n0.x + 1, n0.y, n0.z};
+  if constexpr (EVEN) {
+    // x positions of the second cell's sources; the first cell's for e_x = -RM .. RM are n0.xo
+    int x1[2 * RM + 1];
+#pragma unroll
+    for (int sh = -RM; sh <= RM; ++sh) x1[sh + RM] = Neigh<L>::wrap1(n0.x + 1 - sh, sh == 0 ? 1 : sh, p.n[0]);
+    chain_wait();
+    static_for<Q>([&](auto i) {
+      constexpr int I = decltype(i)::value;
+      constexpr Vel v = L::e(I);
+      const int yz = n0.yo[RM + v.y] + (L::D == 3 ? n0.zo[RM + v.z] : 0);
+      const ST* a = fin + size_t(I) * N + (n0.xo[RM + v.x] + yz);
+      if constexpr (v.x % 2 == 0) {
+        if constexpr (DEV) f[I] = dec_word<ST>(*reinterpret_cast<const uint32_t*>(a));
+        else f[I] = *reinterpret_cast<const F2*>(a);
+      } else {
+        f[I] = F2(one(a), one(fin + size_t(I) * N + (x1[RM + v.x] + yz)));
+      }
+    });
+  } else {
+    const Neigh<L> n1(two ? cell + 1 : cell, p.n, p.div_m, p.div_s);
+    c1[0] = n1.x;
+    c1[1] = n1.y;
+    c1[2] = n1.z;
+    chain_wait();
+    static_for<Q>([&](auto i) {
+      constexpr int I = decltype(i)::value;
+      f[I] = F2(one(fin + size_t(I) * N + n0.template src<I>()), one(fin + size_t(I) * N + n1.template src<I>()));
+    });
+  }
+  F2 F[3];
+  const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, c0, c1, F);
+  F2 phi_prev(0.f), phi_now(0.f);
+  if constexpr (EQ == LBM_NCDE) {
+    if constexpr (EVEN) phi_prev = *reinterpret_cast<const F2*>(phi + cell);
+    else phi_prev = F2(phi[cell], phi[two ? cell + 1 : cell]);
+  }
+  constexpr bool AG = GradTerm<L, EQ>::kOn;
+  F2 gr[3];
+  const F2* grad = nullptr;
+  if constexpr (AG) {
+    if (two) {
+      grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, c0, c1, gr);
+    } else if (p.grad_on) {
+      float d[3];
+      field_differences<L>(p.n, p.grad_in, cell, c0[0], c0[1], c0[2], d);
+      static_for<L::D>([&](auto a) { gr[decltype(a)::value] = p.gscale[decltype(a)::value] * F2(d[decltype(a)::value]); });
+      grad = gr;
+    }
+  }
+  collide<L, F2, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
+  float a, b;
+  auto field_out = [&](float* g) {
+    if constexpr (EVEN) {
+      *reinterpret_cast<F2*>(g + cell) = phi_now;
+    } else {
+      phi_now.get(a, b);
+      g[cell] = a;
+      if (two) g[cell + 1] = b;
+    }
+  };
+  if constexpr (EQ == LBM_NCDE) field_out(phi);
+  if constexpr (AG && EQ == LBM_NSE) {
+    if (p.grad_on) field_out(p.rho_out);
+  }
+  static_for<Q>([&](auto i) {
+    constexpr int I = decltype(i)::value;
+    ST* o = fout + size_t(I) * N + cell;
+    if constexpr (EVEN && !DEV) {
+      *reinterpret_cast<F2*>(o) = f[I];
+    } else {
+      f[I].get(a, b);
+      if constexpr (EVEN) {
+        *reinterpret_cast<uint32_t*>(o) = enc_word<ST>(a, b);
+      } else if constexpr (DEV) {
+        k1_store(o, RawCodec<ST>::enc(a));
+        if (two) k1_store(o + 1, RawCodec<ST>::enc(b));
+      } else {
+        k1_store(o, a);
+        if (two) k1_store(o + 1, b);
+      }
+    }
   });
 }
 
@@ -1143,6 +1278,11 @@ lbm_status BatchLaunch<KIND>::occupancy(const BatchGroup& g, int* blocks_per_sm)
   });
 }
 
+// Cells from which a step takes two of them per thread. Below, the halved number of threads leaves SMs
+// short of warps (us a step, one cell / two cells per thread: rD2Q21 256x200 2.44 / 2.61, 333x301 4.16 /
+// 3.77; rD3Q45 36^3 5.6 / 6.3, 45^3 6.6 / 5.9, 64^3 14.0 / 11.4).
+constexpr int kPairCells = 80000;
+
 // Host launchers for one lattice kind (instantiated in k_<lattice>.cu).
 template <class L, class CT, class ST>
 lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
@@ -1211,9 +1351,14 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       }
     }
   }
+  // two cells per thread where the halved thread count still fills the GPU
+  [[maybe_unused]] const bool pairs = !std::is_same<CT, double>::value && collide_on && !high && !tensor && !rows &&
+                                      m->ncells >= kPairCells;
+  if (pairs) make_step_params(m, &p2);
+  const int grid2 = (m->ncells / 2 + m->ncells % 2 + kBlock - 1) / kBlock;
   const bool hist = collide_on && m->m2g_aniso;
   p.grad_on = collide_on && p.grad_on;
-  if (rows) p2.grad_on = p.grad_on;
+  if (rows || pairs) p2.grad_on = p.grad_on;
   for (int64_t s = 0; s < nsteps; ++s) {
     const ST* fin = static_cast<const ST*>(m->f[m->cur]);
     ST* fout = static_cast<ST*>(m->f[m->cur ^ 1]);
@@ -1250,6 +1395,23 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       if (tensor32) {
         if (m->eq == LBM_NSE) go(k_step_tc32_high<L, LBM_NSE>, tgrid, 128, tsmem, p, tp32);
         else go(k_step_tc32_high<L, LBM_NCDE>, tgrid, 128, tsmem, p, tp32);
+        done = true;
+      }
+    }
+    if constexpr (!std::is_same<CT, double>::value) {
+      if (pairs) {
+        auto pick = [&](auto eq, auto keep) {
+          constexpr int E = decltype(eq)::value;
+          constexpr bool K = decltype(keep)::value;
+          if (m->n[0] % 2 == 0) go(k_step_pair<L, ST, E, K, true>, grid2, kBlock, 0, p2);
+          else go(k_step_pair<L, ST, E, K, false>, grid2, kBlock, 0, p2);
+        };
+        auto by_keep = [&](auto eq) {
+          if (m->s_high == 1.0) pick(eq, std::false_type{});
+          else pick(eq, std::true_type{});
+        };
+        if (m->eq == LBM_NSE) by_keep(std::integral_constant<int, LBM_NSE>{});
+        else by_keep(std::integral_constant<int, LBM_NCDE>{});
         done = true;
       }
     }

@@ -47,17 +47,13 @@ __device__ __forceinline__ uint16_t enc16(float v) {
   return b;
 }
 
-// Two neighbouring values of a row, decoded into a packed pair; the 32-bit word at a register address
-// plus a compile-time byte offset.
+// The 32-bit word (two neighbouring values of a row) at a register address plus a compile-time byte
+// offset.
 template <int OFF>
 __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
   uint32_t v;
   asm volatile("ld.shared.b32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(OFF));
   return v;
-}
-template <class ST>
-__device__ __forceinline__ F2 dec16x2(uint32_t b) {
-  return F2(dec16<ST>(uint16_t(b & 0xFFFFu)), dec16<ST>(uint16_t(b >> 16)));
 }
 
 // Resident CTAs per SM (128 threads each). 4 leave 128 registers and, on the largest lattice, two
@@ -179,7 +175,7 @@ __global__ void __launch_bounds__(kRowPairs, row_ctas<KEEP && COLLIDE>())
       });
       if constexpr (COLLIDE) {
         F2 f[Q];
-        static_for<Q>([&](auto i) { f[decltype(i)::value] = dec16x2<ST>(raw[decltype(i)::value]); });
+        static_for<Q>([&](auto i) { f[decltype(i)::value] = dec_word<ST>(raw[decltype(i)::value]); });
         raw_moments<L>(f, mu);
       }
     }
@@ -203,13 +199,14 @@ __global__ void __launch_bounds__(kRowPairs, row_ctas<KEEP && COLLIDE>())
           y = r - z * ny;
         }
         F2 F[3];
-        const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, x, y, z, F);
+        const int c0[3] = {x, y, z}, c1[3] = {x + 1, y, z};
+        const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, c0, c1, F);
         F2 phi_prev(0.f), phi_now(0.f);
         if constexpr (EQ == LBM_NCDE) phi_prev = *reinterpret_cast<const F2*>(phi + cell);
         constexpr bool AG = GradTerm<L, EQ>::kOn;
         F2 gr[3];
         const F2* grad = nullptr;
-        if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
+        if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, c0, c1, gr);
         F2 h[L::R];
         collide_moments<L, F2, EQ, true>(mu, p, p, forced, F, phi_prev, phi_now, h, grad);
         if constexpr (EQ == LBM_NCDE) *reinterpret_cast<F2*>(phi + cell) = phi_now;
@@ -221,7 +218,7 @@ __global__ void __launch_bounds__(kRowPairs, row_ctas<KEEP && COLLIDE>())
           static_for<Q>([&](auto i) {
             constexpr int I = decltype(i)::value;
             asm volatile("" : "+r"(raw[I]));  // decoded again, not kept decoded since the moments
-            f[I] = dec16x2<ST>(raw[I]);
+            f[I] = dec_word<ST>(raw[I]);
           });
         }
         back_project<L, KEEP>(f, p, h, p.one_minus_sh);
@@ -229,7 +226,7 @@ __global__ void __launch_bounds__(kRowPairs, row_ctas<KEEP && COLLIDE>())
           constexpr int I = decltype(i)::value;
           float a, b;
           f[I].get(a, b);
-          *reinterpret_cast<uint32_t*>(out + size_t(I) * N) = pack16x2<ST>(a, b);
+          *reinterpret_cast<uint32_t*>(out + size_t(I) * N) = enc_word<ST>(a, b);
         });
       } else {
         static_for<Q>([&](auto i) {

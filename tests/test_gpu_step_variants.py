@@ -80,3 +80,62 @@ def test_population_io_keeps_every_value():
     gm.close()
     assert np.array_equal(g, f0, equal_nan=True)
     assert np.array_equal(np.signbit(g[f0 == 0]), np.signbit(f0[f0 == 0]))
+
+
+def _batched(spec, eq, n, f0, steps, prepare=lambda m: None, **kw):
+    """The same solve in the work-list kernel of a batch, which takes one cell per thread."""
+    from paper_2512_16230_gb300 import lbm
+    m = gpu_model(spec, eq, n, _rates(spec), **kw)
+    prepare(m)
+    m.set_populations(f0)
+    b = lbm.Batch()
+    b.set_solo_threshold(0)
+    b.add(m)
+    b.step(steps)
+    out = m.get_populations()
+    b.remove(m)
+    b.close()
+    m.close()
+    return out
+
+
+# just above the size from which two cells go to a thread: n_x even, n_x odd with an odd and an even cell count
+PAIR_GRIDS = {2: [(322, 250), (287, 283), (283, 286)], 3: [(46, 43, 41), (45, 43, 43)]}
+
+
+@pytest.mark.parametrize("store", ["f32", "bf16_dev"])
+@pytest.mark.parametrize("s_high", [1.0, 1.3])
+@pytest.mark.parametrize("eq", ["nse", "ncde"])
+@pytest.mark.parametrize("name", ["rD2Q13", "rD2Q25", "rD3Q33", "rD3Q53"])
+def test_two_cells_per_thread(name, eq, s_high, store):
+    spec = W.LATTICES[name]
+    for n in PAIR_GRIDS[spec.d]:
+        f0 = _populations(spec, n, 8, eq)
+        kw = dict(store=store, **_kwargs(eq, spec.d, s_high))
+        m = gpu_model(spec, eq, n, _rates(spec), **kw)
+        m.set_populations(f0)
+        m.step(3)
+        one = m.get_populations()
+        m.close()
+        assert np.array_equal(one, _batched(spec, eq, n, f0, 3, **kw)), n
+
+
+def test_two_cells_per_thread_with_gradient_terms():
+    """The density history of M2G on rD3Q27 and the cross diffusion of the NCDE, both read at neighbours."""
+    for name, eq, n, extra in (("rD3Q27", "nse", (45, 43, 43), lambda m: m.set_m2g_anisotropy(1)),
+                               ("rD3Q27", "nse", (46, 43, 41), lambda m: m.set_m2g_anisotropy(1)),
+                               ("rD2Q21", "ncde", (287, 283), None), ("rD2Q21", "ncde", (322, 250), None)):
+        spec = W.LATTICES[name]
+        f0 = _populations(spec, n, 9, eq)
+        kw = dict(store="f32", **_kwargs(eq, spec.d, 1.0))
+        if extra is None:
+            kw.update(ncde_mode="rate", a1=-0.2, a2=0.02,
+                      psi=np.random.default_rng(7).uniform(-1, 1, size=tuple(reversed(n))))
+        prepare = extra or (lambda m: None)
+        m = gpu_model(spec, eq, n, _rates(spec), **kw)
+        prepare(m)
+        m.set_populations(f0)
+        m.step(4)
+        one = m.get_populations()
+        m.close()
+        assert np.array_equal(one, _batched(spec, eq, n, f0, 4, prepare, **kw)), (name, n)
