@@ -157,6 +157,7 @@ struct StepParams : LatTables<V>, Rates<V> {
   int div_s[2];          // by n[0] (slot 0) and n[1] (slot 1) for every v < 2^31
   int force_a, force_b;  // force_b < 0: no body force
   const FT* force_tab;
+  int release;           // where a block lets the next launch of the chain start (kRelease...)
 };
 
 // Rows of order >= 4 that relax with their own rates (the full Q x Q collision). The kernel
@@ -314,8 +315,35 @@ inline size_t dtype_bytes(int dt) { return dt == LBM_F64 ? 8 : dt == LBM_F32 ? 4
 // its writes are visible. Since every kernel waits before it writes, the order is transitive. A
 // kernel that takes tensor memory calls chain_release() only once it holds it: a later kernel's
 // block can then never hold columns that an earlier one still waits for.
-__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+//
+// Where a kernel releases the next one (StepParams::release). Blocks of the next kernel take their slots
+// as soon as they are released and wait there. With a grid of at most one wave they would find free slots
+// at once, then the kernel after that, and the blocks of a grid would end up piled on the SMs that still
+// had room: the release comes last, before the stores (rD2Q17 FP32, us a step, first / after the wait /
+// last: 200x150 3.76 / 2.29 / 1.91, 333x301 4.75 / 3.87 / 3.59; rD3Q33 32^3 4.59 / 3.27 / 2.59). With a
+// few waves the released blocks fill the last wave, and the earlier the better (rD3Q33 64^3 8.35 / 8.59 /
+// 8.65); with many waves it should not be before the wait (rD3Q45 101x103x97 59.3 / 57.7 / 60.0).
+enum { kReleaseFirst = 0, kReleaseAfterWait = 1, kReleaseLast = 2 };
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;"); }
+// Predicated, not branched over: a branch would keep the loads, the arithmetic and the stores on its two
+// sides apart (rD3Q33 64^3 8.4 -> 9.1 us a step).
+__device__ __forceinline__ void chain_release_if(int point, int here) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.eq.s32 q, %0, %1;\n\t@q griddepcontrol.launch_dependents;\n\t}" ::"r"(point),
+               "r"(here));
+}
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... KA>
+int release_point(void (*kernel)(KA...), int grid, int block, int device) {
+  int per_sm = 0, sms = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+    cudaGetLastError();
+    return kReleaseAfterWait;
+  }
+  const int64_t slots = int64_t(per_sm) * sms;
+  return grid <= slots ? kReleaseLast : (grid <= 4 * slots ? kReleaseFirst : kReleaseAfterWait);
+}
 
 template <class... KA, class... A>
 cudaError_t launch_chained(void (*kernel)(KA...), int grid, int block, size_t smem, cudaStream_t stream,

@@ -846,11 +846,12 @@ __device__ __forceinline__ const F2* cell_field_gradient(const Rates<F2>& p, con
 template <class L, class CT, class ST, int EQ, bool COLLIDE, bool KEEP>
 __global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepParams<CT> p, const ST* fin, ST* fout,
                                                                         CT* phi) {
-  chain_release();
+  chain_release_if(p.release, kReleaseFirst);
   const int cell = blockIdx.x * kBlock + threadIdx.x;
   if (cell >= p.ncells) return;
   const Neigh<L> nb(cell, p);
   chain_wait();
+  chain_release_if(p.release, kReleaseAfterWait);
   const size_t N = size_t(p.ncells);
   CT f[L::Q];
   constexpr bool DEV = is_deviation_storage<ST>();
@@ -874,6 +875,7 @@ __global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepPa
       if (p.grad_on) p.rho_out[cell] = phi_now;
     }
   }
+  chain_release_if(p.release, kReleaseLast);
   static_for<L::Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
     if constexpr (DEV) k1_store(fout + size_t(I) * N + cell, RawCodec<ST>::enc(f[I]));
@@ -919,7 +921,7 @@ __global__ void __launch_bounds__(kBlock, KEEP && L::Q > 33 ? 2 : (L::Q > 45 && 
     k_step_pair(const StepParams<F2, float> p, const ST* fin, ST* fout, float* phi) {
   constexpr int Q = L::Q, RM = L::RMAX;
   constexpr bool DEV = is_deviation_storage<ST>();
-  chain_release();
+  chain_release_if(p.release, kReleaseFirst);
   const int cell = 2 * (blockIdx.x * kBlock + threadIdx.x);
   if (cell >= p.ncells) return;
   const size_t N = size_t(p.ncells);
@@ -937,6 +939,7 @@ __global__ void __launch_bounds__(kBlock, KEEP && L::Q > 33 ? 2 : (L::Q > 45 && 
 #pragma unroll
     for (int sh = -RM; sh <= RM; ++sh) x1[sh + RM] = Neigh<L>::wrap1(n0.x + 1 - sh, sh == 0 ? 1 : sh, p.n[0]);
     chain_wait();
+    chain_release_if(p.release, kReleaseAfterWait);
     static_for<Q>([&](auto i) {
       constexpr int I = decltype(i)::value;
       constexpr Vel v = L::e(I);
@@ -955,6 +958,7 @@ __global__ void __launch_bounds__(kBlock, KEEP && L::Q > 33 ? 2 : (L::Q > 45 && 
     c1[1] = n1.y;
     c1[2] = n1.z;
     chain_wait();
+    chain_release_if(p.release, kReleaseAfterWait);
     static_for<Q>([&](auto i) {
       constexpr int I = decltype(i)::value;
       f[I] = F2(one(fin + size_t(I) * N + n0.template src<I>()), one(fin + size_t(I) * N + n1.template src<I>()));
@@ -995,6 +999,7 @@ __global__ void __launch_bounds__(kBlock, KEEP && L::Q > 33 ? 2 : (L::Q > 45 && 
   if constexpr (AG && EQ == LBM_NSE) {
     if (p.grad_on) field_out(p.rho_out);
   }
+  chain_release_if(p.release, kReleaseLast);
   static_for<Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
     ST* o = fout + size_t(I) * N + cell;
@@ -1023,13 +1028,13 @@ __global__ void __launch_bounds__(kBlock, 3) k_step_high(const StepParams<CT> p,
                                                           const HighParams<CT> hp, const ST* fin, ST* fout,
                                                           CT* phi) {
   __shared__ HighTable<L, CT> tab;
-  chain_release();
   tab.fill(hp);
   __syncthreads();
   const int cell = blockIdx.x * kBlock + threadIdx.x;
   if (cell >= p.ncells) return;
   const Neigh<L> nb(cell, p);
   chain_wait();
+  chain_release();
   const size_t N = size_t(p.ncells);
   CT f[L::Q];
   constexpr bool DEV = is_deviation_storage<ST>();
@@ -1123,6 +1128,7 @@ __device__ __forceinline__ void batch_cell(const LatTables<CT>& t, const SolveDe
   if constexpr (AG && EQ == LBM_NSE) {
     if (sd.grad_on) sd.rho_out[parity][cell] = phi_now;
   }
+  chain_release();  // of the block's first tile: before the stores, as a step of one wave
   static_for<L::Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
     if constexpr (DEV) k1_store(fout + size_t(I) * N + cell, RawCodec<ST>::enc(f[I]));
@@ -1144,7 +1150,6 @@ template <class L, class CT, class ST, int EQ, int BLOCK, bool KEEP>
 __global__ void __launch_bounds__(BLOCK, batch_min_blocks<BLOCK>())
     k_step_batch(const LatTables<CT> t, const SolveDesc<CT>* descs, const Tile* tiles, int ntiles, int parity) {
   __shared__ SolveDesc<CT> sd;
-  chain_release();
   chain_wait();
   int staged = -1;
   for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
@@ -1170,7 +1175,6 @@ __global__ void __launch_bounds__(kBlock, 3)
                       const Tile* tiles, int ntiles, int parity) {
   __shared__ SolveDesc<CT> sd;
   __shared__ HighTable<L, CT> tab;
-  chain_release();
   chain_wait();
   int staged = -1;
   for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
@@ -1357,6 +1361,7 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
   if (pairs) make_step_params(m, &p2);
   const int grid2 = (m->ncells / 2 + m->ncells % 2 + kBlock - 1) / kBlock;
   const bool hist = collide_on && m->m2g_aniso;
+  int release = -1;
   p.grad_on = collide_on && p.grad_on;
   if (rows || pairs) p2.grad_on = p.grad_on;
   for (int64_t s = 0; s < nsteps; ++s) {
@@ -1372,6 +1377,8 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
     }
     cudaError_t err = cudaSuccess;
     auto go = [&](auto kernel, int blocks, int threads, size_t smem, const auto&... args) {
+      if (release < 0) release = release_point(kernel, blocks, threads, m->device);
+      p.release = p2.release = release;
       err = launch_chained(kernel, blocks, threads, smem, m->stream, args..., fin, fout, phi);
     };
     bool done = false;

@@ -92,7 +92,6 @@ __global__ void __launch_bounds__(kRowPairs, row_ctas<KEEP && COLLIDE>())
   const int K = (rp.ntiles - int(blockIdx.x) + G - 1) / G;  // tiles of this CTA (the grid is <= ntiles)
   const int NS = rp.stages, RPT = rp.rpt;
   const size_t N = size_t(p.ncells);
-  chain_release();
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) tc::mbar_init(&full[s], kRowPairs);
     tc::mbar_fence_init();
@@ -103,6 +102,7 @@ __global__ void __launch_bounds__(kRowPairs, row_ctas<KEEP && COLLIDE>())
   }
   __syncthreads();
   chain_wait();
+  chain_release();
 
   // copies: lane group g of a warp takes the populations warp * groups + g, + 4 groups, ...; lane c of
   // the group takes 16-byte piece c of the tile's rows
