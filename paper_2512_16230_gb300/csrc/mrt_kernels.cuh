@@ -26,6 +26,8 @@
 // 16.4 -> 13.9 ms.
 #pragma once
 
+#include <algorithm>
+
 #include "lbm_internal.cuh"
 
 // Tuning knobs of the collide-stream kernel (defaults measured best on GB300 for rD3Q53 on
@@ -1195,6 +1197,7 @@ __global__ void __launch_bounds__(kBlock, 3)
 }  // namespace lbm
 
 #include "io_kernels.cuh"
+#include "resident.cuh"
 #include "tc_kernels.cuh"
 
 namespace lbm {
@@ -1353,6 +1356,31 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
         if (st != LBM_OK) return st;
         make_step_params(m, &p2);
       }
+    }
+  }
+  // small 2D grids: the whole call in one launch, the populations in a cluster's shared memory
+  if constexpr (!std::is_same<CT, double>::value && L::D == 2) {
+    int ctas = 0;
+    if (collide_on && !high && !tensor && resident_plan<L, ST>(m, nsteps, &ctas)) {
+      constexpr int64_t kMost = 1 << 16;  // steps of one launch
+      for (int64_t s = 0; s < nsteps;) {
+        const int n = int(std::min<int64_t>(kMost, nsteps - s));
+        const void* fin = m->f[m->cur];
+        void* fout = m->f[m->cur ^ 1];
+        cudaError_t err;
+        if (m->eq == LBM_NSE)
+          err = m->s_high == 1.0 ? launch_resident<L, ST, LBM_NSE, false>(m, p, n, ctas, fin, fout, phi)
+                                 : launch_resident<L, ST, LBM_NSE, true>(m, p, n, ctas, fin, fout, phi);
+        else
+          err = m->s_high == 1.0 ? launch_resident<L, ST, LBM_NCDE, false>(m, p, n, ctas, fin, fout, phi)
+                                 : launch_resident<L, ST, LBM_NCDE, true>(m, p, n, ctas, fin, fout, phi);
+        if (err != cudaSuccess) return cuda_error(err, "resident steps launch");
+        m->cur ^= 1;
+        m->launches += 1;
+        m->steps += n;
+        s += n;
+      }
+      return LBM_OK;
     }
   }
   // two cells per thread where the halved thread count still fills the GPU

@@ -139,3 +139,41 @@ def test_two_cells_per_thread_with_gradient_terms():
         one = m.get_populations()
         m.close()
         assert np.array_equal(one, _batched(spec, eq, n, f0, 4, prepare, **kw)), (name, n)
+
+
+# small 2D grids: a call of several steps runs in one launch on a cluster, calls of one step do not. Rows that
+# do not divide by the CTAs, fewer rows than CTAs, the largest grid taken and the first one that is not
+@pytest.mark.parametrize("store", ["f32", "f16_dev"])
+@pytest.mark.parametrize("s_high", [1.0, 1.3])
+@pytest.mark.parametrize("eq", ["nse", "ncde"])
+@pytest.mark.parametrize("name,grids", [("rD2Q13", [(37, 29), (5, 3), (630, 16), (631, 16)]), ("rD2Q25", [(64, 48), (7, 6), (20, 256)])])
+def test_steps_of_a_small_grid_in_one_launch(name, grids, eq, s_high, store):
+    spec = W.LATTICES[name]
+    for n in grids:
+        f0 = _populations(spec, n, 10, eq)
+        out = []
+        for calls in ([1] * 7, [5, 2]):
+            m = gpu_model(spec, eq, n, _rates(spec), store=store, **_kwargs(eq, 2, s_high))
+            m.set_populations(f0)
+            for k in calls:
+                m.step(k)
+            assert m.counters()[0] == 7
+            out.append(m.get_populations())
+            m.close()
+        assert np.array_equal(out[0], out[1]), n
+
+
+def test_steps_in_one_launch_with_per_cell_rates_and_cross_diffusion():
+    spec, n = W.LATTICES["rD2Q17"], (41, 23)
+    f0 = _populations(spec, n, 11, "ncde")
+    psi = np.random.default_rng(7).uniform(-1, 1, size=(n[1], n[0]))
+    out = []
+    for calls in ([1] * 6, [6]):
+        m = gpu_model(spec, "ncde", n, _rates(spec), store="f32", ncde_mode="rate", a1=-0.2, a2=0.02, psi=psi,
+                      **_kwargs("ncde", 2, 1.0))
+        m.set_populations(f0)
+        for k in calls:
+            m.step(k)
+        out.append(m.get_populations())
+        m.close()
+    assert np.array_equal(out[0], out[1])
