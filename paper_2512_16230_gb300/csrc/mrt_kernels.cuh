@@ -1363,8 +1363,8 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
     int ctas = 0;
     if (collide_on && !high && !tensor && resident_plan<L, ST>(m, nsteps, &ctas)) {
       constexpr int64_t kMost = 1 << 16;  // steps of one launch
-      for (int64_t s = 0; s < nsteps;) {
-        const int n = int(std::min<int64_t>(kMost, nsteps - s));
+      while (nsteps > 0) {
+        const int n = int(std::min<int64_t>(kMost, nsteps));
         const void* fin = m->f[m->cur];
         void* fout = m->f[m->cur ^ 1];
         cudaError_t err;
@@ -1374,13 +1374,16 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
         else
           err = m->s_high == 1.0 ? launch_resident<L, ST, LBM_NCDE, false>(m, p, n, ctas, fin, fout, phi)
                                  : launch_resident<L, ST, LBM_NCDE, true>(m, p, n, ctas, fin, fout, phi);
-        if (err != cudaSuccess) return cuda_error(err, "resident steps launch");
+        if (err != cudaSuccess) {  // no room for the cluster (a partitioned GPU): step by step
+          cudaGetLastError();
+          break;
+        }
         m->cur ^= 1;
         m->launches += 1;
         m->steps += n;
-        s += n;
+        nsteps -= n;
       }
-      return LBM_OK;
+      if (nsteps == 0) return LBM_OK;
     }
   }
   // two cells per thread where the halved thread count still fills the GPU

@@ -14,6 +14,7 @@
 namespace lbm {
 
 constexpr int kResidentThreads = 512;   // at most, one CTA per SM
+constexpr int kResidentSmem = 160 * 1024;  // above what the largest grid taken asks for
 constexpr int kResidentCtas = 16;       // CTAs of the cluster, at most (above 8 the size is opt-in)
 
 struct ResidentParams {
@@ -148,7 +149,7 @@ bool resident_plan(const lbm_model* m, int64_t nsteps, int* ctas) {
   // 100x76 2.07 / 2.01)
   if (rows * m->n[0] * L::Q > 8192) return false;
   *ctas = n;
-  return true;
+  return resident_smem<L, ST>(m, rows) <= size_t(kResidentSmem);
 }
 
 template <class L, class ST, int EQ, bool KEEP>
@@ -159,7 +160,8 @@ cudaError_t launch_resident(const lbm_model* m, const StepParams<float>& p, int 
   rp.rows = int((m->n[1] + ctas - 1) / ctas);
   const size_t smem = resident_smem<L, ST>(m, rp.rows);
   auto kernel = k_steps_resident<L, ST, EQ, KEEP>;
-  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  // (one limit for every grid: a thread that launches another grid must not lower it in between)
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmem);
   if (err == cudaSuccess && ctas > 8)
     err = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (err != cudaSuccess) return err;

@@ -698,8 +698,11 @@ lbm_status row_tc_kernel(int store, int eq, bool high, F&& fn) {
 template <int KIND>
 lbm_status RowLaunch<KIND>::configure(const lbm_model* m, const RowPlan& plan, bool collide) {
   using L = Lat<KIND>;
+  int most = 0;  // one limit for every plan of a kernel, whichever thread sets it last
+  if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, m->device) != cudaSuccess)
+    return cuda_error(cudaGetLastError(), "row-staged kernel attributes");
   auto set = [&](auto kernel) -> lbm_status {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(plan.smem)) != cudaSuccess ||
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
         cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                              int(cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
       return cuda_error(cudaGetLastError(), "row-staged kernel attributes");
