@@ -333,6 +333,12 @@ __device__ __forceinline__ void chain_release_if(int point, int here) {
 }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+inline int sm_count(int device) {
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) cudaGetLastError();
+  return sms;
+}
+
 template <class... KA>
 int release_point(void (*kernel)(KA...), int grid, int block, int device) {
   int per_sm = 0, sms = 0;

@@ -138,24 +138,29 @@ __device__ __forceinline__ Signed4<V> signed4(V pp, V pm, V mp, V mm) {
 // are formed once: for rD3Q53 104 operations in dir_sums and 88 here, against 152 with one
 // multiply-add per direction and monomial.
 template <class L, class V>
+__device__ __forceinline__ void raw_moments_2d(V f0, const DirSums<V>& X, const DirSums<V>& Y, const DirSums<V>& P,
+                                               const DirSums<V>& M, V (&mu)[L::R]) {
+  mu[0] = (f0 + (X.s0 + Y.s0)) + (P.s0 + M.s0);
+  mu[1] = X.s1 + (P.s1 + M.s1);
+  mu[2] = Y.s1 + (P.s1 - M.s1);
+  const V d2 = P.s2 + M.s2, o3 = P.s3 + M.s3, q3 = P.s3 - M.s3;
+  mu[row2<2>(0, 0)] = X.s2 + d2;
+  mu[row2<2>(1, 1)] = Y.s2 + d2;
+  mu[row2<2>(0, 1)] = P.s2 - M.s2;
+  mu[row3<2>(0, 1, 1)] = o3;
+  mu[row3<2>(0, 0, 1)] = q3;
+  if constexpr (!L::SINGLE) {
+    mu[row3<2>(0, 0, 0)] = X.s3 + o3;
+    mu[row3<2>(1, 1, 1)] = Y.s3 + q3;
+  }
+}
+
+template <class L, class V>
 __device__ __forceinline__ void raw_moments(const V (&f)[L::Q], V (&mu)[L::R]) {
   constexpr int D = L::D;
   if constexpr (D == 2) {
-    const DirSums<V> X = dir_sums<L, 1, 0, 0>(f), Y = dir_sums<L, 0, 1, 0>(f);
-    const DirSums<V> P = dir_sums<L, 1, 1, 0>(f), M = dir_sums<L, 1, -1, 0>(f);
-    mu[0] = (f[0] + (X.s0 + Y.s0)) + (P.s0 + M.s0);
-    mu[1] = X.s1 + (P.s1 + M.s1);
-    mu[2] = Y.s1 + (P.s1 - M.s1);
-    const V d2 = P.s2 + M.s2, o3 = P.s3 + M.s3, q3 = P.s3 - M.s3;
-    mu[row2<2>(0, 0)] = X.s2 + d2;
-    mu[row2<2>(1, 1)] = Y.s2 + d2;
-    mu[row2<2>(0, 1)] = P.s2 - M.s2;
-    mu[row3<2>(0, 1, 1)] = o3;
-    mu[row3<2>(0, 0, 1)] = q3;
-    if constexpr (!L::SINGLE) {
-      mu[row3<2>(0, 0, 0)] = X.s3 + o3;
-      mu[row3<2>(1, 1, 1)] = Y.s3 + q3;
-    }
+    raw_moments_2d<L>(f[0], dir_sums<L, 1, 0, 0>(f), dir_sums<L, 0, 1, 0>(f), dir_sums<L, 1, 1, 0>(f),
+                      dir_sums<L, 1, -1, 0>(f), mu);
   } else {
     const DirSums<V> ax[3] = {dir_sums<L, 1, 0, 0>(f), dir_sums<L, 0, 1, 0>(f), dir_sums<L, 0, 0, 1>(f)};
     // space diagonals (1, +-1, +-1)
@@ -231,29 +236,40 @@ __device__ __forceinline__ void dir_out(V (&f)[L::Q], const LatTables<V>& lt, V 
   });
 }
 
+// The populations of one direction of a 2D lattice: W = 0 (1, 0) and the rest, 1 (0, 1), 2 (1, 1), 3 (1, -1).
+template <class L, bool KEEP, int W, class V>
+__device__ __forceinline__ void back_direction_2d(V (&f)[L::Q], const LatTables<V>& lt, const V (&h)[L::R], V oms) {
+  const V h0 = h[0];
+  if constexpr (W == 0) {
+    if constexpr (KEEP) f[0] = fmaf_t(oms, f[0], lt.w[0] * h0);
+    else f[0] = lt.w[0] * h0;
+  }
+  if constexpr (W < 2) {
+    V cube = V(0.f);
+    if constexpr (!L::SINGLE) cube = h[row3<2>(W, W, W)];
+    dir_out<L, W == 0, W == 1, 0, KEEP>(f, lt, oms, h0, h[1 + W], h[row2<2>(W, W)], cube);
+  } else {
+    V ox = h[row3<2>(0, 1, 1)], oy = h[row3<2>(0, 0, 1)];
+    if constexpr (!L::SINGLE) {
+      ox = h[row3<2>(0, 0, 0)] + ox;
+      oy = h[row3<2>(1, 1, 1)] + oy;
+    }
+    const V s2 = h[row2<2>(0, 0)] + h[row2<2>(1, 1)], m = h[row2<2>(0, 1)];
+    if constexpr (W == 2) dir_out<L, 1, 1, 0, KEEP>(f, lt, oms, h0, h[1] + h[2], s2 + m, ox + oy);
+    else dir_out<L, 1, -1, 0, KEEP>(f, lt, oms, h0, h[1] - h[2], s2 - m, ox - oy);
+  }
+}
+
 // f_i = (1 - s_h) f_i + w_i sum_k mono_k(e_i) h_k, with the sums of raw_moments transposed.
 template <class L, bool KEEP, class V>
 __device__ __forceinline__ void back_project(V (&f)[L::Q], const LatTables<V>& lt, const V (&h)[L::R], V oms) {
   constexpr int D = L::D;
-  const V h0 = h[0];
-  if constexpr (KEEP) f[0] = fmaf_t(oms, f[0], lt.w[0] * h0);
-  else f[0] = lt.w[0] * h0;
   if constexpr (D == 2) {
-    V hx3 = V(0.f), hy3 = V(0.f);
-    const V o = h[row3<2>(0, 1, 1)], q = h[row3<2>(0, 0, 1)];
-    V ox = o, oy = q;
-    if constexpr (!L::SINGLE) {
-      hx3 = h[row3<2>(0, 0, 0)];
-      hy3 = h[row3<2>(1, 1, 1)];
-      ox = hx3 + o;
-      oy = hy3 + q;
-    }
-    dir_out<L, 1, 0, 0, KEEP>(f, lt, oms, h0, h[1], h[row2<2>(0, 0)], hx3);
-    dir_out<L, 0, 1, 0, KEEP>(f, lt, oms, h0, h[2], h[row2<2>(1, 1)], hy3);
-    const V s2 = h[row2<2>(0, 0)] + h[row2<2>(1, 1)], m = h[row2<2>(0, 1)];
-    dir_out<L, 1, 1, 0, KEEP>(f, lt, oms, h0, h[1] + h[2], s2 + m, ox + oy);
-    dir_out<L, 1, -1, 0, KEEP>(f, lt, oms, h0, h[1] - h[2], s2 - m, ox - oy);
+    static_for<4>([&](auto w) { back_direction_2d<L, KEEP, decltype(w)::value>(f, lt, h, oms); });
   } else {
+    const V h0 = h[0];
+    if constexpr (KEEP) f[0] = fmaf_t(oms, f[0], lt.w[0] * h0);
+    else f[0] = lt.w[0] * h0;
     V cube[3];
     static_for<3>([&](auto aa) {
       constexpr int A = decltype(aa)::value;
@@ -1022,6 +1038,94 @@ __global__ void __launch_bounds__(kBlock, KEEP && L::Q > 33 ? 2 : (L::Q > 45 && 
   });
 }
 
+// K1 on a small 2D grid in FP64, four threads per cell. GB300 runs one FP64 warp instruction per 64
+// clocks and SM sub-partition, whatever the number of active lanes, so a grid with fewer warps of cells
+// than there are sub-partitions (608) takes the time of one cell's instructions on a few of them. Here warp
+// W of a block owns direction W of 32 cells: it loads, sums and writes that direction's populations, the
+// sums go through shared memory, warps 0 and 1 do the even and the odd rows of the moment-space part, and its
+// result goes through shared memory too. Same operations in the same order as k_step, bitwise the same
+// results. rD2Q25 64x48: 9.5 us per step with one thread per cell, 4.9 here, of which 1.9 is a launch in a
+// chain; the longest chain is now the even or odd rows' (a quarter of the cell's operations each).
+template <class L, int EQ, bool KEEP, int W>
+__device__ __forceinline__ void split_direction(const StepParams<double>& p, const double* fin, double* fout,
+                                                double* phi, const Neigh<L>& nb, int cell, bool live,
+                                                double (&sums)[17][32], double (&coef)[10][32]) {
+  constexpr int Q = L::Q;
+  constexpr int DX = W != 1, DY = W == 0 ? 0 : (W == 3 ? -1 : 1);
+  const int lane = threadIdx.x & 31;
+  const size_t N = size_t(p.ncells);
+  double f[Q];
+  double phi_prev = 0.0, phi_now = 0.0;
+  auto mine = [](int i) constexpr {
+    return i == 0 ? W == 0 : same_vel(primitive(L::e(i)), Vel{DX, DY, 0});
+  };
+  if (live) {
+    static_for<Q>([&](auto i) {
+      constexpr int I = decltype(i)::value;
+      if constexpr (mine(I)) f[I] = k1_load(fin + size_t(I) * N + nb.template src<I>());
+    });
+    if constexpr (EQ == LBM_NCDE) phi_prev = phi[cell];
+    const DirSums<double> r = dir_sums<L, DX, DY, 0>(f);
+    sums[4 * W][lane] = r.s0;
+    sums[4 * W + 1][lane] = r.s1;
+    sums[4 * W + 2][lane] = r.s2;
+    sums[4 * W + 3][lane] = r.s3;
+    if constexpr (W == 0) sums[16][lane] = f[0];
+  }
+  asm volatile("bar.sync 1, 128;" ::: "memory");  // one barrier for the block's four warps, each from its own code
+  // W = 0: the coefficients of 1, aa, ab; W = 1: of a and the third order (what the other needs is dropped by
+  // the compiler)
+  auto mine_row = [](int r) constexpr { return (degree(mono<2>(r)) % 2 == 0) == (W == 0); };
+  double h[L::R];
+  if (W < 2 && live) {
+    auto dir = [&](int d) {
+      return DirSums<double>{sums[4 * d][lane], sums[4 * d + 1][lane], sums[4 * d + 2][lane], sums[4 * d + 3][lane]};
+    };
+    double mu[L::R], F[3], gr[3];
+    raw_moments_2d<L>(sums[16][lane], dir(0), dir(1), dir(2), dir(3), mu);
+    const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, nb.x, nb.y, 0, F);
+    constexpr bool AG = GradTerm<L, EQ>::kOn;
+    const double* grad = nullptr;
+    if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, nb.x, nb.y, 0, gr);
+    collide_moments<L, double, EQ, false>(mu, p, p, forced, F, phi_prev, phi_now, h, grad);
+    if constexpr (W == 0 && EQ == LBM_NCDE) phi[cell] = phi_now;
+    if constexpr (W == 0 && AG && EQ == LBM_NSE) {
+      if (p.grad_on) p.rho_out[cell] = phi_now;
+    }
+    static_for<L::R>([&](auto r) {
+      constexpr int Rr = decltype(r)::value;
+      if constexpr (mine_row(Rr)) coef[Rr][lane] = h[Rr];
+    });
+  }
+  asm volatile("bar.sync 1, 128;" ::: "memory");
+  if (!live) return;
+  static_for<L::R>([&](auto r) { h[decltype(r)::value] = coef[decltype(r)::value][lane]; });
+  back_direction_2d<L, KEEP, W>(f, p, h, p.one_minus_sh);
+  static_for<Q>([&](auto i) {
+    constexpr int I = decltype(i)::value;
+    if constexpr (mine(I)) k1_store(fout + size_t(I) * N + cell, f[I]);
+  });
+}
+
+template <class L, int EQ, bool KEEP>
+__global__ void __launch_bounds__(128) k_step_split(const StepParams<double> p, const double* fin, double* fout,
+                                                    double* phi) {
+  __shared__ double sums[17][32];  // per direction and degree, and the rest population
+  __shared__ double coef[10][32];  // the coefficients of the monomials
+  const int raw_cell = blockIdx.x * 32 + (threadIdx.x & 31);
+  const bool live = raw_cell < p.ncells;
+  const int cell = live ? raw_cell : p.ncells - 1;
+  const Neigh<L> nb(cell, p);
+  chain_wait();
+  chain_release();
+  switch (threadIdx.x >> 5) {
+    case 0: split_direction<L, EQ, KEEP, 0>(p, fin, fout, phi, nb, cell, live, sums, coef); break;
+    case 1: split_direction<L, EQ, KEEP, 1>(p, fin, fout, phi, nb, cell, live, sums, coef); break;
+    case 2: split_direction<L, EQ, KEEP, 2>(p, fin, fout, phi, nb, cell, live, sums, coef); break;
+    default: split_direction<L, EQ, KEEP, 3>(p, fin, fout, phi, nb, cell, live, sums, coef); break;
+  }
+}
+
 // K1 with distinct rates for the orders >= 4: the same gather / collide / store plus the two
 // contractions with the higher rows (about 2 (Q - 1) (Q - R) / 2 more FMAs per cell, so the
 // kernel is bound by instruction issue rather than HBM; 3 resident blocks leave it 168 registers).
@@ -1391,6 +1495,13 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
                                       m->ncells >= kPairCells;
   if (pairs) make_step_params(m, &p2);
   const int grid2 = (m->ncells / 2 + m->ncells % 2 + kBlock - 1) / kBlock;
+  // FP64 on a small 2D grid: four threads per cell while every block of 32 cells has an SM of its own. Us per
+  // step, one thread per cell against four (a first version): 80x60 cells, 150 blocks, rD2Q13 6.4 / 5.2, rD2Q25
+  // 9.6 / 6.1; 100x76, 238 blocks, 6.4 / 7.7 and 9.6 / 9.2; 128x96 6.5 / 10.5 and 9.6 / 13.
+  [[maybe_unused]] const int grid_split = (m->ncells + 31) / 32;
+  [[maybe_unused]] bool split = false;
+  if constexpr (std::is_same<CT, double>::value && L::D == 2)
+    split = collide_on && !high && grid_split <= sm_count(m->device);
   const bool hist = collide_on && m->m2g_aniso;
   int release = -1;
   p.grad_on = collide_on && p.grad_on;
@@ -1450,6 +1561,18 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
         };
         if (m->eq == LBM_NSE) by_keep(std::integral_constant<int, LBM_NSE>{});
         else by_keep(std::integral_constant<int, LBM_NCDE>{});
+        done = true;
+      }
+    }
+    if constexpr (std::is_same<CT, double>::value && L::D == 2) {
+      if (split) {
+        if (m->eq == LBM_NSE) {
+          if (m->s_high == 1.0) go(k_step_split<L, LBM_NSE, false>, grid_split, 128, 0, p);
+          else go(k_step_split<L, LBM_NSE, true>, grid_split, 128, 0, p);
+        } else {
+          if (m->s_high == 1.0) go(k_step_split<L, LBM_NCDE, false>, grid_split, 128, 0, p);
+          else go(k_step_split<L, LBM_NCDE, true>, grid_split, 128, 0, p);
+        }
         done = true;
       }
     }

@@ -177,3 +177,21 @@ def test_steps_in_one_launch_with_per_cell_rates_and_cross_diffusion():
         out.append(m.get_populations())
         m.close()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("s_high", [1.0, 1.3])
+@pytest.mark.parametrize("eq", ["nse", "ncde"])
+@pytest.mark.parametrize("name", ["rD2Q9", "rD2Q13", "rD2Q25"])
+def test_fp64_small_grid_is_the_large_one_periodically(name, eq, s_high):
+    """A small FP64 grid takes four threads per cell, a large one one thread: repeated periodically along x, the
+    small solve is bitwise the large one (48 x 33 against 12 copies of it)."""
+    spec, n, copies = W.LATTICES[name], (48, 33), 12
+    f0 = _populations(spec, n, 12, eq)
+    out = []
+    for k in (1, copies):
+        m = gpu_model(spec, eq, (n[0] * k, n[1]), _rates(spec), store="f64", **_kwargs(eq, 2, s_high))
+        m.set_populations(np.tile(f0, (1, 1, k)))
+        m.step(3)
+        out.append(m.get_populations())
+        m.close()
+    assert np.array_equal(np.tile(out[0], (1, 1, copies)), out[1])
