@@ -199,8 +199,9 @@ lbm_status lbm_model_set_bulk(lbm_model* m, double s_bulk);
  * matrix; the higher rows as in lbm_lattice_query_high): s_order[k] is the rate of order 4 + k,
  * k < n_orders <= 9; the orders not given relax with s_high. Rates must lie in (0, 2]. Since the
  * equilibrium and the sources have no moments of order >= 4, the update adds
- * -w_i sum_r (s_r - s_high) H_r(c_i) (sum_j H_r(c_j) f_j) / N_r over those rows, which costs the
- * step two more contractions with them. n_orders = 0 restores the shared rate.
+ * -w_i sum_r (s_r - s_high) H_r(c_i) (sum_j H_r(c_j) f_j) / N_r over those rows. The kernels apply it in
+ * the functions adapted to the reflections of the axes, where it is block diagonal (469 multiply-adds
+ * per cell on rD3Q53). n_orders = 0 restores the shared rate.
  * Inside a batch the solve joins a group of solves with per-order rates (CUDA cores).
  * Errors: LBM_ERR_ARG, LBM_ERR_LATTICE_INFEASIBLE (lattice without complete higher rows). */
 lbm_status lbm_model_set_high_rates(lbm_model* m, const double* s_order, int n_orders);
@@ -216,9 +217,9 @@ lbm_status lbm_model_set_high_rates(lbm_model* m, const double* s_order, int n_o
  * G_ij = sum_r a_r H_r(c_i) H_r(c_j) (a_r = -(s_r - s_high) / N_r, built in FP64), one product
  * per 128-cell tile with both operands as FP16 high/low splits of power-of-two scaled values
  * (three products, about 22 bits); without per-order rates FP32 storage always uses the
- * CUDA-core kernel. Default, until this is
- * called: the tensor cores with distinct higher-order rates (there they are the faster kernel),
- * the CUDA cores otherwise.
+ * CUDA-core kernel. Default, until this is called: the CUDA cores, except with per-order rates on
+ * 16-bit storage where the row-staged kernel is the faster one (rD3Q53, n_x = 240 .. 256, at least 64
+ * rows per SM) or the gather is forced to ROWS.
  * Device-side waits are bounded; a timeout is latched in the model's status word and returned as
  * LBM_ERR_TIMEOUT by the next lbm_model_synchronize / read / get / sums call. After a timeout the
  * populations (and the NCDE / density history fields) are undefined: re-initialise the model

@@ -23,7 +23,7 @@ struct GroupHost {
   lbm::BatchGroup g;
   lbm::LatTables<float> tables;
   std::vector<lbm::SolveDesc<float>> desc;
-  std::vector<lbm::HighParams<float>> high;  // per solve, for a group with per-order rates
+  std::vector<lbm::HighCoefs<float>> high;  // per solve, for a group with per-order rates
   std::vector<lbm_model*> members;
 };
 
@@ -290,7 +290,7 @@ lbm_status rebuild(lbm_batch* b) {
     for (size_t j = 0; j < gh.members.size(); ++j) {
       fill_desc(gh.members[j], &gh.desc[j]);
       if (gh.members[j]->s_high != 1.0) gh.g.keep = 1;
-      if (gh.g.high) make_high_params<float>(gh.members[j], &gh.high[j]);
+      if (gh.g.high) make_high_coefs(gh.members[j], &gh.high[j]);
       for (int c0 = 0; c0 < gh.members[j]->ncells; c0 += gh.g.block) tiles.push_back(Tile{int(j), c0});
     }
     gh.g.nsolves = int(gh.members.size());
@@ -302,7 +302,7 @@ lbm_status rebuild(lbm_batch* b) {
     cudaError_t err = ensure(&buf.desc, &buf.desc_cap, gh.desc.size() * sizeof(SolveDesc<float>));
     if (err == cudaSuccess) err = ensure(&buf.tiles, &buf.tiles_cap, tiles.size() * sizeof(Tile));
     if (err == cudaSuccess && gh.g.high)
-      err = ensure(&buf.high, &buf.high_cap, gh.high.size() * sizeof(HighParams<float>));
+      err = ensure(&buf.high, &buf.high_cap, gh.high.size() * sizeof(HighCoefs<float>));
     gh.g.d_desc = buf.desc;
     gh.g.d_tiles = static_cast<Tile*>(buf.tiles);
     gh.g.d_high = gh.g.high ? buf.high : nullptr;
@@ -310,7 +310,7 @@ lbm_status rebuild(lbm_batch* b) {
       err = cudaMemcpyAsync(gh.g.d_tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice,
                             b->stream);
     if (err == cudaSuccess && gh.g.high)
-      err = cudaMemcpyAsync(gh.g.d_high, gh.high.data(), gh.high.size() * sizeof(HighParams<float>),
+      err = cudaMemcpyAsync(gh.g.d_high, gh.high.data(), gh.high.size() * sizeof(HighCoefs<float>),
                             cudaMemcpyHostToDevice, b->stream);
     if (err != cudaSuccess) return cuda_error(err, "batch work-list allocation");
     lbm_status st = upload_desc(b, gh);

@@ -3,7 +3,7 @@
 // the Q loads of a cell are independent and in flight together. (A first form read the velocities
 // from a table with a run-time index, one load after another. rD3Q53 256x256x192 fields FP32 950 -> 497
 // us (452 us at the copy bandwidth), FP16 1000 -> 452 us; 128x128x96 FP32 populations in FP64 190 ->
-// 173 us (147), into the model 170 -> 152 us (147), conservation sums 111 -> 95 us (49).)
+// 173 us (147), into the model 170 -> 152 us (147), conservation sums 111 -> 68 us (49).)
 #pragma once
 
 namespace lbm {
@@ -129,7 +129,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // order and writes its four partial sums. Streaming is a permutation, so the stored array has
 // the same totals as f-bar and needs no gather.
 template <class L, class CT, class ST>
-__global__ void __launch_bounds__(256) k_sums_partial(const StepParams<CT> p, const double3 c,
+__global__ void __launch_bounds__(256, 4) k_sums_partial(const StepParams<CT> p, const double3 c,
                                                       const ST* __restrict__ A, double* __restrict__ partials) {
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   const size_t N = size_t(p.ncells);

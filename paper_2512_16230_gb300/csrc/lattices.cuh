@@ -214,25 +214,6 @@ constexpr int pair_plus(int p) {
     }
   return -1;
 }
-// Rows of order >= 4 of the complete Q x Q Hermite matrix, split by parity under e -> -e: the
-// even lattice functions span the rest velocity and one function per pair (num_pairs + 1), the
-// odd ones one per pair; the orders <= 3 take the even rows of degree 0, 2 and the odd ones of
-// degree 1, 3.
-template <class L>
-constexpr int low_rows_even() {
-  int n = 0;
-  for (int r = 0; r < L::R; ++r) n += (degree(mono<L::D>(r)) % 2 == 0) ? 1 : 0;
-  return n;
-}
-template <class L>
-constexpr int high_even() {
-  return num_pairs<L>() + 1 - low_rows_even<L>();
-}
-template <class L>
-constexpr int high_odd() {
-  return num_pairs<L>() - (L::R - low_rows_even<L>());
-}
-
 // static_for<N>(f) calls f(std::integral_constant<int, 0>) ... f(integral_constant<int, N-1>).
 // Inside nested lambdas, read a captured index as decltype(i)::value (a constant expression
 // whatever the capture); the constexpr helpers above are evaluated at compile time only.
@@ -268,20 +249,6 @@ inline int lattice_q(int kind) {
   return 0;
 }
 inline Vel lattice_e(int kind, int j) { return lattice_dims(kind) == 2 ? kQ25[j] : q53(j); }
-// Host view of the pair order above: plus[p] for p < (Q - 1) / 2.
-inline void lattice_pairs(int kind, int* plus) {
-  const int Q = lattice_q(kind);
-  int n = 0;
-  for (int i = 1; i < Q; ++i) {
-    const Vel a = lattice_e(kind, i);
-    int opp = -1;
-    for (int j = 0; j < Q; ++j) {
-      const Vel b = lattice_e(kind, j);
-      if (a.x == -b.x && a.y == -b.y && a.z == -b.z) opp = j;
-    }
-    if (opp > i) plus[n++] = i;
-  }
-}
 inline int lattice_rmax(int kind) {
   if (lattice_single(kind)) return 1;
   return (kind == LBM_RD2Q17 || kind == LBM_RD2Q21 || kind == LBM_RD2Q25) ? 3 : 2;
@@ -289,9 +256,6 @@ inline int lattice_rmax(int kind) {
 
 constexpr int kMaxQ = 53;
 constexpr int kMaxR = 20;
-constexpr int kMaxPairs = 26;  // rD3Q53
-constexpr int kMaxHighEven = 20;
-constexpr int kMaxHighOdd = 13;
 constexpr int kMaxOrder = 12;  // highest monomial degree tried when completing the Hermite matrix
 
 }  // namespace lbm

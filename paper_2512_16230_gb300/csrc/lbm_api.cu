@@ -214,26 +214,9 @@ bool has_high_rates(const lbm_model* m) {
   return false;
 }
 
-template <class CT>
-void make_high_params(const lbm_model* m, HighParams<CT>* hp) {
-  const lbm_lattice* L = m->lat;
-  std::memset(hp, 0, sizeof(*hp));
-  int plus[kMaxPairs];
-  lattice_pairs(L->kind, plus);
-  const int np = (L->Q - 1) / 2;
-  int ne = 0, no = 0;
-  for (int r = 0; r < L->nhigh; ++r) {
-    const double* h = L->Hh + size_t(r) * L->Q;
-    const double a = -(high_rate(m, L->h_order[r]) - m->s_high) / L->Nh[r];
-    if ((L->h_order[r] & 1) == 0) {
-      hp->he[ne][0] = CT(h[0]);
-      for (int q = 0; q < np; ++q) hp->he[ne][q + 1] = CT(h[plus[q]]);
-      hp->ae[ne++] = CT(a);
-    } else {
-      for (int q = 0; q < np; ++q) hp->ho[no][q] = CT(h[plus[q]]);
-      hp->ao[no++] = CT(a);
-    }
-  }
+template <class V>
+void make_high_coefs(const lbm_model* m, HighCoefs<V>* hc) {
+  for (int k = 0; k < kMaxHighCoefs; ++k) hc->c[k] = V(m->high_c[k]);
 }
 
 void make_tc_params(const lbm_model* m, TcParams* tp) {
@@ -304,8 +287,8 @@ int tc_grid(const lbm_model* m, int ntiles, const void* kernel, int ctas_per_sm,
   return ntiles < g ? ntiles : g;
 }
 
-template void make_high_params<float>(const lbm_model*, HighParams<float>*);
-template void make_high_params<double>(const lbm_model*, HighParams<double>*);
+template void make_high_coefs<float>(const lbm_model*, HighCoefs<float>*);
+template void make_high_coefs<double>(const lbm_model*, HighCoefs<double>*);
 
 namespace {
 
@@ -492,6 +475,15 @@ lbm_status dispatch_kind(int kind, F&& f) {
     case LBM_RD3Q27: return f(std::integral_constant<int, LBM_RD3Q27>{});
   }
   return set_error(LBM_ERR_ARG, "unknown lattice kind");
+}
+
+// The operator of the rows of order >= 4, when one of the rates has changed.
+void update_high(lbm_model* m) {
+  if (!has_high_rates(m)) return;
+  dispatch_kind(m->lat->kind, [&](auto kind) -> lbm_status {
+    Launch<decltype(kind)::value>::high_operator_blocks(m, m->high_c);
+    return LBM_OK;
+  });
 }
 
 // Run fn with a device staging buffer of `bytes` when the user buffer is in host memory.
@@ -691,6 +683,7 @@ lbm_status lbm_model_set_relaxation(lbm_model* m, const double* s, double s_high
   if (!(s_high > 0.0 && s_high <= 2.0)) return set_error(LBM_ERR_ARG, "rates must lie in (0, 2]");
   for (int r = 0; r < m->lat->R; ++r) m->s[r] = s[r];
   m->s_high = s_high;
+  update_high(m);
   batch_mark_dirty(m->batch);
   return LBM_OK;
 }
@@ -722,6 +715,7 @@ lbm_status lbm_model_set_high_rates(lbm_model* m, const double* s_order, int n_o
                                                      ? "the graded monomials do not complete the Hermite matrix"
                                                      : "a higher-order row has zero W-norm (zero weights)");
   for (int k = 0; k <= kMaxOrder; ++k) m->s_order[k] = next[k];
+  update_high(m);
   batch_mark_dirty(m->batch);
   return LBM_OK;
 }

@@ -13,6 +13,10 @@
 #include "lattices.cuh"
 #include "lbm_mrt.h"
 
+namespace lbm {
+constexpr int kMaxHighCoefs = 472;  // rD3Q53: 469
+}
+
 // Host-side lattice handle: the FP64 tables built on the GPU by the set-up kernel.
 struct lbm_lattice {
   int kind, d, Q, R, rmax;
@@ -64,7 +68,7 @@ struct lbm_model {
   double s_high, cs2_eq, rho_ref;
   double s_bulk;  // bulk relaxation rate of Eq. (4-27); <= 0: normal rows relax with their own rates
   double s_order[lbm::kMaxOrder + 1];  // rate of the rows of each order >= 4 (defaults to s_high)
-  bool high_explicit;                  // some order >= 4 has a rate other than s_high
+  double high_c[lbm::kMaxHighCoefs];   // the operator of those rows for the rates set (high.cuh)
   int force_a, force_b, force_k;
   double force_A, force_phase;
   double u_const[3];
@@ -160,16 +164,19 @@ struct StepParams : LatTables<V>, Rates<V> {
   int release;           // where a block lets the next launch of the chain start (kRelease...)
 };
 
-// Rows of order >= 4 that relax with their own rates (the full Q x Q collision). The kernel
-// adds w_i sum_r h_r(c_i) a_r y_r with y_r = sum_j h_r(c_j) f_j and a_r = -(s_r - s_high) / N_r
-// to the reduced-form update; even rows are read at the rest velocity and at the + member of
-// each +-e pair, odd rows at the + members (their value at -e is the negative).
-template <class CT>
-struct HighParams {
-  CT he[kMaxHighEven][kMaxPairs + 1];
-  CT ho[kMaxHighOdd][kMaxPairs];
-  CT ae[kMaxHighEven];
-  CT ao[kMaxHighOdd];
+// The operator of the rows of order >= 4 with rates of their own, in blocks (high.cuh).
+// the type of one coefficient in a kernel that works on V
+template <class V>
+struct Coef {
+  using type = V;
+};
+template <>
+struct Coef<F2> {
+  using type = float;
+};
+template <class V>
+struct alignas(16) HighCoefs {
+  V c[kMaxHighCoefs];
 };
 
 // Tensor-core kernel parameters: the monomial table mono_k(e_i) (paper's row order) and the
@@ -340,9 +347,9 @@ inline int sm_count(int device) {
 }
 
 template <class... KA>
-int release_point(void (*kernel)(KA...), int grid, int block, int device) {
+int release_point(void (*kernel)(KA...), int grid, int block, size_t smem, int device) {
   int per_sm = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
     cudaGetLastError();
     return kReleaseAfterWait;
@@ -405,7 +412,7 @@ struct BatchGroup {
   const lbm_lattice* lat;
   void* tables;     // host copy of LatTables<CT>
   void* d_desc;     // device SolveDesc<CT>[nsolves]
-  void* d_high;     // device HighParams<CT>[nsolves] (high groups)
+  void* d_high;     // device HighCoefs<CT>[nsolves] (high groups)
   Tile* d_tiles;    // device work-list
   int nsolves, ntiles, grid;
 };
@@ -429,6 +436,7 @@ struct IoCall {
 template <int KIND>
 struct Launch {
   static lbm_status io(lbm_model* m, const IoCall& io);
+  static void high_operator_blocks(const lbm_model* m, double* c);
   static lbm_status step(lbm_model* m, int64_t nsteps, bool collide);
   static lbm_status init(lbm_model* m, const double* rho_or_phi, const double* u);
 };
@@ -454,8 +462,10 @@ lbm_status setup_lattice_fp64(lbm_lattice* lat);
 // Host-side construction of the step parameters from a model.
 template <class V, class FT>
 void make_step_params(const lbm_model* m, StepParams<V, FT>* p);
-template <class CT>
-void make_high_params(const lbm_model* m, HighParams<CT>* hp);
+// the higher rows' operator of the model, in the type of a kernel
+template <class V>
+void make_high_coefs(const lbm_model* m, HighCoefs<V>* hc);
+double high_rate(const lbm_model* m, int order);
 // true when some row of order >= 4 relaxes with a rate other than s_high
 bool has_high_rates(const lbm_model* m);
 void make_tc_params(const lbm_model* m, TcParams* tp);

@@ -388,143 +388,11 @@ __device__ __forceinline__ V ncde_flux(const Rates<V>& rt, V phi) {
   return fmaf_t(rt.nonlin_third, phi * phi * phi, phi);
 }
 
-// Coefficients of the rows of order >= 4 staged in shared memory, row-major (the values of one
-// row at the rest velocity, c = 0, and at the + member of each +-e pair, c = P + 1, adjacent, so
-// that one vector load serves four pairs), with a per-thread slot for each row's z_r. The row
-// loops run at run time (rows outermost, pairs unrolled), which keeps the register footprint at
-// the populations plus one accumulator per pair.
-template <class L, class CT>
-struct HighTable {
-  static constexpr int HE = high_even<L>(), HO = high_odd<L>();
-  static constexpr int NP = num_pairs<L>();
-  static constexpr int CE = (NP + 1 + 3) / 4 * 4, CO = (NP + 3) / 4 * 4;  // padded row lengths
-  alignas(16) CT he[HE * CE];
-  alignas(16) CT ho[(HO > 0 ? HO : 1) * CO];
-  CT ae[HE];
-  CT ao[HO > 0 ? HO : 1];
-  CT z[(HE + HO) * kBlock];  // z_r of thread t at z[r * kBlock + t]
-  // block-wide copy from the kernel parameters (call before any thread returns)
-  __device__ __forceinline__ void fill(const HighParams<CT>& hp) {
-    for (int idx = threadIdx.x; idx < HE * (NP + 1); idx += blockDim.x)
-      he[(idx / (NP + 1)) * CE + idx % (NP + 1)] = hp.he[idx / (NP + 1)][idx % (NP + 1)];
-    for (int idx = threadIdx.x; idx < HO * NP; idx += blockDim.x) ho[(idx / NP) * CO + idx % NP] = hp.ho[idx / NP][idx % NP];
-    for (int idx = threadIdx.x; idx < HE; idx += blockDim.x) ae[idx] = hp.ae[idx];
-    for (int idx = threadIdx.x; idx < HO; idx += blockDim.x) ao[idx] = hp.ao[idx];
-  }
-};
-
-// Four consecutive coefficients of a 16-byte-aligned shared-memory row.
-template <class CT>
-__device__ __forceinline__ void load4(const CT* p, CT (&v)[4]) {
-  if constexpr (std::is_same<CT, float>::value) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-  } else {
-    const double2 a = *reinterpret_cast<const double2*>(p);
-    const double2 b = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-  }
-}
-
-// Rows of order >= 4 with their own rates: z_r = a_r sum_j h_r(c_j) f_j, a_r = -(s_r - s_h) / N_r,
-// kept in the table's per-thread slots. Even rows take f_+ + f_- of each +-e pair, odd rows
-// f_+ - f_- (h_r(-c) = +-h_r(c)). For deviation storage the reference state drops out (every
-// such row is W-orthogonal to H_0).
-template <class L, class CT>
-__device__ __forceinline__ void high_moments(const CT (&f)[L::Q], HighTable<L, CT>& tb) {
-  using T = HighTable<L, CT>;
-  constexpr int NP = T::NP;
-  CT sp[NP], sm[NP];
-  static_for<NP>([&](auto q) {
-    constexpr int P = decltype(q)::value;
-    constexpr int ip = pair_plus<L>(P);
-    constexpr int im = opposite<L>(ip);
-    sp[P] = f[ip] + f[im];
-    sm[P] = f[ip] - f[im];
-  });
-#pragma unroll 1
-  for (int r = 0; r < T::HE; ++r) {
-    const CT* h = tb.he + r * T::CE;
-    CT acc = CT(0);
-    static_for<T::CE / 4>([&](auto g) {
-      CT v[4];
-      load4(h + 4 * decltype(g)::value, v);
-      static_for<4>([&](auto j) {
-        constexpr int C = 4 * decltype(g)::value + decltype(j)::value;  // c = 0: rest, c = P + 1: pair P
-        if constexpr (C == 0) acc = fma(v[decltype(j)::value], f[0], acc);
-        else if constexpr (C <= NP) acc = fma(v[decltype(j)::value], sp[C - 1], acc);
-      });
-    });
-    tb.z[r * kBlock + threadIdx.x] = acc * tb.ae[r];
-  }
-#pragma unroll 1
-  for (int r = 0; r < T::HO; ++r) {
-    const CT* h = tb.ho + r * T::CO;
-    CT acc = CT(0);
-    static_for<T::CO / 4>([&](auto g) {
-      CT v[4];
-      load4(h + 4 * decltype(g)::value, v);
-      static_for<4>([&](auto j) {
-        constexpr int C = 4 * decltype(g)::value + decltype(j)::value;
-        if constexpr (C < NP) acc = fma(v[decltype(j)::value], sm[C], acc);
-      });
-    });
-    tb.z[(T::HE + r) * kBlock + threadIdx.x] = acc * tb.ao[r];
-  }
-}
-
-// f_i += w_i sum_r h_r(c_i) z_r over the rows of order >= 4 (the weights of a +-e pair are equal).
-template <class L, class CT, class P>
-__device__ __forceinline__ void high_back(CT (&f)[L::Q], const P& p, const HighTable<L, CT>& tb) {
-  using T = HighTable<L, CT>;
-  constexpr int NP = T::NP;
-  CT ev[NP + 1], od[NP];
-  static_for<NP + 1>([&](auto q) { ev[decltype(q)::value] = CT(0); });
-  static_for<NP>([&](auto q) { od[decltype(q)::value] = CT(0); });
-#pragma unroll 1
-  for (int r = 0; r < T::HE; ++r) {
-    const CT* h = tb.he + r * T::CE;
-    const CT zr = tb.z[r * kBlock + threadIdx.x];
-    static_for<T::CE / 4>([&](auto g) {
-      CT v[4];
-      load4(h + 4 * decltype(g)::value, v);
-      static_for<4>([&](auto j) {
-        constexpr int C = 4 * decltype(g)::value + decltype(j)::value;
-        if constexpr (C <= NP) ev[C] = fma(v[decltype(j)::value], zr, ev[C]);
-      });
-    });
-  }
-#pragma unroll 1
-  for (int r = 0; r < T::HO; ++r) {
-    const CT* h = tb.ho + r * T::CO;
-    const CT zr = tb.z[(T::HE + r) * kBlock + threadIdx.x];
-    static_for<T::CO / 4>([&](auto g) {
-      CT v[4];
-      load4(h + 4 * decltype(g)::value, v);
-      static_for<4>([&](auto j) {
-        constexpr int C = 4 * decltype(g)::value + decltype(j)::value;
-        if constexpr (C < NP) od[C] = fma(v[decltype(j)::value], zr, od[C]);
-      });
-    });
-  }
-  f[0] = fma(p.w[0], ev[0], f[0]);
-  static_for<NP>([&](auto q) {
-    constexpr int Pq = decltype(q)::value;
-    constexpr int ip = pair_plus<L>(Pq);
-    constexpr int im = opposite<L>(ip);
-    f[ip] = fma(p.w[ip], ev[Pq + 1] + od[Pq], f[ip]);
-    f[im] = fma(p.w[im], ev[Pq + 1] - od[Pq], f[im]);
-  });
-}
-
 // One collision (Eq. (2-3)) of the populations f of one cell, in place.
 // F: body force at the cell (NSE); phi_prev / phi_now: the NCDE field at t_{n-1} and t_n.
 // DEV: f holds deviations f - w rho_ref (16-bit storage). The moments of the reference state are
 // added back (only 1 and the squares c_a^2 have non-zero lattice moments), and the update
 // f* - w rho_ref = (1 - s_h)(f - w rho_ref) + w H(h) - s_h w rho_ref folds the last term into h_0.
-// HP = HighTable<L, CT>: the rows of order >= 4 relax with the rates in hp (the full Q x Q
-// collision); HP = NoHigh: they share s_high (the reduced form alone).
-struct NoHigh {};
 
 // The collision in moment space: from the raw moments mu_k = sum_i mono_k(e_i) f_i (k < R) to
 // the monomial-basis coefficients h of the update f*_i = (1 - s_h) f_i + w_i sum_k mono_k(e_i) h_k.
@@ -695,18 +563,14 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
 
 // KEEP = false: every row of order >= 4 relaxes with s_h = 1 (the default), so that f* depends on the
 // moments alone and the populations need not stay in registers through the collision.
-template <class L, class V, int EQ, bool DEV, bool KEEP, class HP = NoHigh>
+template <class L, class V, int EQ, bool DEV, bool KEEP>
 __device__ __forceinline__ void collide(V (&f)[L::Q], const LatTables<V>& lt, const Rates<V>& rt, bool forced,
-                                        const V (&F)[3], V phi_prev, V& phi_now, HP* hp = nullptr,
-                                        const V* gr = nullptr) {
-  constexpr bool HI = !std::is_same<HP, NoHigh>::value;
-  if constexpr (HI) high_moments<L>(f, *hp);
+                                        const V (&F)[3], V phi_prev, V& phi_now, const V* gr = nullptr) {
   V mu[L::R];
   raw_moments<L>(f, mu);
   V h[L::R];
   collide_moments<L, V, EQ, DEV>(mu, lt, rt, forced, F, phi_prev, phi_now, h, gr);
   back_project<L, KEEP>(f, lt, h, rt.one_minus_sh);
-  if constexpr (HI) high_back<L>(f, lt, *hp);
 }
 
 // Equilibrium populations of given fields, Eq. (feq-1): f^eq_i = w_i sum_r H_ri m^eq_r / N_r
@@ -740,6 +604,12 @@ __device__ __forceinline__ void equilibrium(V (&f)[L::Q], const LatTables<V>& lt
   rows_to_monomials<L>(lt, gN, h);
   back_project<L, false>(f, lt, h, V(0.f));
 }
+
+}  // namespace lbm
+
+#include "high.cuh"
+
+namespace lbm {
 
 // Cell coordinates and periodic neighbour offsets.
 template <class L>
@@ -887,7 +757,7 @@ __global__ void __launch_bounds__(kBlock, LBM_K1_MIN_BLOCKS) k_step(const StepPa
     CT gr[3];
     const CT* grad = nullptr;
     if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, nb.x, nb.y, nb.z, gr);
-    collide<L, CT, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
+    collide<L, CT, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, grad);
     if constexpr (EQ == LBM_NCDE) phi[cell] = phi_now;
     if constexpr (AG && EQ == LBM_NSE) {
       if (p.grad_on) p.rho_out[cell] = phi_now;
@@ -934,108 +804,141 @@ __device__ __forceinline__ uint32_t enc_word(float a, float b) {
 // 10.2 / 8.4, rD3Q53 256x256x192 FP32 776 / 759, rD3Q53 150x131x147 BF16 153 / 116, rD3Q45 101x103x97
 // FP32 62.8 / 59.2. 4 blocks per SM leave 128 registers; on rD3Q53 the single accesses spill at that, with 3
 // blocks 81^3 FP32 takes 39.0 us (one cell per thread 40.0) and 149x131x147 BF16 139 us (156).
-template <class L, class ST, int EQ, bool KEEP, bool EVEN>
-__global__ void __launch_bounds__(kBlock, KEEP && L::Q > 33 ? 2 : (L::Q > 45 && (!EVEN || is_deviation_storage<ST>()) ? 3 : 4))
-    k_step_pair(const StepParams<F2, float> p, const ST* fin, ST* fout, float* phi) {
+//
+// HI: with the operator of the higher rows (hc). FP32 storage waits for memory and takes one block per SM
+// more than fits without spills (which stay in L1); 16-bit storage is bound by issue, and its blocks stay
+// resident, so that each stages the operator once. us a step, without spills / with one block more: rD3Q53
+// 160x144x120 FP32 245 / 232, FP16 202 / 225; rD3Q45 205 / 175, 159 / 169; rD2Q25 1024x768 26.5 / 25.5, 21.5 /
+// 22.7. Blocks that stay resident: FP32 265 (245 with a block per 256 cells), FP16 202 (220). Also measured: the
+// sources of the next two cells copied to shared memory meanwhile (cp.async, 64 threads, 4 blocks per SM): 311.
+struct NoCoefs {};
+template <class L, class ST>
+constexpr int pair_high_blocks() {
+  return (L::Q > 33 ? 2 : (L::Q >= 27 ? 3 : 4)) + (is_deviation_storage<ST>() ? 0 : 1);
+}
+template <class L, class ST, bool KEEP, bool EVEN, bool HI>
+constexpr int pair_blocks() {
+  if (HI) return pair_high_blocks<L, ST>();
+  if (KEEP && L::Q > 33) return 2;
+  return L::Q > 45 && (!EVEN || is_deviation_storage<ST>()) ? 3 : 4;
+}
+template <class L, class ST, int EQ, bool KEEP, bool EVEN, bool HI = false>
+__global__ void __launch_bounds__(kBlock, pair_blocks<L, ST, KEEP, EVEN, HI>())
+    k_step_pair(const StepParams<F2, float> p, const std::conditional_t<HI, HighCoefs<float>, NoCoefs> hc, const ST* fin,
+                ST* fout, float* phi) {
   constexpr int Q = L::Q, RM = L::RMAX;
   constexpr bool DEV = is_deviation_storage<ST>();
+  __shared__ std::conditional_t<HI, HighCoefs<float>, NoCoefs> coefs;
+  if constexpr (HI) {
+    stage_coefs<L>(coefs, hc);
+    __syncthreads();
+  }
   chain_release_if(p.release, kReleaseFirst);
-  const int cell = 2 * (blockIdx.x * kBlock + threadIdx.x);
-  if (cell >= p.ncells) return;
   const size_t N = size_t(p.ncells);
-  const bool two = EVEN || cell + 1 < p.ncells;
-  const Neigh<L> n0(cell, p.n, p.div_m, p.div_s);
-  F2 f[Q];
-  auto one = [&](const ST* a) -> float {
-    if constexpr (DEV) return RawCodec<ST>::dec(k1_load(a));
-    else return k1_load(a);
-  };
-  int c0[3] = {n0.x, n0.y, n0.z}, c1[3] = {n0.x + 1, n0.y, n0.z};
-  if constexpr (EVEN) {
-    // x positions of the second cell's sources; the first cell's for e_x = -RM .. RM are n0.xo
-    int x1[2 * RM + 1];
-#pragma unroll
-    for (int sh = -RM; sh <= RM; ++sh) x1[sh + RM] = Neigh<L>::wrap1(n0.x + 1 - sh, sh == 0 ? 1 : sh, p.n[0]);
-    chain_wait();
-    chain_release_if(p.release, kReleaseAfterWait);
-    static_for<Q>([&](auto i) {
-      constexpr int I = decltype(i)::value;
-      constexpr Vel v = L::e(I);
-      const int yz = n0.yo[RM + v.y] + (L::D == 3 ? n0.zo[RM + v.z] : 0);
-      const ST* a = fin + size_t(I) * N + (n0.xo[RM + v.x] + yz);
-      if constexpr (v.x % 2 == 0) {
-        if constexpr (DEV) f[I] = dec_word<ST>(*reinterpret_cast<const uint32_t*>(a));
-        else f[I] = *reinterpret_cast<const F2*>(a);
-      } else {
-        f[I] = F2(one(a), one(fin + size_t(I) * N + (x1[RM + v.x] + yz)));
-      }
-    });
-  } else {
-    const Neigh<L> n1(two ? cell + 1 : cell, p.n, p.div_m, p.div_s);
-    c1[0] = n1.x;
-    c1[1] = n1.y;
-    c1[2] = n1.z;
-    chain_wait();
-    chain_release_if(p.release, kReleaseAfterWait);
-    static_for<Q>([&](auto i) {
-      constexpr int I = decltype(i)::value;
-      f[I] = F2(one(fin + size_t(I) * N + n0.template src<I>()), one(fin + size_t(I) * N + n1.template src<I>()));
-    });
-  }
-  F2 F[3];
-  const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, c0, c1, F);
-  F2 phi_prev(0.f), phi_now(0.f);
-  if constexpr (EQ == LBM_NCDE) {
-    if constexpr (EVEN) phi_prev = *reinterpret_cast<const F2*>(phi + cell);
-    else phi_prev = F2(phi[cell], phi[two ? cell + 1 : cell]);
-  }
-  constexpr bool AG = GradTerm<L, EQ>::kOn;
-  F2 gr[3];
-  const F2* grad = nullptr;
-  if constexpr (AG) {
-    if (two) {
-      grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, c0, c1, gr);
-    } else if (p.grad_on) {
-      float d[3];
-      field_differences<L>(p.n, p.grad_in, cell, c0[0], c0[1], c0[2], d);
-      static_for<L::D>([&](auto a) { gr[decltype(a)::value] = p.gscale[decltype(a)::value] * F2(d[decltype(a)::value]); });
-      grad = gr;
-    }
-  }
-  collide<L, F2, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
-  float a, b;
-  auto field_out = [&](float* g) {
+  auto step = [&](int cell) {
+    const bool two = EVEN || cell + 1 < p.ncells;
+    const Neigh<L> n0(cell, p.n, p.div_m, p.div_s);
+    F2 f[Q];
+    auto one = [&](const ST* a) -> float {
+      if constexpr (DEV) return RawCodec<ST>::dec(k1_load(a));
+      else return k1_load(a);
+    };
+    int c0[3] = {n0.x, n0.y, n0.z}, c1[3] = {n0.x + 1, n0.y, n0.z};
     if constexpr (EVEN) {
-      *reinterpret_cast<F2*>(g + cell) = phi_now;
+      // x positions of the second cell's sources; the first cell's for e_x = -RM .. RM are n0.xo
+      int x1[2 * RM + 1];
+#pragma unroll
+      for (int sh = -RM; sh <= RM; ++sh) x1[sh + RM] = Neigh<L>::wrap1(n0.x + 1 - sh, sh == 0 ? 1 : sh, p.n[0]);
+      chain_wait();
+      chain_release_if(p.release, kReleaseAfterWait);
+      static_for<Q>([&](auto i) {
+        constexpr int I = decltype(i)::value;
+        constexpr Vel v = L::e(I);
+        const int yz = n0.yo[RM + v.y] + (L::D == 3 ? n0.zo[RM + v.z] : 0);
+        const ST* a = fin + size_t(I) * N + (n0.xo[RM + v.x] + yz);
+        if constexpr (v.x % 2 == 0) {
+          if constexpr (DEV) f[I] = dec_word<ST>(*reinterpret_cast<const uint32_t*>(a));
+          else f[I] = *reinterpret_cast<const F2*>(a);
+        } else {
+          f[I] = F2(one(a), one(fin + size_t(I) * N + (x1[RM + v.x] + yz)));
+        }
+      });
     } else {
-      phi_now.get(a, b);
-      g[cell] = a;
-      if (two) g[cell + 1] = b;
+      const Neigh<L> n1(two ? cell + 1 : cell, p.n, p.div_m, p.div_s);
+      c1[0] = n1.x;
+      c1[1] = n1.y;
+      c1[2] = n1.z;
+      chain_wait();
+      chain_release_if(p.release, kReleaseAfterWait);
+      static_for<Q>([&](auto i) {
+        constexpr int I = decltype(i)::value;
+        f[I] = F2(one(fin + size_t(I) * N + n0.template src<I>()), one(fin + size_t(I) * N + n1.template src<I>()));
+      });
     }
-  };
-  if constexpr (EQ == LBM_NCDE) field_out(phi);
-  if constexpr (AG && EQ == LBM_NSE) {
-    if (p.grad_on) field_out(p.rho_out);
-  }
-  chain_release_if(p.release, kReleaseLast);
-  static_for<Q>([&](auto i) {
-    constexpr int I = decltype(i)::value;
-    ST* o = fout + size_t(I) * N + cell;
-    if constexpr (EVEN && !DEV) {
-      *reinterpret_cast<F2*>(o) = f[I];
-    } else {
-      f[I].get(a, b);
-      if constexpr (EVEN) {
-        *reinterpret_cast<uint32_t*>(o) = enc_word<ST>(a, b);
-      } else if constexpr (DEV) {
-        k1_store(o, RawCodec<ST>::enc(a));
-        if (two) k1_store(o + 1, RawCodec<ST>::enc(b));
-      } else {
-        k1_store(o, a);
-        if (two) k1_store(o + 1, b);
+    F2 F[3];
+    const bool forced = body_force(p.force_a, p.force_b, p.force_tab, p.invc, c0, c1, F);
+    F2 phi_prev(0.f), phi_now(0.f);
+    if constexpr (EQ == LBM_NCDE) {
+      if constexpr (EVEN) phi_prev = *reinterpret_cast<const F2*>(phi + cell);
+      else phi_prev = F2(phi[cell], phi[two ? cell + 1 : cell]);
+    }
+    constexpr bool AG = GradTerm<L, EQ>::kOn;
+    F2 gr[3];
+    const F2* grad = nullptr;
+    if constexpr (AG) {
+      if (two) {
+        grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, c0, c1, gr);
+      } else if (p.grad_on) {
+        float d[3];
+        field_differences<L>(p.n, p.grad_in, cell, c0[0], c0[1], c0[2], d);
+        static_for<L::D>([&](auto a) { gr[decltype(a)::value] = p.gscale[decltype(a)::value] * F2(d[decltype(a)::value]); });
+        grad = gr;
       }
     }
-  });
+    if constexpr (HI) collide_high<L, F2, EQ, DEV>(f, coefs.c, p, p, forced, F, phi_prev, phi_now, grad);
+    else collide<L, F2, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, grad);
+    float a, b;
+    auto field_out = [&](float* g) {
+      if constexpr (EVEN) {
+        *reinterpret_cast<F2*>(g + cell) = phi_now;
+      } else {
+        phi_now.get(a, b);
+        g[cell] = a;
+        if (two) g[cell + 1] = b;
+      }
+    };
+    if constexpr (EQ == LBM_NCDE) field_out(phi);
+    if constexpr (AG && EQ == LBM_NSE) {
+      if (p.grad_on) field_out(p.rho_out);
+    }
+    chain_release_if(p.release, kReleaseLast);
+    static_for<Q>([&](auto i) {
+      constexpr int I = decltype(i)::value;
+      ST* o = fout + size_t(I) * N + cell;
+      if constexpr (EVEN && !DEV) {
+        *reinterpret_cast<F2*>(o) = f[I];
+      } else {
+        f[I].get(a, b);
+        if constexpr (EVEN) {
+          *reinterpret_cast<uint32_t*>(o) = enc_word<ST>(a, b);
+        } else if constexpr (DEV) {
+          k1_store(o, RawCodec<ST>::enc(a));
+          if (two) k1_store(o + 1, RawCodec<ST>::enc(b));
+        } else {
+          k1_store(o, a);
+          if (two) k1_store(o + 1, b);
+        }
+      }
+    });
+  };
+  const int first = 2 * (blockIdx.x * kBlock + threadIdx.x);
+  if constexpr (HI && DEV) {
+    // (as many blocks as are resident: the operator is staged once by each)
+    const int64_t stride = int64_t(2) * kBlock * gridDim.x;
+    for (int64_t cell = first; cell < p.ncells; cell += stride) step(int(cell));
+  } else {
+    if (first < p.ncells) step(first);
+  }
 }
 
 // K1 on a small 2D grid in FP64, four threads per cell. GB300 runs one FP64 warp instruction per 64
@@ -1126,15 +1029,15 @@ __global__ void __launch_bounds__(128) k_step_split(const StepParams<double> p, 
   }
 }
 
-// K1 with distinct rates for the orders >= 4: the same gather / collide / store plus the two
-// contractions with the higher rows (about 2 (Q - 1) (Q - R) / 2 more FMAs per cell, so the
-// kernel is bound by instruction issue rather than HBM; 3 resident blocks leave it 168 registers).
+// K1 with distinct rates for the orders >= 4: the same gather / collide / store with the operator of the
+// higher rows (high.cuh), one cell per thread. Bound by issue and by too few warps to hide the loads: us a
+// step of rD3Q53 160x144x120 FP32 with 3 / 4 / 5 blocks per SM 270 / 241 / 246 (4: 128 registers, 20 bytes
+// spilled); the rows' two contractions instead of the operator took 555 (2.45 ms on 256x256x192).
 template <class L, class CT, class ST, int EQ>
-__global__ void __launch_bounds__(kBlock, 3) k_step_high(const StepParams<CT> p,
-                                                          const HighParams<CT> hp, const ST* fin, ST* fout,
-                                                          CT* phi) {
-  __shared__ HighTable<L, CT> tab;
-  tab.fill(hp);
+__global__ void __launch_bounds__(kBlock, std::is_same<CT, double>::value ? 2 : 4)
+    k_step_high(const StepParams<CT> p, const HighCoefs<CT> hc, const ST* fin, ST* fout, CT* phi) {
+  __shared__ HighCoefs<CT> coefs;
+  stage_coefs<L>(coefs, hc);
   __syncthreads();
   const int cell = blockIdx.x * kBlock + threadIdx.x;
   if (cell >= p.ncells) return;
@@ -1157,7 +1060,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_step_high(const StepParams<CT> p,
   CT gr[3];
   const CT* grad = nullptr;
   if constexpr (AG) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, nb.x, nb.y, nb.z, gr);
-  collide<L, CT, EQ, DEV, true>(f, p, p, forced, F, phi_prev, phi_now, &tab, grad);
+  collide_high<L, CT, EQ, DEV>(f, coefs.c, p, p, forced, F, phi_prev, phi_now, grad);
   if constexpr (EQ == LBM_NCDE) phi[cell] = phi_now;
   if constexpr (AG && EQ == LBM_NSE) {
     if (p.grad_on) p.rho_out[cell] = phi_now;
@@ -1206,10 +1109,10 @@ constexpr int batch_min_blocks() {
 }
 
 // One cell of a batched step: the same gather / collide / store as k_step, with the solve's
-// parameters from its staged descriptor (HP: the higher-row table of a per-order-rate group).
-template <class L, class CT, class ST, int EQ, bool KEEP, class HP>
+// parameters from its staged descriptor (HI: hc, the staged operator of a per-order-rate group).
+template <class L, class CT, class ST, int EQ, bool KEEP, bool HI>
 __device__ __forceinline__ void batch_cell(const LatTables<CT>& t, const SolveDesc<CT>& sd, int cell, int parity,
-                                           HP* hp) {
+                                           const CT* hc) {
   const Neigh<L> nb(cell, sd.n, sd.div_m, sd.div_s);
   const size_t N = size_t(sd.ncells);
   const ST* fin = static_cast<const ST*>(sd.f[parity]);
@@ -1229,7 +1132,8 @@ __device__ __forceinline__ void batch_cell(const LatTables<CT>& t, const SolveDe
   CT gr[3];
   const CT* grad = nullptr;
   if constexpr (AG) grad = cell_field_gradient<L>(sd, sd.n, sd.grad_in[parity], cell, nb.x, nb.y, nb.z, gr);
-  collide<L, CT, EQ, DEV, KEEP>(f, t, sd, forced, F, phi_prev, phi_now, hp, grad);
+  if constexpr (HI) collide_high<L, CT, EQ, DEV>(f, hc, t, sd, forced, F, phi_prev, phi_now, grad);
+  else collide<L, CT, EQ, DEV, KEEP>(f, t, sd, forced, F, phi_prev, phi_now, grad);
   if constexpr (EQ == LBM_NCDE) sd.phi[cell] = phi_now;
   if constexpr (AG && EQ == LBM_NSE) {
     if (sd.grad_on) sd.rho_out[parity][cell] = phi_now;
@@ -1268,19 +1172,18 @@ __global__ void __launch_bounds__(BLOCK, batch_min_blocks<BLOCK>())
     }
     const int cell = tile.cell0 + int(threadIdx.x);
     if (cell >= sd.ncells) continue;
-    batch_cell<L, CT, ST, EQ, KEEP>(t, sd, cell, parity, static_cast<NoHigh*>(nullptr));
+    batch_cell<L, CT, ST, EQ, KEEP, false>(t, sd, cell, parity, nullptr);
   }
 }
 
 // The batched step of a group whose solves have one rate per order >= 4: tiles of kBlock cells,
-// and the solve's higher-row table (rows of the lattice, rates of the solve) staged in shared
-// memory with its descriptor, as k_step_high does for one solve.
+// and the solve's operator of the higher rows staged in shared memory with its descriptor.
 template <class L, class CT, class ST, int EQ>
 __global__ void __launch_bounds__(kBlock, 3)
-    k_step_batch_high(const LatTables<CT> t, const SolveDesc<CT>* descs, const HighParams<CT>* highs,
+    k_step_batch_high(const LatTables<CT> t, const SolveDesc<CT>* descs, const HighCoefs<CT>* highs,
                       const Tile* tiles, int ntiles, int parity) {
   __shared__ SolveDesc<CT> sd;
-  __shared__ HighTable<L, CT> tab;
+  __shared__ HighCoefs<CT> coefs;
   chain_wait();
   int staged = -1;
   for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
@@ -1288,13 +1191,13 @@ __global__ void __launch_bounds__(kBlock, 3)
     if (tile.solve != staged) {
       __syncthreads();
       stage_desc<CT, kBlock>(sd, descs, tile.solve);
-      tab.fill(highs[tile.solve]);
+      stage_coefs<L>(coefs, highs[tile.solve]);
       __syncthreads();
       staged = tile.solve;
     }
     const int cell = tile.cell0 + int(threadIdx.x);
     if (cell >= sd.ncells) continue;
-    batch_cell<L, CT, ST, EQ, true>(t, sd, cell, parity, &tab);
+    batch_cell<L, CT, ST, EQ, true, true>(t, sd, cell, parity, coefs.c);
   }
 }
 
@@ -1362,7 +1265,7 @@ lbm_status BatchLaunch<KIND>::launch(const BatchGroup& g, int parity, cudaStream
       const LatTables<float>& t = *static_cast<const LatTables<float>*>(g.tables);
       cudaError_t err = launch_chained(kernel, g.grid, kBlock, 0, stream, t,
                                        static_cast<const SolveDesc<float>*>(g.d_desc),
-                                       static_cast<const HighParams<float>*>(g.d_high), g.d_tiles, g.ntiles, parity);
+                                       static_cast<const HighCoefs<float>*>(g.d_high), g.d_tiles, g.ntiles, parity);
       return err == cudaSuccess ? LBM_OK : cuda_error(err, "batched step launch");
     });
   }
@@ -1402,11 +1305,19 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
   const int grid = (m->ncells + kBlock - 1) / kBlock;
   CT* phi = static_cast<CT*>(m->phi_prev);
   const bool high = collide_on && has_high_rates(m);
-  HighParams<CT> hp;
-  if (high) make_high_params<CT>(m, &hp);
-  // tcgen05 when asked for, and by default with per-order rates (where the dense higher rows make
-  // it the faster kernel); on FP32 storage only the higher rows go to the tensor cores
-  [[maybe_unused]] const bool tensor = collide_on && (m->tensor_cores || (m->tc_auto && high));
+  // tcgen05 when asked for (on FP32 storage only the higher rows go to the tensor cores), and for per-order
+  // rates with a forced row-staged gather, which has no other form, or where the row-staged tcgen05 kernel
+  // is the faster one: its blocks of 256 threads need nearly full rows, many of them per block, and a
+  // lattice of many rows. us a step in FP16, CUDA cores / tcgen05: rD3Q53 256x128x96 227 / 214, 256x64x64
+  // 80 / 86, 192x96x96 130 / 158, 160x144x120 201 / 267; rD3Q45 256x128x96 180 / 185.
+  [[maybe_unused]] bool tensor =
+      collide_on && (m->tensor_cores || (m->tc_auto && high && m->gather == LBM_GATHER_ROWS));
+  if constexpr (is_deviation_storage<ST>() && L::Q > 45) {
+    RowPlan wide;
+    if (high && !tensor && m->tc_auto && m->gather == LBM_GATHER_AUTO && m->n[0] >= 240 &&
+        m->ncells / m->n[0] >= 64 * sm_count(m->device))
+      tensor = RowLaunch<L::KIND>::plan(m, &wide, true, true);
+  }
   [[maybe_unused]] const bool tensor32 = std::is_same<ST, float>::value && tensor && high;
   TcParams tp;
   [[maybe_unused]] Tc32Params tp32;
@@ -1490,10 +1401,14 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       if (nsteps == 0) return LBM_OK;
     }
   }
-  // two cells per thread where the halved thread count still fills the GPU
-  [[maybe_unused]] const bool pairs = !std::is_same<CT, double>::value && collide_on && !high && !tensor && !rows &&
-                                      m->ncells >= kPairCells;
+  // two cells per thread where the halved thread count still fills the GPU (with the higher rows' operator
+  // not on ragged FP32 grids of the largest lattice: rD3Q53 101x103x97 99 us a step against 94 with one)
+  [[maybe_unused]] const bool pairs = !std::is_same<CT, double>::value && collide_on && !tensor && !rows &&
+                                      m->ncells >= kPairCells &&
+                                      !(high && L::Q > 45 && std::is_same<ST, float>::value && m->n[0] % 2 != 0);
   if (pairs) make_step_params(m, &p2);
+  HighCoefs<CT> hc;
+  if (high && !tensor) make_high_coefs(m, &hc);
   const int grid2 = (m->ncells / 2 + m->ncells % 2 + kBlock - 1) / kBlock;
   // FP64 on a small 2D grid: four threads per cell while every block of 32 cells has an SM of its own. Us per
   // step, one thread per cell against four (a first version): 80x60 cells, 150 blocks, rD2Q13 6.4 / 5.2, rD2Q25
@@ -1519,7 +1434,7 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
     }
     cudaError_t err = cudaSuccess;
     auto go = [&](auto kernel, int blocks, int threads, size_t smem, const auto&... args) {
-      if (release < 0) release = release_point(kernel, blocks, threads, m->device);
+      if (release < 0) release = release_point(kernel, blocks, threads, smem, m->device);
       p.release = p2.release = release;
       err = launch_chained(kernel, blocks, threads, smem, m->stream, args..., fin, fout, phi);
     };
@@ -1549,18 +1464,25 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
     }
     if constexpr (!std::is_same<CT, double>::value) {
       if (pairs) {
-        auto pick = [&](auto eq, auto keep) {
+        auto pick = [&](auto eq, auto even) {
           constexpr int E = decltype(eq)::value;
-          constexpr bool K = decltype(keep)::value;
-          if (m->n[0] % 2 == 0) go(k_step_pair<L, ST, E, K, true>, grid2, kBlock, 0, p2);
-          else go(k_step_pair<L, ST, E, K, false>, grid2, kBlock, 0, p2);
+          constexpr bool EV = decltype(even)::value;
+          if (high) {
+            go(k_step_pair<L, ST, E, true, EV, true>,
+               is_deviation_storage<ST>() ? std::min(grid2, sm_count(m->device) * pair_high_blocks<L, ST>()) : grid2, kBlock, 0,
+               p2, hc);
+          } else if (m->s_high == 1.0) {
+            go(k_step_pair<L, ST, E, false, EV>, grid2, kBlock, 0, p2, NoCoefs{});
+          } else {
+            go(k_step_pair<L, ST, E, true, EV>, grid2, kBlock, 0, p2, NoCoefs{});
+          }
         };
-        auto by_keep = [&](auto eq) {
-          if (m->s_high == 1.0) pick(eq, std::false_type{});
-          else pick(eq, std::true_type{});
+        auto by_even = [&](auto eq) {
+          if (m->n[0] % 2 == 0) pick(eq, std::true_type{});
+          else pick(eq, std::false_type{});
         };
-        if (m->eq == LBM_NSE) by_keep(std::integral_constant<int, LBM_NSE>{});
-        else by_keep(std::integral_constant<int, LBM_NCDE>{});
+        if (m->eq == LBM_NSE) by_even(std::integral_constant<int, LBM_NSE>{});
+        else by_even(std::integral_constant<int, LBM_NCDE>{});
         done = true;
       }
     }
@@ -1578,8 +1500,8 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
     }
     if (done) {
     } else if (high) {
-      if (m->eq == LBM_NSE) go(k_step_high<L, CT, ST, LBM_NSE>, grid, kBlock, 0, p, hp);
-      else go(k_step_high<L, CT, ST, LBM_NCDE>, grid, kBlock, 0, p, hp);
+      if (m->eq == LBM_NSE) go(k_step_high<L, CT, ST, LBM_NSE>, grid, kBlock, 0, p, hc);
+      else go(k_step_high<L, CT, ST, LBM_NCDE>, grid, kBlock, 0, p, hc);
     } else if (!collide_on) {
       go(k_step<L, CT, ST, LBM_NSE, false, true>, grid, kBlock, 0, p);
     } else if (m->eq == LBM_NSE) {

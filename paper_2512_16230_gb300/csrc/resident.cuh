@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
       float gr[3];
       const float* grad = nullptr;
       if constexpr (EQ == LBM_NCDE) grad = cell_field_gradient<L>(p, p.n, p.grad_in, int(g0) + c, x, y, 0, gr);
-      collide<L, float, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
+      collide<L, float, EQ, DEV, KEEP>(f, p, p, forced, F, phi_prev, phi_now, grad);
       if constexpr (EQ == LBM_NCDE) s_phi[c] = phi_now;
       static_for<Q>([&](auto i) {
         constexpr int I = decltype(i)::value;

@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(128, Tc32Shape<L>::CTAS)
     if constexpr (AG) {
       if (live) grad = cell_field_gradient<L>(p, p.n, p.grad_in, cell, x, y, z, gr);
     }
-    collide<L, float, EQ, false, true>(f, p, p, forced, F, phi_prev, phi_now, static_cast<NoHigh*>(nullptr), grad);
+    collide<L, float, EQ, false, true>(f, p, p, forced, F, phi_prev, phi_now, grad);
     if constexpr (EQ == LBM_NCDE) {
       if (live) phi[cell] = phi_now;
     }

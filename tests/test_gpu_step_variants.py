@@ -195,3 +195,47 @@ def test_fp64_small_grid_is_the_large_one_periodically(name, eq, s_high):
         out.append(m.get_populations())
         m.close()
     assert np.array_equal(np.tile(out[0], (1, 1, copies)), out[1])
+
+
+# one rate per order >= 4: two cells per thread against one (the batch), and FP64, whose blocks are the same
+@pytest.mark.parametrize("store", ["f32", "f16_dev"])
+@pytest.mark.parametrize("name,n", [("rD2Q25", (322, 250)), ("rD2Q17", (287, 283)), ("rD3Q27", (46, 43, 41)),
+                                    ("rD3Q33", (45, 43, 43)), ("rD3Q53", (46, 43, 41)), ("rD3Q45", (45, 43, 43)),
+                                    ("rD3Q53", (45, 43, 43))])
+def test_order_rates_two_cells_per_thread(name, n, store):
+    spec = W.LATTICES[name]
+    f0 = _populations(spec, n, 13, "nse")
+    kw = dict(store=store, s_orders={4: 0.8, 5: 1.35, 6: 1.6, 7: 0.9, 8: 1.25}, **_kwargs("nse", spec.d, 1.2))
+    m = gpu_model(spec, "nse", n, _rates(spec), **kw)
+    m.set_populations(f0)
+    m.step(2)
+    one = m.get_populations()
+    m.close()
+    assert np.array_equal(one, _batched(spec, "nse", n, f0, 2, **kw))
+    if store == "f32":
+        m = gpu_model(spec, "nse", n, _rates(spec), **dict(kw, store="f64"))
+        m.set_populations(f0)
+        m.step(2)
+        ref = m.get_populations()
+        m.close()
+        # two roundings of the populations to FP32 and some 40 in sums of the collision, each 2^-24 of the largest
+        assert np.abs(one - ref).max() <= 2 * 42 * 2.0 ** -24 * np.abs(ref).max()
+
+
+# wide, many rows: the row-staged tcgen05 kernel is the default; one row fewer than it asks for: the CUDA cores
+@pytest.mark.parametrize("fewer", [0, 1])
+def test_order_rates_default_on_wide_rows(fewer):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    spec, n = W.LATTICES["rD3Q53"], (240, sms - fewer, 64)
+    rho, u = np.ones(tuple(reversed(n))), np.random.default_rng(14).uniform(-0.02, 0.02, size=(3,) + tuple(reversed(n)))
+    out = []
+    for mode in (None, 1 - fewer, fewer):
+        m = gpu_model(spec, "nse", n, _rates(spec), store="f16_dev", s_high=1.2, s_orders={4: 0.8, 5: 1.35, 8: 1.25})
+        if mode is not None:
+            m.set_tensor_cores(mode)
+        m.init_fields(rho, u)
+        m.step(2)
+        out.append(m.read_fields()[1])
+        m.close()
+    assert np.array_equal(out[0], out[1]) and not np.array_equal(out[0], out[2])
