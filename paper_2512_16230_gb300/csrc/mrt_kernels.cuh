@@ -822,7 +822,7 @@ constexpr int pair_blocks() {
   if (KEEP && L::Q > 33) return 2;
   return L::Q > 45 && (!EVEN || is_deviation_storage<ST>()) ? 3 : 4;
 }
-template <class L, class ST, int EQ, bool KEEP, bool EVEN, bool HI = false>
+template <class L, class ST, int EQ, bool KEEP, bool EVEN, bool HI = false, bool LATE = false>
 __global__ void __launch_bounds__(kBlock, pair_blocks<L, ST, KEEP, EVEN, HI>())
     k_step_pair(const StepParams<F2, float> p, const std::conditional_t<HI, HighCoefs<float>, NoCoefs> hc, const ST* fin,
                 ST* fout, float* phi) {
@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(kBlock, pair_blocks<L, ST, KEEP, EVEN, HI>())
     stage_coefs<L>(coefs, hc);
     __syncthreads();
   }
-  chain_release_if(p.release, kReleaseFirst);
+  if constexpr (!LATE && EVEN) chain_release();
   const size_t N = size_t(p.ncells);
   auto step = [&](int cell) {
     const bool two = EVEN || cell + 1 < p.ncells;
@@ -850,7 +850,6 @@ __global__ void __launch_bounds__(kBlock, pair_blocks<L, ST, KEEP, EVEN, HI>())
 #pragma unroll
       for (int sh = -RM; sh <= RM; ++sh) x1[sh + RM] = Neigh<L>::wrap1(n0.x + 1 - sh, sh == 0 ? 1 : sh, p.n[0]);
       chain_wait();
-      chain_release_if(p.release, kReleaseAfterWait);
       static_for<Q>([&](auto i) {
         constexpr int I = decltype(i)::value;
         constexpr Vel v = L::e(I);
@@ -869,7 +868,7 @@ __global__ void __launch_bounds__(kBlock, pair_blocks<L, ST, KEEP, EVEN, HI>())
       c1[1] = n1.y;
       c1[2] = n1.z;
       chain_wait();
-      chain_release_if(p.release, kReleaseAfterWait);
+      if constexpr (!LATE) chain_release();
       static_for<Q>([&](auto i) {
         constexpr int I = decltype(i)::value;
         f[I] = F2(one(fin + size_t(I) * N + n0.template src<I>()), one(fin + size_t(I) * N + n1.template src<I>()));
@@ -911,7 +910,7 @@ __global__ void __launch_bounds__(kBlock, pair_blocks<L, ST, KEEP, EVEN, HI>())
     if constexpr (AG && EQ == LBM_NSE) {
       if (p.grad_on) field_out(p.rho_out);
     }
-    chain_release_if(p.release, kReleaseLast);
+    if constexpr (LATE) chain_release();
     static_for<Q>([&](auto i) {
       constexpr int I = decltype(i)::value;
       ST* o = fout + size_t(I) * N + cell;
@@ -1296,6 +1295,12 @@ lbm_status BatchLaunch<KIND>::occupancy(const BatchGroup& g, int* blocks_per_sm)
 // short of warps (us a step, one cell / two cells per thread: rD2Q21 256x200 2.44 / 2.61, 333x301 4.16 /
 // 3.77; rD3Q45 36^3 5.6 / 6.3, 45^3 6.6 / 5.9, 64^3 14.0 / 11.4).
 constexpr int kPairCells = 80000;
+// Cells below which the two-cell kernel releases the next launch before its stores (few waves: a block of the
+// next step takes a free place while others of this one end), and above which at its start (ragged grids: once
+// the wait is over, where the second cell's indices are ready). us a step,
+// rD3Q33 64^3 8.4 at the start of every block (8.9 with the point picked at run time), rD3Q53 150x131x147 BF16
+// 110.8 (114.8), rD2Q25 512x384 before the stores 5.3 (5.4).
+constexpr int kPairLateCells = 200000;
 
 // Host launchers for one lattice kind (instantiated in k_<lattice>.cu).
 template <class L, class CT, class ST>
@@ -1471,6 +1476,8 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
             go(k_step_pair<L, ST, E, true, EV, true>,
                is_deviation_storage<ST>() ? std::min(grid2, sm_count(m->device) * pair_high_blocks<L, ST>()) : grid2, kBlock, 0,
                p2, hc);
+          } else if (m->s_high == 1.0 && m->ncells < kPairLateCells) {
+            go(k_step_pair<L, ST, E, false, EV, false, true>, grid2, kBlock, 0, p2, NoCoefs{});
           } else if (m->s_high == 1.0) {
             go(k_step_pair<L, ST, E, false, EV>, grid2, kBlock, 0, p2, NoCoefs{});
           } else {
