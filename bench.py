@@ -38,11 +38,13 @@ GRID = (256, 256, 192)
 Q = 53
 # DRAM traffic of the benchmark kernel per cell update, from an ncu capture of the same workload on
 # 256 x 256 x 96 cells (half the grid: 2.7 GB on the device), scaled to the benchmark grid by cells
-PROFILE = os.path.join(ROOT, "profiles", "k_step_rd3q53_f32_tgv3d_256x256x96.md")
+PROFILE = os.path.join(ROOT, "profiles", "k_step_pair_rd3q53_f32_tgv3d_256x256x96.md")
 # the sources the benchmark kernel is compiled from (the traffic figure is void once their code,
 # comments aside, changes)
 KERNEL_SOURCES = ("include/lbm_mrt.h", "paper_2512_16230_gb300/csrc/lattices.cuh",
                   "paper_2512_16230_gb300/csrc/lbm_internal.cuh", "paper_2512_16230_gb300/csrc/mrt_kernels.cuh",
+                  "paper_2512_16230_gb300/csrc/f32x2.cuh", "paper_2512_16230_gb300/csrc/high.cuh",
+                  "paper_2512_16230_gb300/csrc/io_kernels.cuh", "paper_2512_16230_gb300/csrc/resident.cuh",
                   "paper_2512_16230_gb300/csrc/tc_kernels.cuh", "paper_2512_16230_gb300/csrc/tcgen05.cuh",
                   "paper_2512_16230_gb300/csrc/k_rd3q53.cu")
 CPU_SAMPLE_GRID = (256, 256, 16)    # cpu_baseline: ~10-30 s of oracle work on the GPU machine
@@ -110,10 +112,11 @@ def _profile_traffic(cells):
 def _kernel_name(args, grid):
     """The collide-stream kernel the library runs for this storage and grid."""
     rows = args.store != "f32" and grid[0] % 8 == 0 and grid[0] <= 256
+    threads = "k_step_pair" if math.prod(grid) >= 80000 else "k_step"  # two cells per thread or one
     if args.store == "f32":
-        return "k_step<rD3Q53, f32, NSE>"
+        return f"{threads}<rD3Q53, f32, NSE>"
     base = ("k_step_rows_tc" if args.tensor_cores else "k_step_rows") if rows else \
-        ("k_step_tc" if args.tensor_cores else "k_step")
+        ("k_step_tc" if args.tensor_cores else threads)
     return f"{base}<rD3Q53, {args.store}, NSE>"
 
 
@@ -447,7 +450,7 @@ def bench_ours(args):
     io_bytes = (rho_h.numel() + u_h.numel()) * 8
 
     # the full Q x Q collision with one rate per order >= 4 on the same solve: the CUDA-core
-    # kernel with explicit higher rows (k_step_high), then the higher rows on tcgen05
+    # kernel with the higher rows' block-diagonal operator, then the higher rows on tcgen05
     model.set_high_rates([HIGH_RATES[k] for k in sorted(HIGH_RATES)])
     vsteps = min(args.steps, VARIANT_STEPS)
     v0 = torch.cuda.Event(enable_timing=True)
@@ -497,7 +500,7 @@ def bench_ours(args):
             "mass_sum": float(sums[0]),
             "variants": {
                 "high_order_rates": {
-                    "kernel": "k_step_high<rD3Q53, f32, NSE> (explicit rows of order >= 4, one rate per order)",
+                    "kernel": "k_step_pair<rD3Q53, f32, NSE, higher rows> (block-diagonal operator of the rows of order >= 4)",
                     "rates": {str(k): v for k, v in HIGH_RATES.items()}, "steps": vsteps,
                     "ms_per_step": high_ms, "mlups": cells / high_ms / 1e3,
                     "hbm_frac": algo_bytes / (high_ms / 1e3) / 1e9 / peak},
@@ -514,16 +517,24 @@ def bench_ours(args):
     model.close()
     del model
     torch.cuda.empty_cache()
-    # the same variant with FP16-deviation storage, where its dense higher rows run on tcgen05
+    # the same variant with FP16-deviation storage: on tcgen05 with dense higher rows, and on the CUDA cores
     m16 = lbm.Model(lat, "nse", wl.n, store="f16_dev", stream=stream.cuda_stream)
     m16.set_relaxation(wl.s, wl.s_high)
     m16.set_high_rates([HIGH_RATES[k] for k in sorted(HIGH_RATES)])
     m16.init_fields(rho_d, u_d)
+    m16.set_tensor_cores(0)
+    high16_cc_ms = time_steps(m16)
+    m16.set_tensor_cores(1)
     high16_ms = time_steps(m16)
     m16.close()
     del m16
     torch.cuda.empty_cache()
     if rank == 0:
+        line["variants"]["high_order_rates_f16"] = {
+            "kernel": "k_step_pair<rD3Q53, f16_dev, NSE, higher rows> (block-diagonal operator)",
+            "rates": {str(k): v for k, v in HIGH_RATES.items()}, "steps": vsteps,
+            "ms_per_step": high16_cc_ms, "mlups": cells / high16_cc_ms / 1e3,
+            "hbm_frac": 2 * Q * 2 * cells / (high16_cc_ms / 1e3) / 1e9 / peak}
         line["variants"]["high_order_rates_f16_tensor_cores"] = {
             "kernel": "k_step_rows_tc<rD3Q53, f16_dev, NSE, higher rows> (row-staged, tcgen05 products with the "
                       "dense higher rows)",
@@ -537,7 +548,7 @@ def bench_ours(args):
              "k_step_rows<rD3Q53, f16_dev, NSE> (source x-rows staged in shared memory by cp.async)"),
             ("bf16_deviations", "bf16_dev", 0, "auto", "k_step_rows<rD3Q53, bf16_dev, NSE>"),
             ("f16_deviations_thread_gather", "f16_dev", 0, "threads",
-             "k_step<rD3Q53, f16_dev, NSE> (per-thread gather from global memory)"),
+             "k_step_pair<rD3Q53, f16_dev, NSE> (per-thread gather from global memory)"),
             ("f16_deviations_tensor_cores", "f16_dev", 1, "auto",
              "k_step_rows_tc<rD3Q53, f16_dev, NSE> (row-staged, contractions on tcgen05)"),
             ("f16_deviations_tensor_cores_thread_gather", "f16_dev", 1, "threads",
