@@ -90,7 +90,7 @@ typedef enum {
 
 /* How the CUDA-core collide-stream kernel of 16-bit storage gathers the pull sources. */
 typedef enum {
-  LBM_GATHER_AUTO = 0,    /* rows when they apply (default), threads otherwise                 */
+  LBM_GATHER_AUTO = 0,    /* the faster one (default): rows on the tensor cores, else threads */
   LBM_GATHER_THREADS = 1, /* every thread loads its Q sources from global memory               */
   LBM_GATHER_ROWS = 2     /* bulk copies of whole source x-rows into shared memory             */
 } lbm_gather;
@@ -234,13 +234,13 @@ lbm_status lbm_model_set_tensor_cores(lbm_model* m, int enable);
  * (the reduced-form collision and lbm_model_stream_only). ROWS: a CTA works on whole x-rows; the
  * source x-row (y - e_y, z - e_z) of each population comes into a shared-memory row buffer by
  * 16-byte asynchronous copies (n_x * 2 bytes per population, counted on an mbarrier, a few rows
- * ahead), every thread reads its sources there at (x - e_x) mod n_x, writes its collided cell
- * back into the buffer, and the row goes to memory by 16-byte stores. It applies when n_x is a
- * multiple of 8 (16-byte rows) and at most 256 cells. THREADS: every thread loads and stores its own cell's
- * populations in global memory. Both give bitwise the same populations.
+ * ahead), and every thread reads the sources of its cells there at (x - e_x) mod n_x. It applies when
+ * n_x is a multiple of 8 (16-byte rows) and at most 256 cells. THREADS: every thread loads and stores the
+ * populations of its one or two cells in global memory. Both give bitwise the same populations.
  * With the tensor cores selected (lbm_model_set_tensor_cores), ROWS runs the two contractions
  * on tcgen05 with the A operands written into tensor memory, also with per-order rates (bitwise
- * the per-thread tcgen05 kernel). AUTO (default) takes ROWS where it applies. Errors: LBM_ERR_ARG
+ * the per-thread tcgen05 kernel). AUTO (default) takes ROWS on tcgen05 where it applies, and THREADS on the
+ * CUDA cores, where it is the faster one. Errors: LBM_ERR_ARG
  * for an unknown mode, or ROWS on a model it does not apply to; a step with ROWS forced and
  * per-order rates on the CUDA cores (no row-staged kernel) returns LBM_ERR_NOT_IMPLEMENTED.
  * mode = 3 is a test hook of the bounded waits: ROWS with no row copy issued, so every wait on a

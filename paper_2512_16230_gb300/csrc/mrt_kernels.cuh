@@ -801,9 +801,11 @@ __device__ __forceinline__ uint32_t enc_word(float a, float b) {
 //
 // What bounds it: HBM on large FP32 grids, instruction issue elsewhere; packing halves the FP32 arithmetic. us a
 // step on GB300, one cell / two cells per thread: rD2Q13 1024x768 FP32 11.5 / 8.8, rD3Q33 64^3 FP32
-// 10.2 / 8.4, rD3Q53 256x256x192 FP32 776 / 759, rD3Q53 150x131x147 BF16 153 / 116, rD3Q45 101x103x97
-// FP32 62.8 / 59.2. 4 blocks per SM leave 128 registers; on rD3Q53 the single accesses spill at that, with 3
-// blocks 81^3 FP32 takes 39.0 us (one cell per thread 40.0) and 149x131x147 BF16 139 us (156).
+// 10.2 / 8.4, rD3Q53 256x256x192 FP32 776 / 759, rD3Q53 150x131x147 BF16 153 / 111, rD3Q45 101x103x97
+// FP32 62.8 / 57.5. 4 blocks per SM leave 128 registers; on rD3Q53 the single accesses spill at that, with 3
+// blocks 81^3 FP32 takes 39.0 us (one cell per thread 40.0) and 149x131x147 BF16 139 us (156). s_h != 1
+// (KEEP) holds the old populations as well: 3 blocks, spilling a little, against 2 without: rD3Q53 256x128x96
+// FP32 218 -> 198, FP16 168 -> 136, rD3Q45 FP32 187 -> 165, FP16 148 -> 114.
 //
 // HI: with the operator of the higher rows (hc). FP32 storage waits for memory and takes one block per SM
 // more than fits without spills (which stay in L1); 16-bit storage is bound by issue, and its blocks stay
@@ -819,7 +821,7 @@ constexpr int pair_high_blocks() {
 template <class L, class ST, bool KEEP, bool EVEN, bool HI>
 constexpr int pair_blocks() {
   if (HI) return pair_high_blocks<L, ST>();
-  if (KEEP && L::Q > 33) return 2;
+  if (KEEP && L::Q > 33) return 3;
   return L::Q > 45 && (!EVEN || is_deviation_storage<ST>()) ? 3 : 4;
 }
 template <class L, class ST, int EQ, bool KEEP, bool EVEN, bool HI = false, bool LATE = false>
@@ -1359,8 +1361,11 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       tgrid = tc_grid(m, tp32.ntiles, k, Tc32Shape<L>::CTAS, tsmem);
     }
   }
-  // 16-bit storage: the row-staged gather where it applies (or is forced), with the contractions
-  // on the CUDA cores or, when the tensor cores are selected, on tcgen05
+  // 16-bit storage: the row-staged gather on tcgen05, for a step without a collision, or when forced. On the
+  // CUDA cores the per-thread kernels are the faster ones since they take two cells per thread: us a step of
+  // FP16, row-staged / per thread: rD3Q53 256x256x192 460 / 441, 96^3 43 / 35, 32^3 5.6 / 3.3, with s_h != 1
+  // 256x128x96 150 / 136; rD3Q33 64^3 10.6 / 7.4; rD2Q17 256x4096 14.7 / 11.5. (A step without a collision on
+  // 256x256x192: 439 row-staged, 550 per thread.)
   [[maybe_unused]] RowPlan rplan;
   [[maybe_unused]] StepParams<F2, float> p2;  // the row-staged CUDA-core kernel works on two cells at a time
   bool rows = false;
@@ -1368,7 +1373,7 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
     if (m->gather == LBM_GATHER_ROWS && high && !tensor)
       return set_error(LBM_ERR_NOT_IMPLEMENTED,
                        "the row-staged gather runs per-order rates on the tensor cores only");
-    if (m->gather != LBM_GATHER_THREADS && (!high || tensor)) {
+    if (m->gather == LBM_GATHER_ROWS || (m->gather == LBM_GATHER_AUTO && (tensor || !collide_on))) {
       rows = RowLaunch<L::KIND>::plan(m, &rplan, tensor, high);
       if (!rows && m->gather == LBM_GATHER_ROWS) return set_error(LBM_ERR_ARG, "the row-staged gather does not apply");
       if (rows && nsteps > 0) {

@@ -280,8 +280,9 @@ class Model:
         _check(load().lbm_model_set_tensor_cores(self.handle, int(enable)), "lbm_model_set_tensor_cores")
 
     def set_gather(self, mode="auto"):
-        """16-bit storage on the CUDA cores: "rows" (source x-rows staged in shared memory by bulk
-        copies), "threads" (per-thread loads from global memory) or "auto" (rows where they apply)."""
+        """16-bit storage: "rows" (source x-rows staged in shared memory by asynchronous copies),
+        "threads" (per-thread loads from global memory) or "auto" (the faster one: rows on the tensor
+        cores, threads on the CUDA cores)."""
         _check(load().lbm_model_set_gather(self.handle, GATHERS[mode]), "lbm_model_set_gather")
 
     def set_ncde_variant(self, variant="moment", a1=0.0):

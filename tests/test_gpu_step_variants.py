@@ -239,3 +239,20 @@ def test_order_rates_default_on_wide_rows(fewer):
         out.append(m.read_fields()[1])
         m.close()
     assert np.array_equal(out[0], out[1]) and not np.array_equal(out[0], out[2])
+
+
+# 16-bit storage by default: two cells per thread from 80,000 cells, one below; the row-staged kernel's populations
+@pytest.mark.parametrize("s_high", [1.0, 1.3])
+@pytest.mark.parametrize("name,n", [("rD3Q53", (48, 42, 40)), ("rD3Q53", (48, 41, 40)), ("rD3Q45", (48, 42, 40))])
+def test_default_of_16_bit_storage(name, n, s_high):
+    spec = W.LATTICES[name]
+    f0 = _populations(spec, n, 15, "nse")
+    out = []
+    for mode in ("auto", "rows"):
+        gm = gpu_model(spec, "nse", n, _rates(spec), store="bf16_dev", **_kwargs("nse", 3, s_high))
+        gm.set_gather(mode)
+        gm.set_populations(f0)
+        gm.step(3)
+        out.append(gm.get_populations())
+        gm.close()
+    assert np.array_equal(out[0], out[1])
