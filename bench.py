@@ -111,12 +111,10 @@ def _profile_traffic(cells):
 
 def _kernel_name(args, grid):
     """The collide-stream kernel the library runs for this storage and grid."""
-    rows = args.store != "f32" and grid[0] % 8 == 0 and grid[0] <= 256
     threads = "k_step_pair" if math.prod(grid) >= 80000 else "k_step"  # two cells per thread or one
-    if args.store == "f32":
-        return f"{threads}<rD3Q53, f32, NSE>"
-    base = ("k_step_rows_tc" if args.tensor_cores else "k_step_rows") if rows else \
-        ("k_step_tc" if args.tensor_cores else threads)
+    if args.store == "f32" or not args.tensor_cores:
+        return f"{threads}<rD3Q53, {args.store}, NSE>"
+    base = "k_step_rows_tc" if grid[0] % 8 == 0 and grid[0] <= 256 else "k_step_tc"
     return f"{base}<rD3Q53, {args.store}, NSE>"
 
 
@@ -545,10 +543,10 @@ def bench_ours(args):
     # and BF16 on the CUDA cores, FP16 with the contractions on tcgen05
     for key, store, tc, gather, kern in (
             ("f16_deviations", "f16_dev", 0, "auto",
+             "k_step_pair<rD3Q53, f16_dev, NSE> (two cells per thread)"),
+            ("bf16_deviations", "bf16_dev", 0, "auto", "k_step_pair<rD3Q53, bf16_dev, NSE>"),
+            ("f16_deviations_row_gather", "f16_dev", 0, "rows",
              "k_step_rows<rD3Q53, f16_dev, NSE> (source x-rows staged in shared memory by cp.async)"),
-            ("bf16_deviations", "bf16_dev", 0, "auto", "k_step_rows<rD3Q53, bf16_dev, NSE>"),
-            ("f16_deviations_thread_gather", "f16_dev", 0, "threads",
-             "k_step_pair<rD3Q53, f16_dev, NSE> (per-thread gather from global memory)"),
             ("f16_deviations_tensor_cores", "f16_dev", 1, "auto",
              "k_step_rows_tc<rD3Q53, f16_dev, NSE> (row-staged, contractions on tcgen05)"),
             ("f16_deviations_tensor_cores_thread_gather", "f16_dev", 1, "threads",
