@@ -2,8 +2,10 @@
 // f_i - w_i rho_ref, collision arithmetic in FP32).
 //
 // The per-thread pull gather and store of k_step move 64 bytes per warp access when a population
-// takes 2 bytes, too little per memory request to keep HBM busy. Here a CTA works on whole x-rows
-// of the grid. For the row (y, z) the pull sources of population i (Eq. (2-2b)) are the cells
+// takes 2 bytes, too little per memory request to keep HBM busy (k_step_pair, with two cells per thread,
+// moves 128 and has become the faster kernel for a step with a collision on the CUDA cores; the kernels
+// here serve the step without one, tcgen05 and a forced row gather). Here a CTA works on whole x-rows of
+// the grid. For the row (y, z) the pull sources of population i (Eq. (2-2b)) are the cells
 // (x - e_ix, y - e_iy, z - e_iz): the x-row (y - e_iy, z - e_iz) of array i, read with a periodic
 // shift along x. The warps copy these source rows into a shared-memory buffer with 16-byte cp.async
 // copies (up to 512 bytes per warp instruction, completing on the buffer's mbarrier); the periodic
