@@ -322,8 +322,11 @@ lbm_status lbm_model_get_populations(lbm_model* m, double* f, int on_device);
 
 /* Advance nsteps time steps: per step one fused kernel computes the pull-streaming gather
  * (Eq. (2-2b)), the fields of Eq. (2-4-2) / (2-4-1), the collision of Eq. (2-3) in the Hermite
- * basis with the equilibrium of Eq. (feq-1) and the source moments, and the store.
- * Asynchronous on the model's stream. */
+ * basis with the equilibrium of Eq. (feq-1) and the source moments, and the store; on small 2D grids
+ * in FP32 and 16-bit storage one launch does the same for all steps of the call.
+ * Asynchronous on the model's stream. An even number of steps ends in the memory that it started from, so
+ * calls of an even number of steps together, captured in a CUDA graph on the model's stream, advance the
+ * state at every replay. */
 lbm_status lbm_model_step(lbm_model* m, int64_t nsteps);
 
 /* Propagation only (Eq. (2-2b)), no collision: a bit-exact data-movement test mode. */

@@ -1390,20 +1390,18 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
       constexpr int64_t kMost = 1 << 16;  // steps of one launch
       while (nsteps > 0) {
         const int n = int(std::min<int64_t>(kMost, nsteps));
-        const void* fin = m->f[m->cur];
-        void* fout = m->f[m->cur ^ 1];
         cudaError_t err;
         if (m->eq == LBM_NSE)
-          err = m->s_high == 1.0 ? launch_resident<L, ST, LBM_NSE, false>(m, p, n, ctas, fin, fout, phi)
-                                 : launch_resident<L, ST, LBM_NSE, true>(m, p, n, ctas, fin, fout, phi);
+          err = m->s_high == 1.0 ? launch_resident<L, ST, LBM_NSE, false>(m, p, n, ctas, phi)
+                                 : launch_resident<L, ST, LBM_NSE, true>(m, p, n, ctas, phi);
         else
-          err = m->s_high == 1.0 ? launch_resident<L, ST, LBM_NCDE, false>(m, p, n, ctas, fin, fout, phi)
-                                 : launch_resident<L, ST, LBM_NCDE, true>(m, p, n, ctas, fin, fout, phi);
+          err = m->s_high == 1.0 ? launch_resident<L, ST, LBM_NCDE, false>(m, p, n, ctas, phi)
+                                 : launch_resident<L, ST, LBM_NCDE, true>(m, p, n, ctas, phi);
         if (err != cudaSuccess) {  // no room for the cluster (a partitioned GPU): step by step
           cudaGetLastError();
           break;
         }
-        m->cur ^= 1;
+        m->cur ^= n & 1;  // as n launches would have left it
         m->launches += 1;
         m->steps += n;
         nsteps -= n;

@@ -62,7 +62,7 @@ inline size_t resident_smem(const lbm_model* m, int64_t rows) {
 
 template <class L, class ST, int EQ, bool KEEP>
 __global__ void __launch_bounds__(kResidentThreads, 1)
-    k_steps_resident(const StepParams<float> p, const ResidentParams rp, const ST* fin, ST* fout, float* phi) {
+    k_steps_resident(const StepParams<float> p, const ResidentParams rp, ST* cur, ST* other, float* phi) {
   constexpr int Q = L::Q, RM = L::RMAX;
   constexpr uint32_t CELL = sizeof(ST);
   constexpr bool DEV = is_deviation_storage<ST>();
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   const size_t g0 = size_t(y0) * nx;
   static_for<Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
-    for (int c = threadIdx.x; c < own; c += blockDim.x) f0[I * cells + c] = fin[size_t(I) * N + g0 + c];
+    for (int c = threadIdx.x; c < own; c += blockDim.x) f0[I * cells + c] = cur[size_t(I) * N + g0 + c];
   });
   if constexpr (EQ == LBM_NCDE) {
     for (int c = threadIdx.x; c < own; c += blockDim.x) s_phi[c] = phi[g0 + c];
@@ -126,10 +126,15 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
     }
     cluster::sync();
   }
-  const ST* last = f0 + ((rp.nsteps & 1) ? size_t(cells) * Q : 0);
+  // both buffers go back to where a launch per step would have left them: an even number of steps ends in `cur`
+  const ST* f1 = f0 + size_t(cells) * Q;
   static_for<Q>([&](auto i) {
     constexpr int I = decltype(i)::value;
-    for (int c = threadIdx.x; c < own; c += blockDim.x) fout[size_t(I) * N + g0 + c] = last[I * cells + c];
+    for (int c = threadIdx.x; c < own; c += blockDim.x) {
+      const size_t g = size_t(I) * N + g0 + c;
+      cur[g] = f0[I * cells + c];
+      other[g] = f1[I * cells + c];
+    }
   });
   if constexpr (EQ == LBM_NCDE) {
     for (int c = threadIdx.x; c < own; c += blockDim.x) phi[g0 + c] = s_phi[c];
@@ -153,8 +158,7 @@ bool resident_plan(const lbm_model* m, int64_t nsteps, int* ctas) {
 }
 
 template <class L, class ST, int EQ, bool KEEP>
-cudaError_t launch_resident(const lbm_model* m, const StepParams<float>& p, int nsteps, int ctas, const void* fin,
-                            void* fout, float* phi) {
+cudaError_t launch_resident(const lbm_model* m, const StepParams<float>& p, int nsteps, int ctas, float* phi) {
   ResidentParams rp;
   rp.nsteps = nsteps;
   rp.rows = int((m->n[1] + ctas - 1) / ctas);
@@ -180,7 +184,7 @@ cudaError_t launch_resident(const lbm_model* m, const StepParams<float>& p, int 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel, p, rp, static_cast<const ST*>(fin), static_cast<ST*>(fout), phi);
+  return cudaLaunchKernelEx(&cfg, kernel, p, rp, static_cast<ST*>(m->f[m->cur]), static_cast<ST*>(m->f[m->cur ^ 1]), phi);
 }
 
 }  // namespace lbm
