@@ -419,7 +419,9 @@ void Launch<KIND>::high_operator_blocks(const lbm_model* m, double* c) {
       }
       if (s < 0.0) row_class[r] |= 1 << a;
     }
-  const double oms = 1.0 - m->s_high;
+  // s_high as the kernel has it (make_step_params): A and 1 - s_high come from one value, or the rows that carry
+  // mass and momentum would grow by its rounding at every step (s_high = 1.05 in FP32: 4.8e-8)
+  const double sh = fp64 ? m->s_high : double(float(m->s_high)), oms = 1.0 - sh;
   for (int b = 0; b < B::blocks(); ++b) {
     const int o = B::block_off(b), n = B::block_size(b);
     double* M = c + B::coef_off(b);
@@ -427,9 +429,10 @@ void Launch<KIND>::high_operator_blocks(const lbm_model* m, double* c) {
       for (int l = 0; l < n; ++l) {
         double v = k == l ? oms / ((fp64 ? lat->w[rep[o + k]] : double(lat->wf[rep[o + k]])) * members[o + k]) : 0.0;
         for (int r = 0; r < lat->nhigh; ++r) {
-          if (row_class[r] != cls[o + k]) continue;
+          const double s = high_rate(m, lat->h_order[r]);
+          if (row_class[r] != cls[o + k] || s == m->s_high) continue;
           const double* h = lat->Hh + size_t(r) * Q;
-          v -= (high_rate(m, lat->h_order[r]) - m->s_high) / lat->Nh[r] * h[rep[o + k]] * h[rep[o + l]];
+          v -= (s - sh) / lat->Nh[r] * h[rep[o + k]] * h[rep[o + l]];
         }
         const bool odd = (((cls[o + k] & 1) + ((cls[o + k] >> 1) & 1) + ((cls[o + k] >> 2) & 1)) & 1) != 0;
         M[k * n + l] = odd ? v / mult[o + k] : v;

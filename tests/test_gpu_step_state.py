@@ -5,7 +5,7 @@ import torch
 
 from paper_2512_16230_gb300 import workloads as W
 
-from _harness import gpu_model
+from _harness import gpu_model, oracle_lattice
 
 pytestmark = pytest.mark.gpu
 
@@ -53,3 +53,49 @@ def test_replayed_steps_advance_the_state(name, n, one_launch, eq, store, calls)
         out.append(m.get_populations())
         m.close()
     assert np.array_equal(out[0], out[1])
+
+
+def _coefficient_drift(spec, s_high, s_orders):
+    """Largest relative change of the mass in a step by rounding the operator of the higher rows to FP32: each of
+    its coefficients by 2^-24 of itself, the diagonal 1 - s_high and, for an order k with a rate of its own,
+    sum_ij w_i w_j |P_ij| |s_k - s_high|, P the W-orthogonal projector on the rows of that order."""
+    lat = oracle_lattice(spec)
+    total = abs(1.0 - s_high)
+    for k, s in s_orders.items():
+        B = lat.Hfull[[r for r, o in enumerate(lat.full_orders) if o == k]]
+        P = B.T @ np.linalg.inv((B * lat.w) @ B.T) @ B
+        total += abs(s - s_high) * float(lat.w @ np.abs(P) @ lat.w)
+    return 2.0 ** -24 * total
+
+
+# One rate per order >= 4 in FP32, with rates that FP32 does not hold: 1.05 is 4.8e-8 off, which the step must not
+# multiply the mass by. One cell and two cells per thread, and batched.
+@pytest.mark.parametrize("name,n,batched", [("rD3Q53", (32, 32, 32), False), ("rD3Q53", (48, 48, 48), False),
+                                            ("rD3Q53", (32, 32, 32), True)])
+def test_order_rates_conserve_mass(name, n, batched):
+    from paper_2512_16230_gb300 import lbm
+    spec, s_high, s_orders, steps = W.LATTICES[name], 1.05, {4: 1.1}, 200
+    d, cells = len(n), int(np.prod(n))
+    # a vortex of a tenth of the lattice speed, so that no two cells round alike
+    x = [np.arange(k) * (2 * np.pi / k) for k in n]
+    X = np.meshgrid(*reversed(x), indexing="ij")[::-1]
+    u = np.zeros((d,) + tuple(reversed(n)))
+    u[0], u[1] = 0.1 * np.sin(X[0]) * np.cos(X[1]), -0.1 * np.cos(X[0]) * np.sin(X[1])
+    rho = 1.0 + np.random.default_rng(17).uniform(-0.01, 0.01, size=tuple(reversed(n)))
+    m = gpu_model(spec, "nse", n, W.rates_nse(d, 0.01, spec.cs2[0], spec=spec), s_high=s_high, store="f32",
+                  s_orders=s_orders)
+    m.init_fields(rho, u)
+    before = m.conserved_sums()[0]
+    if batched:
+        b = lbm.Batch()
+        b.set_solo_threshold(0)
+        b.add(m)
+        b.step(steps)
+        b.remove(m)
+        b.close()
+    else:
+        m.step(steps)
+    change = m.conserved_sums()[0] / before - 1.0
+    m.close()
+    # and some 40 roundings of 2^-24 per cell and step, independent of each other
+    assert abs(change) <= steps * _coefficient_drift(spec, s_high, s_orders) + 40 * 2.0 ** -24 * np.sqrt(steps / cells)
