@@ -99,3 +99,22 @@ def test_order_rates_conserve_mass(name, n, batched):
     m.close()
     # and some 40 roundings of 2^-24 per cell and step, independent of each other
     assert abs(change) <= steps * _coefficient_drift(spec, s_high, s_orders) + 40 * 2.0 ** -24 * np.sqrt(steps / cells)
+
+
+# A uniform stream in FP32: on its own a rounding of the momentum to FP32 in a step, of a product with 1 / 0.6 that
+# lies a third of a unit in the last place apart for neighbouring momenta, moves it by a third of 2^-24 at most.
+@pytest.mark.parametrize("speed", [0.0387, 0.021])
+@pytest.mark.parametrize("name,n", [("rD3Q45", (24, 20, 16)), ("rD3Q53-cubic", (24, 20, 16)), ("rD3Q45", (48, 44, 40))])
+def test_uniform_stream_keeps_its_momentum(name, n, speed):
+    spec, steps = W.LATTICES[name], 200
+    rng = np.random.default_rng(18)
+    rho = 1.0 + 1e-3 * rng.uniform(-1, 1, size=tuple(reversed(n)))
+    u = 1e-3 * rng.uniform(-1, 1, size=(3,) + tuple(reversed(n)))
+    u[0] += speed
+    m = gpu_model(spec, "nse", n, W.rates_nse(3, 0.05, spec.cs2[0], spec=spec), store="f32")
+    m.init_fields(rho, u)
+    before = m.conserved_sums()[1]
+    m.step(steps)
+    change = m.conserved_sums()[1] / before - 1.0
+    m.close()
+    assert abs(change) <= steps * 2.0 ** -24 / 3
