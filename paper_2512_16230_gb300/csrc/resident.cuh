@@ -145,14 +145,19 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
 // density-gradient term of M2G (a field of the neighbours' last step in global memory) do not.
 template <class L, class ST>
 bool resident_plan(const lbm_model* m, int64_t nsteps, int* ctas) {
-  if (L::D != 2 || nsteps < 2 || m->m2g_aniso || m->gather != LBM_GATHER_AUTO) return false;
+  if (L::D != 2 || m->m2g_aniso || m->gather != LBM_GATHER_AUTO) return false;
   int n = kResidentCtas;
   while (n > 1 && n > m->n[1]) n /= 2;
-  const int64_t rows = (m->n[1] + n - 1) / n;
-  // populations per CTA up to which it is the faster form (us a step, resident / chained: rD2Q17 32x32
-  // 0.81 / 1.90, 64x48 1.07 / 1.87, 100x76 1.57 / 1.88, 128x128 2.39 / 1.91; rD2Q25 64x48 1.37 / 1.91,
-  // 100x76 2.07 / 2.01)
-  if (rows * m->n[0] * L::Q > 8192) return false;
+  const int64_t rows = (m->n[1] + n - 1) / n, cells = rows * m->n[0], pops = cells * L::Q;
+  // Per CTA, a cell a thread at most and the populations up to which a step is the faster one. us a step, resident /
+  // chained: rD2Q17 32x32 0.74 / 1.60, 64x48 0.98 / 1.71, 80x60 1.27 / 1.76; rD2Q25 64x48 1.30 / 1.91, 80x60 (8000
+  // populations) 1.66 / 1.91, 100x76 2.07 / 2.01; with a second cell for some threads rD2Q13 630x16 2.33 / 1.76,
+  // rD2Q9 630x16 1.83 / 1.71.
+  if (cells > kResidentThreads || pops > 8192) return false;
+  // Loading and storing the grid costs a call 4 to 9 us, so that a short one is faster step by step. Steps from which
+  // one launch is faster, measured (on NSE and NCDE, FP32 and FP16): 576 populations 4.2 .. 5.5, 1600 5.0 .. 9.3,
+  // 3264 8.0 .. 8.7, 5440 11 .. 14, 6500 19 .. 24, 8000 9 .. 32.
+  if (nsteps < 4 + pops / 512) return false;
   *ctas = n;
   return resident_smem<L, ST>(m, rows) <= size_t(kResidentSmem);
 }

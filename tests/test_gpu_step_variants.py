@@ -256,3 +256,47 @@ def test_default_of_16_bit_storage(name, n, s_high):
         out.append(gm.get_populations())
         gm.close()
     assert np.array_equal(out[0], out[1])
+
+
+# The same for calls long enough to run in one launch, with the launches counted: the widest rows taken (512 cells, 8192
+# populations a CTA) and the first ones not taken, and the shortest call of 64 x 48 and of 20 x 256 that is.
+@pytest.mark.parametrize("store", ["f32", "f16_dev"])
+@pytest.mark.parametrize("s_high", [1.0, 1.3])
+@pytest.mark.parametrize("eq", ["nse", "ncde"])
+@pytest.mark.parametrize("name,n,calls,launches", [
+    ("rD2Q13", (37, 29), (20, 21), 2), ("rD2Q13", (5, 3), (20, 21), 2), ("rD2Q13", (512, 16), (20, 21), 2),
+    ("rD2Q13", (513, 16), (20, 21), 41), ("rD2Q25", (327, 16), (20, 21), 2), ("rD2Q25", (328, 16), (20, 21), 41),
+    ("rD2Q25", (7, 6), (20, 21), 2), ("rD2Q25", (64, 48), (12, 13), 13), ("rD2Q25", (20, 256), (18, 19), 19)])
+def test_long_calls_on_a_small_grid_in_one_launch(name, n, calls, launches, eq, s_high, store):
+    spec = W.LATTICES[name]
+    f0 = _populations(spec, n, 10, eq)
+    out = []
+    for split in ([1] * sum(calls), calls):
+        m = gpu_model(spec, eq, n, np.random.default_rng(3).uniform(0.9, 1.5, spec.R), store=store, **_kwargs(eq, 2, s_high))
+        m.set_populations(f0)
+        before = m.counters()[1]
+        for k in split:
+            m.step(k)
+        assert m.counters()[1] - before == (sum(calls) if split is not calls else launches)
+        out.append(m.get_populations())
+        m.close()
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("store", ["f32", "bf16_dev"])
+def test_long_call_in_one_launch_with_per_cell_rates_and_cross_diffusion(store):
+    spec, n, steps = W.LATTICES["rD2Q17"], (41, 23), 21
+    f0 = _populations(spec, n, 11, "ncde")
+    psi = np.random.default_rng(7).uniform(-1, 1, size=(n[1], n[0]))
+    out = []
+    for calls in ([1] * steps, [steps]):
+        m = gpu_model(spec, "ncde", n, _rates(spec), store=store, ncde_mode="rate", a1=-0.2, a2=0.02, psi=psi,
+                      **_kwargs("ncde", 2, 1.0))
+        m.set_populations(f0)
+        before = m.counters()[1]
+        for k in calls:
+            m.step(k)
+        assert m.counters()[1] - before == len(calls)
+        out.append(m.get_populations())
+        m.close()
+    assert np.array_equal(out[0], out[1])
