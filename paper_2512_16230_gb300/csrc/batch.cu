@@ -488,13 +488,16 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
     if (err != cudaSuccess) return cuda_error(err, "batch side stream");
   }
   lbm_status st = LBM_OK;
+  int64_t solo_launches = 0;  // (a small 2D solo may run many steps in one launch)
   for (lbm_model* m : b->solos) {
     const cudaStream_t own = m->stream;  // the batch stream while the model is a member
+    const int64_t before = m->launches;
     m->stream = b->side;
     st = dispatch_batch_kind(m->lat->kind, [&](auto kc) {
       return Launch<decltype(kc)::value>::step(m, nsteps, true);
     });
     m->stream = own;
+    solo_launches += m->launches - before;
     if (st != LBM_OK) break;
   }
   for (int64_t c = 0; c < chunks && st == LBM_OK; ++c) {
@@ -531,7 +534,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps) {
       m->launches += nsteps;
     }
   b->steps += nsteps;
-  b->launches += nsteps * int64_t(b->groups.size() + b->solos.size());
+  b->launches += nsteps * int64_t(b->groups.size()) + solo_launches;
   b->stable = true;
   return LBM_OK;
 }

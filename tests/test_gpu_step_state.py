@@ -118,3 +118,24 @@ def test_uniform_stream_keeps_its_momentum(name, n, speed):
     change = m.conserved_sums()[1] / before - 1.0
     m.close()
     assert abs(change) <= steps * 2.0 ** -24 / 3
+
+
+# The launches of a batch of a 64 x 48 and a 128 x 128 solve, 20 steps: one a step for both in one group, one a step for
+# each with the larger one alone, and with both alone a single one for the smaller, whose steps run in one launch.
+@pytest.mark.parametrize("threshold,launches", [(0, 20), (4000, 40), (3000, 21)])
+def test_batch_counts_the_launches_it_issued(threshold, launches):
+    from paper_2512_16230_gb300 import lbm
+    spec = W.LATTICES["rD2Q17"]
+    lat = lbm.Lattice(spec.kind, spec.c, spec.cs2, spec.free_w)
+    models = [gpu_model(spec, "nse", n, W.rates_nse(2, 0.05, spec.cs2[0], spec=spec), lat=lat) for n in ((64, 48), (128, 128))]
+    b = lbm.Batch()
+    b.set_solo_threshold(threshold)
+    for m in models:
+        m.set_populations(_populations(m, m.n, 19, 1.0))
+        b.add(m)
+    b.step(20)
+    counted = b.counters()["launches"]
+    b.close()
+    for m in models:
+        m.close()
+    assert counted == launches
