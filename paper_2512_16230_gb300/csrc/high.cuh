@@ -359,6 +359,19 @@ __device__ __forceinline__ void collide_high(V (&f)[L::Q], const typename Coef<V
   back_project_high<L>(f, lt, h, a);
 }
 
+// Velocity i reflected in axis a.
+template <class L>
+struct Reflected {
+  int v[3][L::Q];
+  constexpr Reflected() : v{} {
+    for (int a = 0; a < L::D; ++a)
+      for (int i = 0; i < L::Q; ++i) {
+        const Vel e = L::e(i);
+        while (!same_vel(L::e(v[a][i]), Vel{a == 0 ? -e.x : e.x, a == 1 ? -e.y : e.y, a == 2 ? -e.z : e.z})) ++v[a][i];
+      }
+  }
+};
+
 // Host: the blocks of M for the rates of the model. rep_k: a velocity with phi_k = +1, so that H_r = sum_k
 // H_r(rep_k) phi_k over the functions of the row's class (the row's behaviour under the reflections).
 template <int KIND>
@@ -404,21 +417,20 @@ void Launch<KIND>::high_operator_blocks(const lbm_model* m, double* c) {
       }
       set(B::corner_odd3(mm), 7, d, mm, 8);
     }
-  int row_class[Q] = {};
-  for (int r = 0; r < lat->nhigh; ++r)
+  // the rows with a rate of their own, by class
+  static constexpr Reflected<L> mirror{};
+  int rows[8][Q], count[8] = {};
+  for (int r = 0; r < lat->nhigh; ++r) {
+    if (high_rate(m, lat->h_order[r]) == m->s_high) continue;
+    const double* h = lat->Hh + size_t(r) * Q;
+    int cl = 0;
     for (int a = 0; a < D; ++a) {
       double s = 0.0;  // <H_r, H_r reflected in axis a>
-      for (int i = 0; i < Q; ++i) {
-        Vel e = L::e(i);
-        if (a == 0) e.x = -e.x;
-        if (a == 1) e.y = -e.y;
-        if (a == 2) e.z = -e.z;
-        int j = 0;
-        while (!same_vel(L::e(j), e)) ++j;
-        s += lat->Hh[size_t(r) * Q + i] * lat->Hh[size_t(r) * Q + j];
-      }
-      if (s < 0.0) row_class[r] |= 1 << a;
+      for (int i = 0; i < Q; ++i) s += h[i] * h[mirror.v[a][i]];
+      if (s < 0.0) cl |= 1 << a;
     }
+    rows[cl][count[cl]++] = r;
+  }
   // s_high as the kernel has it (make_step_params): A and 1 - s_high come from one value, or the rows that carry
   // mass and momentum would grow by its rounding at every step (s_high = 1.05 in FP32: 4.8e-8)
   const double sh = fp64 ? m->s_high : double(float(m->s_high)), oms = 1.0 - sh;
@@ -428,11 +440,10 @@ void Launch<KIND>::high_operator_blocks(const lbm_model* m, double* c) {
     for (int k = 0; k < n; ++k)
       for (int l = 0; l < n; ++l) {
         double v = k == l ? oms / ((fp64 ? lat->w[rep[o + k]] : double(lat->wf[rep[o + k]])) * members[o + k]) : 0.0;
-        for (int r = 0; r < lat->nhigh; ++r) {
-          const double s = high_rate(m, lat->h_order[r]);
-          if (row_class[r] != cls[o + k] || s == m->s_high) continue;
+        for (int q = 0; q < count[cls[o + k]]; ++q) {
+          const int r = rows[cls[o + k]][q];
           const double* h = lat->Hh + size_t(r) * Q;
-          v -= (s - sh) / lat->Nh[r] * h[rep[o + k]] * h[rep[o + l]];
+          v -= (high_rate(m, lat->h_order[r]) - sh) / lat->Nh[r] * h[rep[o + k]] * h[rep[o + l]];
         }
         const bool odd = (((cls[o + k] & 1) + ((cls[o + k] >> 1) & 1) + ((cls[o + k] >> 2) & 1)) & 1) != 0;
         M[k * n + l] = odd ? v / mult[o + k] : v;
