@@ -1365,7 +1365,17 @@ lbm_status launch_step_typed(lbm_model* m, int64_t nsteps, bool collide_on) {
   if constexpr (std::is_same<ST, float>::value) {
     if (tensor32) {
       make_tc32_params(m, &tp32);
+      // With many tiles a CTA, as much shared memory as lets no further CTA beside CTAS of them: the next launch, released
+      // early, would else place its CTAs on the SMs that have room and leave others short of work. us a step with
+      // room / without: rD2Q13 1024x768 27.8 / 20.5, rD3Q33 96^3 70.5 / 59.9 (15 tiles a CTA); 512x384 7.2 / 7.4, rD2Q25
+      // 10.8 / 11.7 (3.4 tiles: the next launch's tables are made meanwhile). rD3Q45 and larger fill the SM anyway.
       tsmem = sizeof(Tc32Smem<L>);
+      int sm_smem = 0;
+      if (tp32.ntiles >= 4 * Tc32Shape<L>::CTAS * sm_count(m->device)) {
+        if (cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, m->device) != cudaSuccess)
+          cudaGetLastError();
+        tsmem = std::max(tsmem, size_t(sm_smem) / (Tc32Shape<L>::CTAS + 1));
+      }
       const void* k = m->eq == LBM_NSE ? reinterpret_cast<const void*>(k_step_tc32_high<L, LBM_NSE>)
                                        : reinterpret_cast<const void*>(k_step_tc32_high<L, LBM_NCDE>);
       tgrid = tc_grid(m, tp32.ntiles, k, Tc32Shape<L>::CTAS, tsmem);
