@@ -417,6 +417,11 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
     });
   }
   V gN[R], me[R], neq[R];
+  // FP32: A mu, the momentum's own part of the first-order rows, is added last. The force and what the third-order
+  // rows add are a few units in its last place. Added to it one after the other, each would be rounded the same
+  // way at every step, a drift of the momentum (u = 0.04: rD3Q45 and the cubic rD3Q53 -4.2e-8 a step, so -0.4e-8 ..
+  // 0.2e-8).
+  constexpr bool LAST = EQ == LBM_NSE && !std::is_same<V, double>::value;
   if constexpr (EQ == LBM_NSE) {
     // Eq. (2-4-2) with S = 0, F_F = F: rho = sum f, rho u = sum c f + F / 2
     const V rho = mu[0];
@@ -433,11 +438,12 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
     gN[0] = rt.A[0] * rho;
     static_for<D>([&](auto a) {
       constexpr int A = decltype(a)::value;
-      // momentum, without its product with A, which comes last (below); A to twice the precision (a rounded
-      // factor would be a bias of every step)
-      if constexpr (std::is_same<V, double>::value) gN[1 + A] = V(0.f);
-      else gN[1 + A] = rt.Alo[A] * mu[1 + A];
-      if (forced) gN[1 + A] = fmaf_t(lt.iN[1 + A], F[A], gN[1 + A]);
+      if constexpr (LAST) {
+        gN[1 + A] = V(0.f);
+      } else {
+        gN[1 + A] = rt.A[1 + A] * mu[1 + A];
+        if (forced) gN[1 + A] = fmaf_t(lt.iN[1 + A], F[A], gN[1 + A]);
+      }
       constexpr int AA = row2<D>(A, A);
       neq[AA] = fmaf_t(lt.nd0[A], rho, mu[AA]) - me[AA];
     });
@@ -476,6 +482,12 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
       }
     });
     if (forced || gr != nullptr) {
+      if (LAST && forced) {
+        static_for<D>([&](auto a) {
+          constexpr int A = decltype(a)::value;
+          gN[1 + A] = product(lt.iN[1 + A], F[A]);
+        });
+      }
       V t[3];
       static_for<D>([&](auto b) {
         constexpr int B = decltype(b)::value;
@@ -559,13 +571,10 @@ __device__ __forceinline__ void collide_moments(V (&mu)[L::R], const LatTables<V
     if constexpr (D == 3) gN[row3<3>(0, 1, 2)] = product(rt.NB[row3<3>(0, 1, 2)], mu[row3<3>(0, 1, 2)]);
   }
   rows_to_monomials<L>(lt, gN, h);
-  if constexpr (EQ == LBM_NSE) {
-    // The force and what the third-order rows add are a few units in the last place of A mu. Added to A mu one
-    // after the other, each would be rounded the same way at every step, a drift of the momentum (u = 0.04 in
-    // FP32: rD3Q45 and the cubic rD3Q53 -4.2e-8 a step, so -0.4e-8 .. 0.2e-8). They are summed first.
+  if constexpr (LAST) {  // (A to twice the precision: a rounded factor would be a bias of every step)
     static_for<D>([&](auto a) {
       constexpr int A = decltype(a)::value;
-      h[1 + A] = fmaf_t(rt.A[1 + A], mu[1 + A], h[1 + A]);
+      h[1 + A] = fmaf_t(rt.A[1 + A], mu[1 + A], fmaf_t(rt.Alo[A], mu[1 + A], h[1 + A]));
     });
   }
   if constexpr (DEV) h[0] = h[0] - rt.sh_rho_ref;
