@@ -30,7 +30,9 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompil
 
 
 # The step kernels: every fused multiply-add is written out, so that the kernels which share the
-# collision (one cell a thread, batched, row-staged) round alike.
+# collision (one cell a thread, batched, row-staged) round alike. The few products left on their own
+# do not show in the error against FP64 (the collision emulated on the host with contraction on and
+# off: 2D vortices and 3D Kolmogorov flows on seven lattices, the same in three digits).
 STEP_FLAGS = ["-fmad=false"]
 
 

@@ -293,9 +293,11 @@ template void make_high_coefs<double>(const lbm_model*, HighCoefs<double>*);
 namespace {
 
 // The weights of the FP32 kernels: rounded to FP32 within a few units in the last place such that the
-// sums that carry mass and momentum come out right with the rounded values, sum w = 1 and
-// sum w e_a^2 = FP32(Delta2_aa / c_a^2). Rounding each weight by itself leaves those sums up to 3e-8
-// off, a bias of every step (48x48x36 Taylor-Green, 188 steps: the mass drifts by 3.5e-6). The
+// sums that carry mass and momentum come out as near as these allow with the rounded values, sum w = 1 and
+// sum w e_a^2 = FP32(Delta2_aa / c_a^2). Rounding each weight by itself leaves those sums up to 6e-8
+// off, a bias of every step (48x48x36 Taylor-Green, 188 steps: the mass drifts by 3.5e-6). On the 3D lattices the
+// sums are then right to 2.4e-9 or better; on the 2D ones, which have fewer weights, to 4e-9 .. 6e-9, 9e-9 on rD2Q13
+// and no better than before on rD2Q9 (3e-8). make_step_params takes 1 / sum w e_a^2 from the rounded weights. The
 // velocities of one reflection class keep one weight. Local search over moves of one or two classes.
 void fp32_weights(const lbm_lattice* L, float* w) {
   const int d = L->d;

@@ -1,9 +1,10 @@
 // The per-cell MRT collision in the Hermite basis and the fused pull collide-stream kernel.
 //
-// One thread owns one cell. It gathers the Q populations of its cell from the neighbours
+// One thread owns one cell (k_step) or, from 80,000 cells in FP32 and 16-bit storage, two neighbouring ones
+// (k_step_pair). It gathers the Q populations of its cells from the neighbours
 // x - e_i of the previous step (pull form of the propagation, Eq. (2-2b)), collides them
 // (Eq. (2-3) with the Hermite-moment collision Eq. (H-MRT-LB-1)) and writes the post-collision
-// populations back at its own cell (aligned, coalesced stores). The stored array is therefore
+// populations back at its own cells (aligned, coalesced stores). The stored array is therefore
 // the post-collision state of the last step; the pre-collision f-bar(x, t_n) of the paper is
 // its pull-gather.
 //
@@ -30,10 +31,11 @@
 
 #include "lbm_internal.cuh"
 
-// Tuning knobs of the collide-stream kernel (defaults measured best on GB300 for rD3Q53 on
-// 256x256x192: 4 blocks of 128 threads per SM leave the kernel 128 registers without spills,
-// 0.833 ms per FP32 step and 0.686 ms per FP16-deviation step, against 0.883 / 0.732 ms with
-// 5 blocks (96 registers) and 0.989 / 0.756 ms with 6; evict-first loads or stores were slower):
+// Tuning knobs of k_step, one cell per thread, which runs FP64, grids below 80,000 cells and the steps without a
+// collision, and of the batched kernel's blocks (k_step_pair has its own block counts, pair_blocks). 4 blocks
+// of 128 threads per SM leave 128 registers. Measured best while it ran every grid, rD3Q53 256x256x192, FP32 / FP16 ms
+// a step with 4 blocks 0.833 / 0.686, with 5 (96 registers) 0.883 / 0.732, with 6 0.989 / 0.756; evict-first loads or
+// stores were slower. (k_step_pair takes 0.759 / 0.44 there.)
 //   LBM_K1_MIN_BLOCKS  minimum resident blocks per SM requested through __launch_bounds__
 //   LBM_K1_LOAD        1: evict-first (__ldcs), 2: plain load. The read-only path (ld.global.nc) is
 //                      not offered: a chained launch starts while the kernel that writes its input
@@ -670,12 +672,6 @@ struct Neigh {
     constexpr Vel v = L::e(I);
     return xo[RM + v.x] + yo[RM + v.y] + (L::D == 3 ? zo[RM + v.z] : 0);
   }
-  // cell index of x + e
-  template <int I>
-  __device__ __forceinline__ int dst() const {
-    constexpr Vel v = L::e(I);
-    return xo[RM - v.x] + yo[RM - v.y] + (L::D == 3 ? zo[RM - v.z] : 0);
-  }
 };
 
 // Body force over c_a at a cell; false (and F unset) without one.
@@ -827,10 +823,10 @@ __device__ __forceinline__ uint32_t enc_word(float a, float b) {
 // FP32 218 -> 198, FP16 168 -> 136, rD3Q45 FP32 187 -> 165, FP16 148 -> 114.
 //
 // HI: with the operator of the higher rows (hc). FP32 storage waits for memory and takes one block per SM
-// more than fits without spills (which stay in L1); 16-bit storage is bound by issue, and its blocks stay
-// resident, so that each stages the operator once. us a step, without spills / with one block more: rD3Q53
-// 160x144x120 FP32 245 / 232, FP16 202 / 225; rD3Q45 205 / 175, 159 / 169; rD2Q25 1024x768 26.5 / 25.5, 21.5 /
-// 22.7. Blocks that stay resident: FP32 265 (245 with a block per 256 cells), FP16 202 (220). Also measured: the
+// more than 16-bit storage, at about 290 bytes of spills a thread on rD3Q53 (they stay in L1); 16-bit storage is bound
+// by issue (96 bytes of spills on even rows of rD3Q53), and its blocks stay resident, so that each stages the operator once. us a
+// step, with 2, 3, 4 blocks per SM (Q > 33, >= 27, below) / with one more: rD3Q53 160x144x120 FP32 245 / 232, FP16 202 /
+// 225; rD3Q45 205 / 175, 159 / 169; rD2Q25 1024x768 26.5 / 25.5, 21.5 / 22.7. Blocks that stay resident: FP32 265 (245 with a block per 256 cells), FP16 202 (220). Also measured: the
 // sources of the next two cells copied to shared memory meanwhile (cp.async, 64 threads, 4 blocks per SM): 311.
 struct NoCoefs {};
 template <class L, class ST>
@@ -1320,7 +1316,8 @@ constexpr int kPairCells = 80000;
 // next step takes a free place while others of this one end), and above which at its start (ragged grids: once
 // the wait is over, where the second cell's indices are ready). us a step,
 // rD3Q33 64^3 8.4 at the start of every block (8.9 with the point picked at run time), rD3Q53 150x131x147 BF16
-// 110.8 (114.8), rD2Q25 512x384 before the stores 5.3 (5.4).
+// 110.8 (114.8), rD2Q25 512x384 before the stores 5.3 (5.4). (The kernels with s_high != 1 and with per-order rates
+// release at the start on every size; where else they might was not measured.)
 constexpr int kPairLateCells = 200000;
 
 // Host launchers for one lattice kind (instantiated in k_<lattice>.cu).
