@@ -19,8 +19,8 @@
 // sums), and through the rows' few entries below the diagonal (collide_moments). Everything is in
 // lattice units: the axis speeds sit in the constants (LatTables, Rates).
 //
-// What bounds it: instruction issue everywhere but on large FP32 grids (HBM), and the FP64 pipe
-// (2 FMAs per clock and SM) in FP64. The shared sums, the scaled rows and s_h = 1 without the old
+// What bounds it: HBM on large FP32 grids, the arithmetic and its latency elsewhere (k_step_pair has the counters),
+// and the FP64 pipe (2 FMAs per clock and SM) in FP64. The shared sums, the scaled rows and s_h = 1 without the old
 // populations take rD3Q53 from about 830 to 600 FP32 operations per cell; whole solves on GB300:
 // rD2Q25 64x48 FP64 x 100 steps 1424 -> 996 us, rD3Q33 64^3 FP32 x 64 816 -> 693 us, rD2Q13
 // 1024x768 FP32 x 100 1361 -> 1190 us, rD3Q53 256x256x192 x 24 FP32 21.8 -> 20.4 ms and FP16
@@ -814,8 +814,9 @@ __device__ __forceinline__ uint32_t enc_word(float a, float b) {
 // with x even; an even e_x is one load of both sources, the stores are pairs. Otherwise the cells are
 // 2 t and 2 t + 1 of the array and every access is by cell (the last cell of an odd grid is done alone).
 //
-// What bounds it: HBM on large FP32 grids, instruction issue elsewhere; packing halves the FP32 arithmetic. us a
-// step on GB300, one cell / two cells per thread: rD2Q13 1024x768 FP32 11.5 / 8.8, rD3Q33 64^3 FP32
+// What bounds it: HBM on large FP32 grids; elsewhere memory, the FMA pipe and latency at 11 to 15 warps per SM
+// together (busy on rD3Q53, DRAM / heavy FMA pipe / issue: FP16 256x256x96 74 / 69 / 50%, BF16 on odd rows 56 / 48 /
+// 50%, FP32 with per-order rates 63 / 41 / 42%). Packing halves the FP32 instructions. us a step on GB300, one cell / two cells per thread: rD2Q13 1024x768 FP32 11.5 / 8.8, rD3Q33 64^3 FP32
 // 10.2 / 8.4, rD3Q53 256x256x192 FP32 776 / 759, rD3Q53 150x131x147 BF16 153 / 111, rD3Q45 101x103x97
 // FP32 62.8 / 57.5. 4 blocks per SM leave 128 registers; on rD3Q53 the single accesses spill at that, with 3
 // blocks 81^3 FP32 takes 39.0 us (one cell per thread 40.0) and 149x131x147 BF16 139 us (156). s_h != 1
